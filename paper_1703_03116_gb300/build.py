@@ -18,8 +18,12 @@ INCLUDE = os.path.join(ROOT, "include")
 OBJDIR = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libfc.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-SOURCES = ["advance.cu", "advance_walk.cu", "advance_band.cu", "fill.cu", "aux_kernels.cu", "noalloc.cu", "adjoint.cu", "sphere.cu",
-           "forest.cpp", "capi.cpp"]
+# (source, precision): the update kernels' many instantiations are compiled
+# one precision a unit, side by side
+SOURCES = [("advance_walk.cu", "float"), ("advance_walk.cu", "double"),
+           ("advance_band.cu", "float"), ("advance_band.cu", "double")] + [
+    (s, None) for s in ("advance.cu", "fill.cu", "aux_kernels.cu", "noalloc.cu", "adjoint.cu",
+                        "sphere.cu", "forest.cpp", "capi.cpp")]
 
 
 def _nvcc() -> str:
@@ -29,8 +33,9 @@ def _nvcc() -> str:
     return "nvcc"
 
 
-def _compile(src: str) -> str:
-    obj = os.path.join(OBJDIR, os.path.splitext(src)[0] + ".o")
+def _compile(unit) -> str:
+    src, real = unit
+    obj = os.path.join(OBJDIR, os.path.splitext(src)[0] + (f"_{real}" if real else "") + ".o")
     path = os.path.join(CSRC, src)
     deps = [path] + [os.path.join(CSRC, f) for f in os.listdir(CSRC)
                      if f.endswith((".hpp", ".cuh"))]
@@ -40,6 +45,8 @@ def _compile(src: str) -> str:
     cmd = [_nvcc(), *ARCH, "-O3", "-std=c++17", "-lineinfo", "--expt-relaxed-constexpr",
            "-Xcompiler", "-fPIC",
            "-I", INCLUDE, "-I", CSRC, "-c", path, "-o", obj]
+    if real:
+        cmd[1:1] = [f"-DFC_REAL={real}"]
     if src.endswith(".cpp"):
         cmd[1:1] = ["-x", "cu"]
     subprocess.run(cmd, check=True)

@@ -52,12 +52,12 @@ constexpr int band_min_blocks() {
 // CAP: the capacity form of the cubed sphere (Sec. 5.3) -- the patch's FP64
 // metric block (kappa, phi_x, phi_y) arrives in dynamic shared memory by a
 // second bulk copy; edge speeds are the edge volume fluxes phi, the
-// correction's dt/h is dt (1/kappa_L + 1/kappa_R)/2, a fluctuation's
-// transverse increment is scaled by dt/2 over the area of the cell it
-// enters, and the update by dt over the cell's area.
-template <typename real, int MX, int R, bool SWIRL, bool CAP>
+// correction's 2 |c| is |c| (1/kappa_L + 1/kappa_R), a fluctuation sum and
+// the update are divided by the area of the cell they enter.
+template <typename real, int MX, int R, bool SWIRL, bool CAP, bool FULL>
 __global__ void __launch_bounds__(band_threads<real, MX, R>(), band_min_blocks<real, MX, R>())
-    advance_band_kernel(DevForest<real> D, int p0, int p1, AdvArgs a, int* err) {
+    advance_band_kernel(DevForest<real> D, int p0, int p1, AdvArgs a, AdvConst<real> ac,
+                        int* err) {
   constexpr int S = MX + 4;
   constexpr int MS = CAP ? metric_stride(S) : 0;
   constexpr uint32_t mbytes = sizeof(double) * MS;
@@ -66,7 +66,7 @@ __global__ void __launch_bounds__(band_threads<real, MX, R>(), band_min_blocks<r
   constexpr int NW = MX * MX / R;  // threads that walk a band
   constexpr int NV = MX + 3;  // corner nodes -1..MX+1 of a row or column
   constexpr int NG = num_ghosts<MX>();
-  constexpr unsigned FULL = 0xffffffffu;
+  constexpr unsigned kAll = 0xffffffffu;
   constexpr uint32_t bytes = sizeof(real) * S * S;
   static_assert(MX % R == 0 && NW % 32 == 0 && NT % 32 == 0, "bands of R rows, whole warps");
   __shared__ __align__(128) real Q[S * S];
@@ -89,21 +89,19 @@ __global__ void __launch_bounds__(band_threads<real, MX, R>(), band_min_blocks<r
   // thread 0 initialises the copy barrier, issues the copies and waits for
   // them; the other threads touch the barrier only after a CTA barrier
   if (tid == 0) mbar_init(&bar, 1);
-  const real cu = real(D.vel[0]), cv = real(D.vel[1]);
-  const real h = real(a.h);
-  const Scheme<real> sc = make_scheme<real>(D.order, D.limiter, D.transverse, a.nu);
-  const real dt = real(a.dt), tdt = D.transverse > 0 ? real(0.5 * a.dt) : real(0);
+  const real cu = ac.cu, cv = ac.cv, h = ac.h;
+  const Scheme<real, FULL> sc = make_scheme<real, FULL>(D.order, D.limiter, D.transverse);
+  const real hdt = ac.hdt, bfac = ac.bfac;
   auto q = [&](int i, int j) -> real { return Q[(j + kMbc) * S + (i + kMbc)]; };
   // capacity form: 1/kappa of cell (i, j), volume flux of x-edge (i, j) /
-  // y-edge (i, j), and an edge's correction dt/h from its two cells
+  // y-edge (i, j) times dt / 2
   auto ik = [&](int i, int j) -> real { return real(1) / real(Ms[(j + kMbc) * S + i + kMbc]); };
   auto phx = [&](int i, int j) -> real {
-    return real(Ms[S * S + (j + kMbc) * (S + 1) + i + kMbc]);
+    return hdt * real(Ms[S * S + (j + kMbc) * (S + 1) + i + kMbc]);
   };
   auto phy = [&](int i, int j) -> real {
-    return real(Ms[S * S + S * (S + 1) + (j + kMbc) * S + i + kMbc]);
+    return hdt * real(Ms[S * S + S * (S + 1) + (j + kMbc) * S + i + kMbc]);
   };
-  auto nu_e = [&](real ika, real ikb) -> real { return dt * (real(0.5) * (ika + ikb)); };
 
   uint32_t parity = 0;
   for (int p = p0 + blockIdx.x; p < p1; p += gridDim.x, parity ^= 1) {
@@ -120,7 +118,7 @@ __global__ void __launch_bounds__(band_threads<real, MX, R>(), band_min_blocks<r
     // ghost); read after the barrier below
     if (SWIRL && tid == NT - 1 && p == p0 + (int)blockIdx.x) {
       const double t = a.t0_dev ? *a.t0_dev + a.t_off : a.t_half;
-      ucoef_s = cospi_ratio<real>(t, a.period) * real(a.sfac);
+      ucoef_s = cospi_ratio<real>(t, a.period) * real(a.sfac * 0.5 * a.nu);
     }
     if (SWIRL) {  // the tables, while the tile is in flight
       for (int k = tid; k < 4 * NV; k += NT) {
@@ -140,7 +138,7 @@ __global__ void __launch_bounds__(band_threads<real, MX, R>(), band_min_blocks<r
     // table itself: no staging pass, no barrier before the gather
     if (a.gather)
       gather_ring<real, MX>(
-          D, [&](int r) { return D.nbr[(size_t)p * 8 + r]; }, p, pm, a.tlevel, real(a.alpha),
+          D, [&](int r) { return D.nbr[(size_t)p * 8 + r]; }, p, pm, a.tlevel, ac.alpha,
           a.direct != 0, ring, ring_w, tid, NT, static_cast<real*>(a.keep_t), a.keep_t_p0);
     // thread 0 observes the copy's completion (bounded), the others after the
     // barrier (at once); the CTA leaves together if it gave up
@@ -175,19 +173,19 @@ __global__ void __launch_bounds__(band_threads<real, MX, R>(), band_min_blocks<r
       real Fn, P, M;
       if (k < MX + 2) {
         const int r = k - 1;
-        const real s = CAP ? phx(MX, r) : SWIRL ? ucoef * Sx[MX + 1] * Ty[r + 1] : cu;
-        const real nu = CAP ? nu_e(ik(MX - 1, r), ik(MX, r)) : sc.nu;
-        edge(s, q(MX - 2, r), q(MX - 1, r), q(MX, r), q(MX + 1, r), nu, sc, Fn, P, M);
+        const real c = CAP ? phx(MX, r) : SWIRL ? (ucoef * Sx[MX + 1]) * Ty[r + 1] : cu;
+        const real kf = CAP ? corr_factor_cap(c, ik(MX - 1, r) + ik(MX, r), sc) : corr_factor(c, sc);
+        edge(c, q(MX - 2, r), q(MX - 1, r), q(MX, r), q(MX + 1, r), kf, sc, Fn, P, M);
         FeN[k] = Fn;
-        FeU[k] = s;
+        FeU[k] = c;
         XMe[k] = M;
       } else {
         const bool right = k >= 2 * MX + 3;
         const int r = k - (right ? 2 * MX + 3 : MX + 2);
-        const int c = right ? MX : -1;
-        const real s = CAP ? phy(c, r) : SWIRL ? -ucoef * Sy[r + 1] * Tx[c + 1] : cv;
-        const real nu = CAP ? nu_e(ik(c, r - 1), ik(c, r)) : sc.nu;
-        edge(s, q(c, r - 2), q(c, r - 1), q(c, r), q(c, r + 1), nu, sc, Fn, P, M);
+        const int i = right ? MX : -1;
+        const real c = CAP ? phy(i, r) : SWIRL ? (-ucoef * Tx[i + 1]) * Sy[r + 1] : cv;
+        const real kf = CAP ? corr_factor_cap(c, ik(i, r - 1) + ik(i, r), sc) : corr_factor(c, sc);
+        edge(c, q(i, r - 2), q(i, r - 1), q(i, r), q(i, r + 1), kf, sc, Fn, P, M);
         (right ? YPp : YPm)[r] = P;
         (right ? YMp : YMm)[r] = M;
       }
@@ -199,8 +197,12 @@ __global__ void __launch_bounds__(band_threads<real, MX, R>(), band_min_blocks<r
     real* bf = a.bflux ? static_cast<real*>(a.bflux) + ((size_t)p * 2 + a.bslot) * 4 * MX
                        : nullptr;
     if (tid < NW) {  // (the warps beyond the bands only gathered ghosts)
-      const real Sx_i = SWIRL ? Sx[li + 1] : real(0), Tx_i = SWIRL ? Tx[li + 1] : real(0);
+      const real ux = SWIRL ? ucoef * Sx[li + 1] : real(0);   // times Ty of the row: x-edge
+      const real vy = SWIRL ? -ucoef * Tx[li + 1] : real(0);  // times Sy of the row: y-edge
       real qa = q(li, r0 - 2), qb = q(li, r0 - 1), qc = q(li, r0), qd = 0;
+      real Wa = qb - qa, Wb = qc - qb;  // jumps of y-edges (li, r), (li, r + 1)
+      // fluctuation sums into cells (capacity form: over the cell's area) and
+      // final fluxes carried from row to row
       real X_prev = 0, Gn_cur = 0, v_cur = 0, YP_cur = 0, Gf_prev = 0, dF_prev = 0;
       // capacity form: 1/kappa of this column's cells in rows r-1, r
       real ik_prev = CAP ? ik(li, r0 - 2) : real(0), ik_cur = CAP ? ik(li, r0 - 1) : real(0);
@@ -208,63 +210,57 @@ __global__ void __launch_bounds__(band_threads<real, MX, R>(), band_min_blocks<r
       for (int it = 0; it < R + 2; ++it) {
         const int r = r0 - 1 + it;
         if (it <= R) qd = q(li, r + 2);
+        const real Wc = qd - qc;  // jump of y-edge (li, r + 2)
         const real ik_next = CAP && it <= R ? ik(li, r + 1) : real(0);
-        real ik_left = CAP ? __shfl_up_sync(FULL, ik_cur, 1, MX) : real(0);  // cell (li-1, r)
+        real ik_left = CAP ? __shfl_up_sync(kAll, ik_cur, 1, MX) : real(0);  // cell (li-1, r)
         if (CAP && li == 0) ik_left = ik(-1, r);
         // x-edge (li, r): cells (li-1, r) | (li, r)
-        const real su = CAP ? phx(li, r) : SWIRL ? ucoef * Sx_i * Ty[r + 1] : cu;
+        const real cx = CAP ? phx(li, r) : SWIRL ? ux * Ty[r + 1] : cu;
         real Fn_r, XP_r, XM_r;
-        edge(su, q(li - 2, r), q(li - 1, r), qb, q(li + 1, r),
-             CAP ? nu_e(ik_left, ik_cur) : sc.nu, sc, Fn_r, XP_r, XM_r);
-        real XMn = __shfl_down_sync(FULL, XM_r, 1, MX);
+        edge(cx, q(li - 2, r), q(li - 1, r), qb, q(li + 1, r),
+             CAP ? corr_factor_cap(cx, ik_left + ik_cur, sc) : corr_factor(cx, sc), sc, Fn_r,
+             XP_r, XM_r);
+        real XMn = __shfl_down_sync(kAll, XM_r, 1, MX);
         if (li == MX - 1) XMn = XMe[r + 1];
-        const real X_r = XP_r + XMn;  // x-fluctuation into cell (li, r)
+        const real X_r = CAP ? (XP_r + XMn) * ik_cur : XP_r + XMn;  // into cell (li, r)
         // y-edge (li, r+1): cells (li, r) | (li, r+1); the last row's is the
         // next band's
         real Gn_n = 0, YP_n = 0, YM_n = 0, v_n = 0;
         if (it <= R) {
-          v_n = CAP ? phy(li, r + 1) : SWIRL ? -ucoef * Sy[r + 2] * Tx_i : cv;
-          edge(v_n, qa, qb, qc, qd, CAP ? nu_e(ik_cur, ik_next) : sc.nu, sc, Gn_n, YP_n, YM_n);
+          v_n = CAP ? phy(li, r + 1) : SWIRL ? vy * Sy[r + 2] : cv;
+          edge_flux(v_n, Wb, upwind_left(v_n) ? Wa : Wc, qb, qc,
+                    CAP ? corr_factor_cap(v_n, ik_cur + ik_next, sc) : corr_factor(v_n, sc), sc,
+                    Gn_n, YP_n, YM_n);
         }
         // final flux at y-edge (li, r)
         real Gf_r = 0;
         if (it >= 1) {
-          if (CAP)
-            Gf_r = Gn_cur - tdt * (fmax(v_cur, real(0)) * X_prev * ik_prev +
-                                   fmin(v_cur, real(0)) * X_r * ik_cur);
-          else
-            Gf_r = Gn_cur - sc.tfac * (fmax(v_cur, real(0)) * X_prev + fmin(v_cur, real(0)) * X_r);
-          if (bf && r == 0) bf[2 * MX + li] = Gf_r;
-          if (bf && r == MX) bf[3 * MX + li] = Gf_r;
+          Gf_r = final_flux(v_cur, X_prev, X_r, Gn_cur, sc);
+          if (bf && r == 0) bf[2 * MX + li] = Gf_r * bfac;
+          if (bf && r == MX) bf[3 * MX + li] = Gf_r * bfac;
         }
         // final fluxes at x-edges (li, r) and (li+1, r), rows of the band
         real dF_r = 0;
         if (it >= 1 && it <= R) {
-          const real Y_r = YP_cur + YM_n;  // y-fluctuation into cell (li, r)
-          real Yl = __shfl_up_sync(FULL, Y_r, 1, MX);
-          if (li == 0) Yl = YPm[r] + YMm[r + 1];
-          const real Ff =
-              CAP ? Fn_r - tdt * (fmax(su, real(0)) * Yl * ik_left + fmin(su, real(0)) * Y_r * ik_cur)
-                  : Fn_r - sc.tfac * (fmax(su, real(0)) * Yl + fmin(su, real(0)) * Y_r);
-          real Fr = __shfl_down_sync(FULL, Ff, 1, MX);
+          // y-fluctuation sum into cell (li, r)
+          const real Y_r = CAP ? (YP_cur + YM_n) * ik_cur : YP_cur + YM_n;
+          real Yl = __shfl_up_sync(kAll, Y_r, 1, MX);
+          if (li == 0) Yl = CAP ? (YPm[r] + YMm[r + 1]) * ik_left : YPm[r] + YMm[r + 1];
+          const real Ff = final_flux(cx, Yl, Y_r, Fn_r, sc);
+          real Fr = __shfl_down_sync(kAll, Ff, 1, MX);
           if (li == MX - 1) {
-            const real ue = FeU[r + 1];
-            if (CAP)
-              Fr = FeN[r + 1] - tdt * (fmax(ue, real(0)) * Y_r * ik_cur +
-                                       fmin(ue, real(0)) * (YPp[r] + YMp[r + 1]) * ik(MX, r));
-            else
-              Fr = FeN[r + 1] - sc.tfac * (fmax(ue, real(0)) * Y_r +
-                                           fmin(ue, real(0)) * (YPp[r] + YMp[r + 1]));
+            const real Yr = CAP ? (YPp[r] + YMp[r + 1]) * ik(MX, r) : YPp[r] + YMp[r + 1];
+            Fr = final_flux(FeU[r + 1], Y_r, Yr, FeN[r + 1], sc);
           }
           dF_r = Fr - Ff;
-          if (bf && li == 0) bf[r] = Ff;
-          if (bf && li == MX - 1) bf[MX + r] = Fr;
+          if (bf && li == 0) bf[r] = Ff * bfac;
+          if (bf && li == MX - 1) bf[MX + r] = Fr * bfac;
         }
         // conservative update of cell (li, r-1)
-        if (it >= 2)
-          dst[(r + 1) * S + (li + kMbc)] =
-              CAP ? qa - dt * ik_prev * (dF_prev + (Gf_r - Gf_prev))
-                  : qa - sc.nu * dF_prev - sc.nu * (Gf_r - Gf_prev);
+        if (it >= 2) {
+          const real d = dF_prev + (Gf_r - Gf_prev);
+          dst[(r + 1) * S + (li + kMbc)] = fma(real(-2), CAP ? d * ik_prev : d, qa);
+        }
         X_prev = X_r;
         Gn_cur = Gn_n;
         v_cur = v_n;
@@ -274,6 +270,8 @@ __global__ void __launch_bounds__(band_threads<real, MX, R>(), band_min_blocks<r
         qa = qb;
         qb = qc;
         qc = qd;
+        Wa = Wb;
+        Wb = Wc;
         ik_prev = ik_cur;
         ik_cur = ik_next;
       }
@@ -282,11 +280,11 @@ __global__ void __launch_bounds__(band_threads<real, MX, R>(), band_min_blocks<r
   }
 }
 
-template <typename real, int MX, int R, bool SWIRL, bool CAP>
+template <typename real, int MX, int R, bool SWIRL, bool CAP, bool FULL>
 cudaError_t band_launch_t(const DevForest<real>& D, int p0, int p1, const AdvArgs& a, int* err,
                           cudaStream_t s) {
   constexpr size_t dyn = CAP ? sizeof(double) * (size_t)metric_stride(MX + 4) : 0;
-  auto kern = advance_band_kernel<real, MX, R, SWIRL, CAP>;
+  auto kern = advance_band_kernel<real, MX, R, SWIRL, CAP, FULL>;
   if (CAP) {  // set once per process; concurrent first calls both set it (idempotent)
     static std::atomic<bool> attr_set{false};
     if (!attr_set.load(std::memory_order_acquire)) {
@@ -296,18 +294,26 @@ cudaError_t band_launch_t(const DevForest<real>& D, int p0, int p1, const AdvArg
       attr_set.store(true, std::memory_order_release);
     }
   }
-  kern<<<p1 - p0, band_threads<real, MX, R>(), dyn, s>>>(D, p0, p1, a, err);
+  kern<<<p1 - p0, band_threads<real, MX, R>(), dyn, s>>>(D, p0, p1, a, adv_const(D, a), err);
   ++launch_counter();
   return cudaGetLastError();
+}
+
+template <typename real, int MX, int R, bool FULL>
+cudaError_t band_launch_f(const DevForest<real>& D, int p0, int p1, const AdvArgs& a, int* err,
+                        cudaStream_t s) {
+  if (D.metric) return band_launch_t<real, MX, R, false, true, FULL>(D, p0, p1, a, err, s);
+  if (D.vel_kind == FC_VEL_SWIRL)
+    return band_launch_t<real, MX, R, true, false, FULL>(D, p0, p1, a, err, s);
+  return band_launch_t<real, MX, R, false, false, FULL>(D, p0, p1, a, err, s);
 }
 
 template <typename real, int MX, int R>
 cudaError_t band_launch(const DevForest<real>& D, int p0, int p1, const AdvArgs& a, int* err,
                         cudaStream_t s) {
-  if (D.metric) return band_launch_t<real, MX, R, false, true>(D, p0, p1, a, err, s);
-  if (D.vel_kind == FC_VEL_SWIRL)
-    return band_launch_t<real, MX, R, true, false>(D, p0, p1, a, err, s);
-  return band_launch_t<real, MX, R, false, false>(D, p0, p1, a, err, s);
+  return full_scheme(D.order, D.limiter, D.transverse)
+             ? band_launch_f<real, MX, R, true>(D, p0, p1, a, err, s)
+             : band_launch_f<real, MX, R, false>(D, p0, p1, a, err, s);
 }
 
 }  // namespace
@@ -331,9 +337,8 @@ cudaError_t launch_advance_band(const DevForest<real>& D, int p0, int p1, const 
   }
 }
 
-template cudaError_t launch_advance_band<float>(const DevForest<float>&, int, int,
-                                                const AdvArgs&, int*, cudaStream_t);
-template cudaError_t launch_advance_band<double>(const DevForest<double>&, int, int,
-                                                 const AdvArgs&, int*, cudaStream_t);
+// (compiled once per precision, see build.py)
+template cudaError_t launch_advance_band<FC_REAL>(const DevForest<FC_REAL>&, int, int,
+                                                  const AdvArgs&, int*, cudaStream_t);
 
 }  // namespace fc

@@ -45,15 +45,16 @@ constexpr int warp_reals() {
   return NB * (32 / MX) * tile_stride<MX>() + (32 / MX) * side_reals<MX>();
 }
 
-template <typename real, int MX, int NW, bool SWIRL, int NB>
+template <typename real, int MX, int NW, bool SWIRL, int NB, bool FULL>
 __global__ void __launch_bounds__(NW * 32) advance_walk_kernel(DevForest<real> D, int p0, int p1,
-                                                               AdvArgs a, int* err) {
+                                                               AdvArgs a, AdvConst<real> ac,
+                                                               int* err) {
   constexpr int S = MX + 4;
   constexpr int PPW = 32 / MX;
   constexpr int TILE = S * S;
   constexpr int TS = tile_stride<MX>();
   constexpr int NS = MX + 3;
-  constexpr unsigned FULL = 0xffffffffu;
+  constexpr unsigned kAll = 0xffffffffu;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t bars[NW][2];
   __shared__ real ucoef_s;
@@ -75,7 +76,7 @@ __global__ void __launch_bounds__(NW * 32) advance_walk_kernel(DevForest<real> D
 
   if (threadIdx.x == 0 && SWIRL) {
     const double t = a.t0_dev ? *a.t0_dev + a.t_off : a.t_half;
-    ucoef_s = cospi_ratio<real>(t, a.period) * real(a.sfac);
+    ucoef_s = cospi_ratio<real>(t, a.period) * real(a.sfac * 0.5 * a.nu);
   }
   if (lane == 0) {
     mbar_init(&bars[warp][0], 1);
@@ -84,9 +85,8 @@ __global__ void __launch_bounds__(NW * 32) advance_walk_kernel(DevForest<real> D
   __syncthreads();
 
   const real ucoef = SWIRL ? ucoef_s : real(0);
-  const real cu = real(D.vel[0]), cv = real(D.vel[1]);
-  const real h = real(a.h);
-  const Scheme<real> sc = make_scheme<real>(D.order, D.limiter, D.transverse, a.nu);
+  const real cu = ac.cu, cv = ac.cv, h = ac.h;
+  const Scheme<real, FULL> sc = make_scheme<real, FULL>(D.order, D.limiter, D.transverse);
 
   const int ngroups = (p1 - p0 + PPW - 1) / PPW;
   const int TW = gridDim.x * NW;
@@ -131,7 +131,7 @@ __global__ void __launch_bounds__(NW * 32) advance_walk_kernel(DevForest<real> D
     }
     uint32_t& par = b ? par1 : par0;
     const bool ok = mbar_wait(&bars[warp][b], par, a.wait_limit);
-    if (!__all_sync(FULL, ok)) {
+    if (!__all_sync(kAll, ok)) {
       if (lane == 0) atomicOr(err, kErrTimeout);
       // let every copy in flight land before leaving
       mbar_wait(&bars[warp][b], par, kWaitLimit);
@@ -152,7 +152,7 @@ __global__ void __launch_bounds__(NW * 32) advance_walk_kernel(DevForest<real> D
         ghost_ij<MX>(k, i, j);
         const NbrEntry& e = ns.e[region_of<MX>(i, j)];
         real v;
-        if (copy_or_average_entry<real, MX>(D, e, pm, a.tlevel, real(a.alpha), i, j, v) ||
+        if (copy_or_average_entry<real, MX>(D, e, pm, a.tlevel, ac.alpha, i, j, v) ||
             interpolate_entry<real, MX>(D, e, pm, a.tlevel, i, j, v))
           T[(j + kMbc) * S + i + kMbc] = v;
       }
@@ -177,19 +177,22 @@ __global__ void __launch_bounds__(NW * 32) advance_walk_kernel(DevForest<real> D
       SyS[r + 1] = sy;
       real Fn, P, M;
       if (r <= MX) {  // x-edge MX of row r
-        const real s = SWIRL ? ucoef * SxE * ty : cu;
-        edge(s, Q(MX - 2, r), Q(MX - 1, r), Q(MX, r), Q(MX + 1, r), sc, Fn, P, M);
+        const real c = SWIRL ? (ucoef * SxE) * ty : cu;
+        edge(c, Q(MX - 2, r), Q(MX - 1, r), Q(MX, r), Q(MX + 1, r), corr_factor(c, sc), sc, Fn, P,
+             M);
         FeN[r + 1] = Fn;
-        FeU[r + 1] = s;
+        FeU[r + 1] = c;
         XMe[r + 1] = M;
       }
       if (r >= 0 && r <= MX) {  // y-edges of ghost columns -1 and MX at row r
-        const real sl = SWIRL ? -ucoef * sy * TxM : cv;
-        edge(sl, Q(-1, r - 2), Q(-1, r - 1), Q(-1, r), Q(-1, r + 1), sc, Fn, P, M);
+        const real cl = SWIRL ? (-ucoef * TxM) * sy : cv;
+        edge(cl, Q(-1, r - 2), Q(-1, r - 1), Q(-1, r), Q(-1, r + 1), corr_factor(cl, sc), sc, Fn,
+             P, M);
         YPm[r] = P;
         YMm[r] = M;
-        const real sr = SWIRL ? -ucoef * sy * TxP : cv;
-        edge(sr, Q(MX, r - 2), Q(MX, r - 1), Q(MX, r), Q(MX, r + 1), sc, Fn, P, M);
+        const real cr = SWIRL ? (-ucoef * TxP) * sy : cv;
+        edge(cr, Q(MX, r - 2), Q(MX, r - 1), Q(MX, r), Q(MX, r + 1), corr_factor(cr, sc), sc, Fn,
+             P, M);
         YPp[r] = P;
         YMp[r] = M;
       }
@@ -198,46 +201,47 @@ __global__ void __launch_bounds__(NW * 32) advance_walk_kernel(DevForest<real> D
 
     // main walk: lane li owns column li; iteration r computes x-edge (li, r)
     // and y-edge (li, r+1), finishes the fluxes of row r and updates row r-1
+    const real ux = ucoef * Sx_i, vy = -ucoef * Tx_i;
     real qa = Q(li, -2), qb = Q(li, -1), qc = Q(li, 0), qd = 0;
+    real Wa = qb - qa, Wb = qc - qb;  // jumps of y-edges (li, r), (li, r + 1)
     real X_prev = 0, Gn_cur = 0, v_cur = 0, YP_cur = 0, Gf_prev = 0, dF_prev = 0;
 #pragma unroll 2  // fully unrolled, the row walk overflowed the instruction cache
     for (int r = -1; r <= MX; ++r) {
       if (r + 2 <= MX + 1) qd = Q(li, r + 2);
+      const real Wc = qd - qc;  // jump of y-edge (li, r + 2)
       // x-edge (li, r): cells (li-1, r) | (li, r)
-      const real su = SWIRL ? ucoef * Sx_i * TyS[r + 1] : cu;
+      const real cx = SWIRL ? ux * TyS[r + 1] : cu;
       real Fn_r, XP_r, XM_r;
-      edge(su, Q(li - 2, r), Q(li - 1, r), qb, Q(li + 1, r), sc, Fn_r, XP_r, XM_r);
-      real XMn = __shfl_down_sync(FULL, XM_r, 1, MX);
+      edge(cx, Q(li - 2, r), Q(li - 1, r), qb, Q(li + 1, r), corr_factor(cx, sc), sc, Fn_r, XP_r,
+           XM_r);
+      real XMn = __shfl_down_sync(kAll, XM_r, 1, MX);
       if (li == MX - 1) XMn = XMe[r + 1];
       const real X_r = XP_r + XMn;  // x-fluctuation into cell (li, r)
       // y-edge (li, r+1): cells (li, r) | (li, r+1)
       real Gn_n = 0, YP_n = 0, YM_n = 0, v_n = 0;
       if (r + 1 <= MX) {
-        v_n = SWIRL ? -ucoef * SyS[r + 2] * Tx_i : cv;
-        edge(v_n, qa, qb, qc, qd, sc, Gn_n, YP_n, YM_n);
+        v_n = SWIRL ? vy * SyS[r + 2] : cv;
+        edge_flux(v_n, Wb, upwind_left(v_n) ? Wa : Wc, qb, qc, corr_factor(v_n, sc), sc, Gn_n,
+                  YP_n, YM_n);
       }
       // final flux at y-edge (li, r)
       real Gf_r = 0;
-      if (r >= 0)
-        Gf_r = Gn_cur - sc.tfac * (fmax(v_cur, real(0)) * X_prev + fmin(v_cur, real(0)) * X_r);
+      if (r >= 0) Gf_r = final_flux(v_cur, X_prev, X_r, Gn_cur, sc);
       // final fluxes at x-edges (li, r) and (li+1, r)
       real dF_r = 0;
       if (r >= 0 && r < MX) {
         const real Y_r = YP_cur + YM_n;  // y-fluctuation into cell (li, r)
-        real Yl = __shfl_up_sync(FULL, Y_r, 1, MX);
+        real Yl = __shfl_up_sync(kAll, Y_r, 1, MX);
         if (li == 0) Yl = YPm[r] + YMm[r + 1];
-        const real Ff = Fn_r - sc.tfac * (fmax(su, real(0)) * Yl + fmin(su, real(0)) * Y_r);
-        real Fr = __shfl_down_sync(FULL, Ff, 1, MX);
-        if (li == MX - 1) {
-          const real ue = FeU[r + 1];
-          Fr = FeN[r + 1] -
-               sc.tfac * (fmax(ue, real(0)) * Y_r + fmin(ue, real(0)) * (YPp[r] + YMp[r + 1]));
-        }
+        const real Ff = final_flux(cx, Yl, Y_r, Fn_r, sc);
+        real Fr = __shfl_down_sync(kAll, Ff, 1, MX);
+        if (li == MX - 1)
+          Fr = final_flux(FeU[r + 1], Y_r, YPp[r] + YMp[r + 1], FeN[r + 1], sc);
         dF_r = Fr - Ff;
       }
       // conservative update of cell (li, r-1)
       if (r >= 1 && valid)
-        dst[(r + 1) * S + (li + 2)] = qa - sc.nu * dF_prev - sc.nu * (Gf_r - Gf_prev);
+        dst[(r + 1) * S + (li + 2)] = fma(real(-2), dF_prev + (Gf_r - Gf_prev), qa);
       X_prev = X_r;
       Gn_cur = Gn_n;
       v_cur = v_n;
@@ -247,19 +251,21 @@ __global__ void __launch_bounds__(NW * 32) advance_walk_kernel(DevForest<real> D
       qa = qb;
       qb = qc;
       qc = qd;
+      Wa = Wb;
+      Wb = Wc;
     }
     __syncwarp();
   }
 }
 
-template <typename real, int MX, int NW, bool SWIRL, int NB>
+template <typename real, int MX, int NW, bool SWIRL, int NB, bool FULL>
 cudaError_t walk_launch(const DevForest<real>& D, int p0, int p1, const AdvArgs& a, int* err,
                         cudaStream_t s) {
   // computed once per process; concurrent first calls compute the same value
   static std::atomic<int> max_ctas_once{0};
   int max_ctas = max_ctas_once.load(std::memory_order_acquire);
   constexpr size_t smem = sizeof(real) * (size_t)NW * warp_reals<real, MX, NB>();
-  auto kern = advance_walk_kernel<real, MX, NW, SWIRL, NB>;
+  auto kern = advance_walk_kernel<real, MX, NW, SWIRL, NB, FULL>;
   if (max_ctas == 0) {
     cudaError_t e =
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -277,29 +283,37 @@ cudaError_t walk_launch(const DevForest<real>& D, int p0, int p1, const AdvArgs&
   int ctas = (groups + NW - 1) / NW;
   const int cap = a.ctas > 0 ? a.ctas : max_ctas;
   if (ctas > cap) ctas = cap;
-  kern<<<ctas, NW * 32, smem, s>>>(D, p0, p1, a, err);
+  kern<<<ctas, NW * 32, smem, s>>>(D, p0, p1, a, adv_const(D, a), err);
   ++launch_counter();
   return cudaGetLastError();
 }
 
-template <typename real, int MX, int NW>
+template <typename real, int MX, int NW, bool FULL>
 cudaError_t walk_vel(const DevForest<real>& D, int p0, int p1, const AdvArgs& a, int* err,
                      cudaStream_t s) {
   const bool one = a.variant == ADV_WALK1;
   if (D.vel_kind == FC_VEL_SWIRL)
-    return one ? walk_launch<real, MX, NW, true, 1>(D, p0, p1, a, err, s)
-               : walk_launch<real, MX, NW, true, 2>(D, p0, p1, a, err, s);
-  return one ? walk_launch<real, MX, NW, false, 1>(D, p0, p1, a, err, s)
-             : walk_launch<real, MX, NW, false, 2>(D, p0, p1, a, err, s);
+    return one ? walk_launch<real, MX, NW, true, 1, FULL>(D, p0, p1, a, err, s)
+               : walk_launch<real, MX, NW, true, 2, FULL>(D, p0, p1, a, err, s);
+  return one ? walk_launch<real, MX, NW, false, 1, FULL>(D, p0, p1, a, err, s)
+             : walk_launch<real, MX, NW, false, 2, FULL>(D, p0, p1, a, err, s);
+}
+
+template <typename real, int MX, int NW>
+cudaError_t walk_opt(const DevForest<real>& D, int p0, int p1, const AdvArgs& a, int* err,
+                     cudaStream_t s) {
+  return full_scheme(D.order, D.limiter, D.transverse)
+             ? walk_vel<real, MX, NW, true>(D, p0, p1, a, err, s)
+             : walk_vel<real, MX, NW, false>(D, p0, p1, a, err, s);
 }
 
 template <typename real, int MX>
 cudaError_t walk_nw(const DevForest<real>& D, int p0, int p1, const AdvArgs& a, int* err,
                     cudaStream_t s) {
   switch (a.warps) {
-    case 2: return walk_vel<real, MX, 2>(D, p0, p1, a, err, s);
-    case 8: return walk_vel<real, MX, 8>(D, p0, p1, a, err, s);
-    default: return walk_vel<real, MX, 4>(D, p0, p1, a, err, s);
+    case 2: return walk_opt<real, MX, 2>(D, p0, p1, a, err, s);
+    case 8: return walk_opt<real, MX, 8>(D, p0, p1, a, err, s);
+    default: return walk_opt<real, MX, 4>(D, p0, p1, a, err, s);
   }
 }
 
@@ -316,9 +330,8 @@ cudaError_t launch_advance_walk(const DevForest<real>& D, int p0, int p1, const 
   }
 }
 
-template cudaError_t launch_advance_walk<float>(const DevForest<float>&, int, int,
-                                                const AdvArgs&, int*, cudaStream_t);
-template cudaError_t launch_advance_walk<double>(const DevForest<double>&, int, int,
-                                                 const AdvArgs&, int*, cudaStream_t);
+// (compiled once per precision, see build.py)
+template cudaError_t launch_advance_walk<FC_REAL>(const DevForest<FC_REAL>&, int, int,
+                                                  const AdvArgs&, int*, cudaStream_t);
 
 }  // namespace fc

@@ -7,7 +7,8 @@ namespace fc {
 
 template <typename real>
 __device__ __forceinline__ real minmod(real a, real b) {
-  if (a * b <= real(0)) return real(0);
+  // by the signs: a product of two small slopes underflows
+  if ((a <= real(0) && b >= real(0)) || (a >= real(0) && b <= real(0))) return real(0);
   return fabs(a) < fabs(b) ? a : b;
 }
 
