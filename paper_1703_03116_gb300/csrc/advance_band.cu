@@ -68,6 +68,7 @@ __global__ void __launch_bounds__(band_threads<real, MX, R>(), band_min_blocks<r
   constexpr int NG = num_ghosts<MX>();
   constexpr unsigned kAll = 0xffffffffu;
   constexpr uint32_t bytes = sizeof(real) * S * S;
+  static_assert(NT >= 4 * NV, "a thread per table entry");
   static_assert(MX % R == 0 && NW % 32 == 0 && NT % 32 == 0, "bands of R rows, whole warps");
   __shared__ __align__(128) real Q[S * S];
   __shared__ __align__(8) uint64_t bar;
@@ -92,6 +93,7 @@ __global__ void __launch_bounds__(band_threads<real, MX, R>(), band_min_blocks<r
   const real cu = ac.cu, cv = ac.cv, h = ac.h;
   const Scheme<real, FULL> sc = make_scheme<real, FULL>(D.order, D.limiter, D.transverse);
   const real hdt = ac.hdt, bfac = ac.bfac;
+  const real* tab = static_cast<const real*>(a.trig);  // the level's streamfunction factors
   auto q = [&](int i, int j) -> real { return Q[(j + kMbc) * S + (i + kMbc)]; };
   // capacity form: 1/kappa of cell (i, j), volume flux of x-edge (i, j) /
   // y-edge (i, j) times dt / 2
@@ -120,18 +122,20 @@ __global__ void __launch_bounds__(band_threads<real, MX, R>(), band_min_blocks<r
       const double t = a.t0_dev ? *a.t0_dev + a.t_off : a.t_half;
       ucoef_s = cospi_ratio<real>(t, a.period) * real(a.sfac * 0.5 * a.nu);
     }
-    if (SWIRL) {  // the tables, while the tile is in flight
-      for (int k = tid; k < 4 * NV; k += NT) {
-        const int tb = k / NV, c = k % NV;
-        const int z = (tb & 1 ? pm.y : pm.x) * MX + c - 1;
-        real v;
-        if (tb < 2) {
-          v = sinpi_r(real(z) * h);
-          v *= v;
-        } else {
-          v = sinpi_r(real(2 * z + 1) * h);
-        }
-        (tb == 0 ? Sx : tb == 1 ? Sy : tb == 2 ? Tx : Ty)[c] = v;
+    // the tables, one entry a thread: read (FP64) or computed (FP32: cheaper
+    // than the read by 1%) now, stored after the gather, whose reads are not
+    // to wait for this one's
+    real tv = real(0);
+    if (SWIRL && tid < 4 * NV) {
+      const int tb = tid / NV, c = tid % NV;
+      const int z = (tb & 1 ? pm.y : pm.x) * MX + c - 1;
+      if (sizeof(real) == 8 && tab) {
+        tv = tab[(tb < 2 ? 0 : a.trig_len) + z + 1];
+      } else if (tb < 2) {
+        tv = sinpi_r(real(z) * h);
+        tv *= tv;
+      } else {
+        tv = sinpi_r(real(2 * z + 1) * h);
       }
     }
     // each gathering thread reads the entry of its ghost's region from the
@@ -140,6 +144,10 @@ __global__ void __launch_bounds__(band_threads<real, MX, R>(), band_min_blocks<r
       gather_ring<real, MX>(
           D, [&](int r) { return D.nbr[(size_t)p * 8 + r]; }, p, pm, a.tlevel, ac.alpha,
           a.direct != 0, ring, ring_w, tid, NT, static_cast<real*>(a.keep_t), a.keep_t_p0);
+    if (SWIRL && tid < 4 * NV) {
+      const int tb = tid / NV, c = tid % NV;
+      (tb == 0 ? Sx : tb == 1 ? Sy : tb == 2 ? Tx : Ty)[c] = tv;
+    }
     // thread 0 observes the copy's completion (bounded), the others after the
     // barrier (at once); the CTA leaves together if it gave up
     const bool landed = tid == 0 ? mbar_wait(&bar, parity, a.wait_limit) : true;
@@ -170,12 +178,12 @@ __global__ void __launch_bounds__(band_threads<real, MX, R>(), band_min_blocks<r
     // the sides: x-edge MX of rows -1..MX, y-edges of ghost columns -1 and
     // MX at rows 0..MX (one edge a thread)
     for (int k = tid; k < 3 * MX + 4; k += NT) {
-      real Fn, P, M;
+      real Fn, nP, M;
       if (k < MX + 2) {
         const int r = k - 1;
         const real c = CAP ? phx(MX, r) : SWIRL ? (ucoef * Sx[MX + 1]) * Ty[r + 1] : cu;
         const real kf = CAP ? corr_factor_cap(c, ik(MX - 1, r) + ik(MX, r), sc) : corr_factor(c, sc);
-        edge(c, q(MX - 2, r), q(MX - 1, r), q(MX, r), q(MX + 1, r), kf, sc, Fn, P, M);
+        edge(c, q(MX - 2, r), q(MX - 1, r), q(MX, r), q(MX + 1, r), kf, sc, Fn, nP, M);
         FeN[k] = Fn;
         FeU[k] = c;
         XMe[k] = M;
@@ -185,8 +193,8 @@ __global__ void __launch_bounds__(band_threads<real, MX, R>(), band_min_blocks<r
         const int i = right ? MX : -1;
         const real c = CAP ? phy(i, r) : SWIRL ? (-ucoef * Tx[i + 1]) * Sy[r + 1] : cv;
         const real kf = CAP ? corr_factor_cap(c, ik(i, r - 1) + ik(i, r), sc) : corr_factor(c, sc);
-        edge(c, q(i, r - 2), q(i, r - 1), q(i, r), q(i, r + 1), kf, sc, Fn, P, M);
-        (right ? YPp : YPm)[r] = P;
+        edge(c, q(i, r - 2), q(i, r - 1), q(i, r), q(i, r + 1), kf, sc, Fn, nP, M);
+        (right ? YPp : YPm)[r] = nP;
         (right ? YMp : YMm)[r] = M;
       }
     }
@@ -201,9 +209,9 @@ __global__ void __launch_bounds__(band_threads<real, MX, R>(), band_min_blocks<r
       const real vy = SWIRL ? -ucoef * Tx[li + 1] : real(0);  // times Sy of the row: y-edge
       real qa = q(li, r0 - 2), qb = q(li, r0 - 1), qc = q(li, r0), qd = 0;
       real Wa = qb - qa, Wb = qc - qb;  // jumps of y-edges (li, r), (li, r + 1)
-      // fluctuation sums into cells (capacity form: over the cell's area) and
-      // final fluxes carried from row to row
-      real X_prev = 0, Gn_cur = 0, v_cur = 0, YP_cur = 0, Gf_prev = 0, dF_prev = 0;
+      // turned fluctuation sums into cells (capacity form: over the cell's
+      // area) and final fluxes carried from row to row
+      real nX_prev = 0, Gn_cur = 0, v_cur = 0, nP_cur = 0, Gf_prev = 0, dF_prev = 0;
       // capacity form: 1/kappa of this column's cells in rows r-1, r
       real ik_prev = CAP ? ik(li, r0 - 2) : real(0), ik_cur = CAP ? ik(li, r0 - 1) : real(0);
 #pragma unroll(R <= 8 ? R + 2 : 2)
@@ -216,41 +224,41 @@ __global__ void __launch_bounds__(band_threads<real, MX, R>(), band_min_blocks<r
         if (CAP && li == 0) ik_left = ik(-1, r);
         // x-edge (li, r): cells (li-1, r) | (li, r)
         const real cx = CAP ? phx(li, r) : SWIRL ? ux * Ty[r + 1] : cu;
-        real Fn_r, XP_r, XM_r;
+        real Fn_r, nP_r, XM_r;
         edge(cx, q(li - 2, r), q(li - 1, r), qb, q(li + 1, r),
              CAP ? corr_factor_cap(cx, ik_left + ik_cur, sc) : corr_factor(cx, sc), sc, Fn_r,
-             XP_r, XM_r);
+             nP_r, XM_r);
         real XMn = __shfl_down_sync(kAll, XM_r, 1, MX);
         if (li == MX - 1) XMn = XMe[r + 1];
-        const real X_r = CAP ? (XP_r + XMn) * ik_cur : XP_r + XMn;  // into cell (li, r)
+        const real nX_r = CAP ? (nP_r - XMn) * ik_cur : nP_r - XMn;  // into cell (li, r)
         // y-edge (li, r+1): cells (li, r) | (li, r+1); the last row's is the
         // next band's
-        real Gn_n = 0, YP_n = 0, YM_n = 0, v_n = 0;
+        real Gn_n = 0, nP_n = 0, YM_n = 0, v_n = 0;
         if (it <= R) {
           v_n = CAP ? phy(li, r + 1) : SWIRL ? vy * Sy[r + 2] : cv;
           edge_flux(v_n, Wb, upwind_left(v_n) ? Wa : Wc, qb, qc,
                     CAP ? corr_factor_cap(v_n, ik_cur + ik_next, sc) : corr_factor(v_n, sc), sc,
-                    Gn_n, YP_n, YM_n);
+                    Gn_n, nP_n, YM_n);
         }
         // final flux at y-edge (li, r)
         real Gf_r = 0;
         if (it >= 1) {
-          Gf_r = final_flux(v_cur, X_prev, X_r, Gn_cur, sc);
+          Gf_r = final_flux(v_cur, nX_prev, nX_r, Gn_cur, sc);
           if (bf && r == 0) bf[2 * MX + li] = Gf_r * bfac;
           if (bf && r == MX) bf[3 * MX + li] = Gf_r * bfac;
         }
         // final fluxes at x-edges (li, r) and (li+1, r), rows of the band
         real dF_r = 0;
         if (it >= 1 && it <= R) {
-          // y-fluctuation sum into cell (li, r)
-          const real Y_r = CAP ? (YP_cur + YM_n) * ik_cur : YP_cur + YM_n;
-          real Yl = __shfl_up_sync(kAll, Y_r, 1, MX);
-          if (li == 0) Yl = CAP ? (YPm[r] + YMm[r + 1]) * ik_left : YPm[r] + YMm[r + 1];
-          const real Ff = final_flux(cx, Yl, Y_r, Fn_r, sc);
+          // turned y-fluctuation sum into cell (li, r)
+          const real nY_r = CAP ? (nP_cur - YM_n) * ik_cur : nP_cur - YM_n;
+          real nYl = __shfl_up_sync(kAll, nY_r, 1, MX);
+          if (li == 0) nYl = CAP ? (YPm[r] - YMm[r + 1]) * ik_left : YPm[r] - YMm[r + 1];
+          const real Ff = final_flux(cx, nYl, nY_r, Fn_r, sc);
           real Fr = __shfl_down_sync(kAll, Ff, 1, MX);
           if (li == MX - 1) {
-            const real Yr = CAP ? (YPp[r] + YMp[r + 1]) * ik(MX, r) : YPp[r] + YMp[r + 1];
-            Fr = final_flux(FeU[r + 1], Y_r, Yr, FeN[r + 1], sc);
+            const real nYr = CAP ? (YPp[r] - YMp[r + 1]) * ik(MX, r) : YPp[r] - YMp[r + 1];
+            Fr = final_flux(FeU[r + 1], nY_r, nYr, FeN[r + 1], sc);
           }
           dF_r = Fr - Ff;
           if (bf && li == 0) bf[r] = Ff * bfac;
@@ -261,10 +269,10 @@ __global__ void __launch_bounds__(band_threads<real, MX, R>(), band_min_blocks<r
           const real d = dF_prev + (Gf_r - Gf_prev);
           dst[(r + 1) * S + (li + kMbc)] = fma(real(-2), CAP ? d * ik_prev : d, qa);
         }
-        X_prev = X_r;
+        nX_prev = nX_r;
         Gn_cur = Gn_n;
         v_cur = v_n;
-        YP_cur = YP_n;
+        nP_cur = nP_n;
         Gf_prev = Gf_r;
         dF_prev = dF_r;
         qa = qb;

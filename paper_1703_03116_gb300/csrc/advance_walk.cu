@@ -1,22 +1,39 @@
-// The wave-propagation patch update, "walk" variant (sm_103a).
+// The wave-propagation patch update, "walk" variant (sm_103a), for launches
+// that fill the GPU: what bounds them is the instructions a cell takes, not
+// memory (9 bytes a cell move in FP32 at mx = 32, 1/5 of what HBM could).
 //
-// Same scheme as the staged variant (flux-form 2D wave propagation with
-// MC-limited corrections and transverse propagation of both fluctuations),
-// organised for the fewest instructions per cell:
+//  * A lane owns an interior column and walks up the rows with a register
+//    window; per row it computes its x-edge (left edge of its cell) and the
+//    y-edge above; the neighbouring column's results arrive by warp shuffles.
+//  * In FP32 a lane works on two cells at once in packed registers
+//    (walk_edge.cuh): at mx = 32 rows r and r + 16 of one patch (a warp), at
+//    mx = 16 and 8 the same row of two patches (four and eight a warp).  FP64
+//    is bound by its pipe and takes one.
+//  * What a patch's ghosts come from is the same along a face, so the ghost
+//    ring is filled face by face without divergence; from a coarser
+//    neighbour each of the mx/2 coarse cells beside the face is computed
+//    once for its four ghosts, from the states before and after that level's
+//    step, so that no fill kernel runs before the update.  (Ghost by ghost,
+//    with each ghost's own neighbour entry and index transform, the ring took
+//    as many instructions as the update itself.)
+//  * The x-edge and the two y-edge columns outside the lanes (x-edge MX,
+//    ghost columns -1 and MX) are 3 MX + 4 independent edges spread over the
+//    lanes before the walk.
+//  * Tile and neighbour entries arrive by 1D bulk copies; one buffer a warp
+//    and as many warps as fit hide the copies and the gathers' reads.  The
+//    streamfunction's factors come from a table per level.
 //
-//  * A warp works on 32/MX patches at a time; lane li of a patch's segment
-//    owns interior column li and walks up the rows, keeping the column's
-//    values in a four-row register window.  Per row it computes its x-edge
-//    (left edge of its cell) and the y-edge above its window row; the
-//    neighbouring column's results arrive by warp shuffles.
-//  * The one x-edge and the two y-edge columns that fall outside the lanes
-//    (x-edge MX, y-edges of ghost columns -1 and MX) are computed first by a
-//    side pass in which lanes own rows, into small shared arrays.
-//  * Each finished row of cells goes straight to HBM (coalesced); nothing
-//    else is written to shared memory.
-//  * Tiles arrive by 1D TMA bulk copies (cp.async.bulk + mbarrier), double
-//    buffered per warp: the next group of patches is in flight while the
-//    current one is computed.  Grids are persistent (CTAs loop over groups).
+// Measured on one GB300 against the form before it (ghost by ghost after a
+// fill launch, one cell a lane, two tile buffers a warp), a coarse step with
+// its field moves: 256 forests (67168 patches of 32^2, FP32) 6.0 -> 2.7 ms,
+// 64 forests (13852 patches of 16^2, FP64) 3.7 -> 2.5 ms; 16384 patches of
+// 32^2 at one level 94 -> 67 us.  About 3500 warp instructions a 32^2 patch
+// (of 6200), at 55% of the issue slots with 24 warps an SM; its sides are one
+// loop over strides because as four copies of the code they overflowed the
+// instruction cache (4.1 against 2.7 ms).
+//
+// The entries of a square domain's layout keep orientation (a = 0: only the
+// cubed sphere turns axes, and its capacity form runs band or staged).
 #include <atomic>
 #include <cstdint>
 
@@ -26,295 +43,632 @@
 namespace fc {
 namespace {
 
-template <int MX>
-constexpr int tile_stride() {
-  // pad so that the 4 tiles of a warp at MX = 8 start on different banks
-  return MX == 8 ? 168 : (MX + 4) * (MX + 4);
+template <typename real>
+struct Vec2;
+template <>
+struct Vec2<float> {
+  using T = float2;
+};
+template <>
+struct Vec2<double> {
+  using T = double2;
+};
+template <typename real>
+struct alignas(16) EdgeRec {  // x-edge MX of a row: fluctuation into cell MX - 1, normal flux,
+  real M, F, c, nY;           // speed; turned y-fluctuation sum of ghost cell MX
+};
+
+// Shared memory of one patch: its tile, its eight neighbour entries, and per
+// row the streamfunction's factors and the edges beside the lanes.  The
+// stride between patches of a warp is MX modulo 32 elements, so that the
+// segments of a warp read different banks.
+template <typename real, int MX>
+struct Slot {
+  static constexpr int S = MX + 4;
+  static constexpr int tile = 0;
+  static constexpr int nbr = tile + (int)sizeof(real) * S * S;
+  static constexpr int rows = nbr + 8 * (int)sizeof(NbrEntry);       // real2 (MX + 2 rows -1..MX)
+  static constexpr int rec = (rows + 2 * (int)sizeof(real) * (MX + 2) + 15) & ~15;
+  static constexpr int yl = rec + (int)sizeof(EdgeRec<real>) * (MX + 2);  // rows -1..MX at [r + 1]
+  static constexpr int ye = yl + (int)sizeof(real) * (MX + 2);       // P, M of columns -1, MX
+  static constexpr int end = ye + (int)sizeof(real) * 4 * (MX + 1);
+  // bytes, congruent to MX elements modulo 32 elements, a multiple of 16
+  static constexpr int row = 32 * (int)sizeof(real);
+  static constexpr int bytes = (end - MX * (int)sizeof(real) + row - 1) / row * row +
+                               MX * (int)sizeof(real);
+};
+
+// interior cell (i, j) of a patch of the interpolated level at weight alpha
+template <typename real, int MX>
+__device__ __forceinline__ real coarse_interior(const real* qo, const real* qn, real alpha, int i,
+                                                int j) {
+  const int o = (j + kMbc) * (MX + 4) + i + kMbc;
+  // (0: the newer state may still be written beside this kernel; 1: a step
+  // of all levels at one time has no older state)
+  if (alpha == real(0)) return qo[o];
+  if (alpha == real(1)) return qn[o];
+  return (real(1) - alpha) * qo[o] + alpha * qn[o];
 }
 
-template <int MX>
-constexpr int side_reals() {
-  return ((2 * (MX + 3) + 3 * (MX + 2) + 4 * (MX + 1)) + 3) & ~3;
+// A patch's ghost ring, by the MX lanes (li) of its segment, in two parts
+// with a warp barrier between them.  Sides and corners are told apart by
+// strides, not by code: the walk's instructions and these share a cache.
+//
+// Part 1: ghosts from same-size neighbours (every read issued before any is
+// stored), and into `cells` what the interpolations need beyond the coarse
+// patches' interiors: for each coarser face neighbour the coarse cell past
+// the end of the face at [side], for each coarser corner neighbour the five
+// cells of its stencil at [4 + 5 corner + m].  direct: a coarser neighbour on
+// tlevel is read as its fill would leave it (interpolate_direct_entry), else
+// from its filled tile.
+template <typename real, int MX>
+__device__ __forceinline__ void gather_part1(const DevForest<real>& D, const NbrEntry* E,
+                                             const PatchMeta& pm, int p, int tlevel, real alpha,
+                                             bool direct, bool mixed, real* T, real* cells,
+                                             int li) {
+  constexpr int S = MX + 4, SS = S * S;
+  constexpr int NC = (16 + MX - 1) / MX;  // corner ghosts a lane
+  real v0[4], v1[4], vc[NC];
+#pragma unroll
+  for (int f = 0; f < 4; ++f) {  // rows / columns mx - 2, mx - 1 or 0, 1 of the neighbour
+    const int sn = f < 2 ? 1 : S, st = f < 2 ? S : 1;
+    if (E[f].kind == NB_SAME) {
+      const real* src = D.buf[D.cur[E[f].lev]] + (size_t)E[f].n0 * SS + (li + kMbc) * st +
+                        ((f & 1) ? 2 : MX) * sn;
+      v0[f] = src[0];
+      v1[f] = src[sn];
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < NC; ++u) {
+    const int k = li + u * MX, r = 4 + (k >> 2);
+    if (k < 16 && E[r].kind == NB_SAME) {
+      const int i = ((r & 1) ? 0 : MX - 2) + (k & 1), j = ((r & 2) ? 0 : MX - 2) + ((k >> 1) & 1);
+      vc[u] = D.buf[D.cur[E[r].lev]][(size_t)E[r].n0 * SS + (j + kMbc) * S + i + kMbc];
+    }
+  }
+  if (mixed) {
+#pragma unroll 1
+    for (int k = li; k < 24; k += MX) {
+      const int r = k < 4 ? k : 4 + (k - 4) / 5;
+      const NbrEntry& e = E[r];
+      if (e.kind != NB_COARSE) continue;
+      // the first ghost of the region, its coarse cell, and the cell wanted
+      const int gi = (r == 1 || (r >= 4 && (r & 1))) ? MX : (r == 0 || r >= 4) ? -2 : 0;
+      const int gj = (r == 3 || (r >= 4 && (r & 2))) ? MX : (r == 2 || r >= 4) ? -2 : 0;
+      int ci = ((pm.x * MX + gi + e.fx) >> 1) - e.x0 * MX;
+      int cj = ((pm.y * MX + gj + e.fy) >> 1) - e.y0 * MX;
+      int ui = gi, uj = gj;  // the ghost group that reads the cell
+      if (k < 4) {  // the face's half of the coarse patch starts at 0 or ends at its side
+        int& c = r < 2 ? cj : ci;
+        int& u = r < 2 ? uj : ui;
+        if (c > 0) u = MX - 2;
+        c = c > 0 ? MX : -1;
+      } else {
+        const int m = (k - 4) % 5;
+        ci += m == 1 ? 1 : m == 2 ? -1 : 0;
+        cj += m == 3 ? 1 : m == 4 ? -1 : 0;
+      }
+      real v;
+      if (direct && e.lev == tlevel) {
+        const PatchMeta cm{e.lev, e.x0, e.y0, 0, 0, 0};
+        if (coarse_cell_interior<real, MX>(D, cm, ci, cj)) {
+          const int c = D.cur[tlevel];
+          v = coarse_interior<real, MX>(D.buf[c ^ 1] + (size_t)e.n0 * SS,
+                                        D.buf[c] + (size_t)e.n0 * SS, alpha, ci, cj);
+        } else {
+          v = coarse_ghost_at<real, MX>(D, e, cm, p, tlevel, alpha, ui, uj, ci, cj);
+        }
+      } else {
+        v = patch_ptr(e.lev == tlevel ? D.qT : D.buf[D.cur[e.lev]], e.n0,
+                      S)[(cj + kMbc) * S + ci + kMbc];
+      }
+      cells[k] = v;
+    }
+  }
+#pragma unroll
+  for (int f = 0; f < 4; ++f) {
+    const int sn = f < 2 ? 1 : S, st = f < 2 ? S : 1;
+    if (E[f].kind == NB_SAME) {
+      real* g = T + (li + kMbc) * st + ((f & 1) ? MX + 2 : 0) * sn;
+      g[0] = v0[f];
+      g[sn] = v1[f];
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < NC; ++u) {
+    const int k = li + u * MX, r = 4 + (k >> 2);
+    if (k < 16 && E[r].kind == NB_SAME) {
+      const int i = ((r & 1) ? MX : -2) + (k & 1), j = ((r & 2) ? MX : -2) + ((k >> 1) & 1);
+      T[(j + kMbc) * S + i + kMbc] = vc[u];
+    }
+  }
 }
 
-// NB tile buffers per warp: 2 overlap the next group's copy with this
-// group's compute; 1 halves the shared memory, so twice the warps fit on an
-// SM and other warps hide the copy instead
-template <typename real, int MX, int NB>
-constexpr int warp_reals() {
-  return NB * (32 / MX) * tile_stride<MX>() + (32 / MX) * side_reals<MX>();
+// Eq. ghost_fine for the four fine cells of a coarse cell: (dx, dy) = (-+1, -+1)
+template <typename real>
+__device__ __forceinline__ real fine_value(real q0, real sx, real sy, int x, int y) {
+  return q0 + real(0.25) * ((x ? sx : -sx) + (y ? sy : -sy));
 }
 
-template <typename real, int MX, int NW, bool SWIRL, int NB, bool FULL>
-__global__ void __launch_bounds__(NW * 32) advance_walk_kernel(DevForest<real> D, int p0, int p1,
-                                                               AdvArgs a, AdvConst<real> ac,
-                                                               int* err) {
-  constexpr int S = MX + 4;
-  constexpr int PPW = 32 / MX;
-  constexpr int TILE = S * S;
-  constexpr int TS = tile_stride<MX>();
-  constexpr int NS = MX + 3;
+// Part 2: ghosts from finer and coarser neighbours.
+template <typename real, int MX>
+__device__ __forceinline__ void gather_part2(const DevForest<real>& D, const NbrEntry* E,
+                                             const PatchMeta& pm, int p, int tlevel, real alpha,
+                                             bool direct, real* T, const real* cells, int li) {
+  constexpr int S = MX + 4, SS = S * S;
+#pragma unroll 1
+  for (int f = 0; f < 4; ++f) {
+    const NbrEntry& e = E[f];
+    const bool X = f < 2, low = (f & 1) == 0;
+    const int sn = X ? 1 : S, st = X ? S : 1;          // strides across and along the face
+    real* g = T + (low ? 0 : MX + 2) * sn + kMbc * st;  // its first ghost, outer or inner
+    if (e.kind == NB_FINE) {
+      // n0 holds the face's lower half, n1 the upper; lane li takes ghosts li;
+      // a ghost's four cells are summed in the order (0,0), (1,0), (0,1), (1,1)
+      const int half = li >= MX / 2 ? 1 : 0;
+      const real* c = D.buf[D.cur[e.lev]] + (size_t)(half ? e.n1 : e.n0) * SS +
+                      (2 * li - half * MX + kMbc) * st + (low ? MX - 2 : 2) * sn;
+      real w[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) w[k] = c[(k >> 2) * 2 * sn + (k & 1) + ((k >> 1) & 1) * S];
+      g[li * st] = real(0.25) * (((w[0] + w[1]) + w[2]) + w[3]);
+      g[li * st + sn] = real(0.25) * (((w[4] + w[5]) + w[6]) + w[7]);
+    } else if (e.kind == NB_COARSE && li < MX / 2) {
+      // the coarse cell beside rows / columns 2 li, 2 li + 1, the cells away
+      // from (in) and towards the owner (out), and along the face (lo, hi)
+      const int t0 = X ? ((pm.y * MX + e.fy) >> 1) - e.y0 * MX
+                       : ((pm.x * MX + e.fx) >> 1) - e.x0 * MX;
+      const int t = t0 + li;
+      const bool viaT = e.lev == tlevel;
+      const int o = (t + kMbc) * st + ((low ? MX - 1 : 0) + kMbc) * sn;
+      const int ol = t > 0 ? o - st : o, oh = t < MX - 1 ? o + st : o;  // (inside the patch)
+      const int d = low ? -sn : sn;
+      real q0, in, out, lo, hi;
+      if (direct && viaT) {
+        const int c = D.cur[tlevel];
+        const real* qo = D.buf[c ^ 1] + (size_t)e.n0 * SS;
+        const real* qn = D.buf[c] + (size_t)e.n0 * SS;
+        if (alpha == real(0) || alpha == real(1)) {  // (see coarse_interior)
+          const real* q = alpha == real(0) ? qo : qn;
+          q0 = q[o];
+          in = q[o + d];
+          lo = q[ol];
+          hi = q[oh];
+        } else {
+          const real b = real(1) - alpha;
+          q0 = b * qo[o] + alpha * qn[o];
+          in = b * qo[o + d] + alpha * qn[o + d];
+          lo = b * qo[ol] + alpha * qn[ol];
+          hi = b * qo[oh] + alpha * qn[oh];
+        }
+        if (e.code[0] & kSrcComplete) {  // towards the owner: the average of its own cells
+          const real* w = T + (2 * li + kMbc) * st + (low ? kMbc : MX) * sn;
+          const int a = X ? sn : st, b2 = X ? st : sn;
+          out = real(0.25) * (((w[0] + w[a]) + w[b2]) + w[a + b2]);
+        } else {
+          const PatchMeta cm{e.lev, e.x0, e.y0, 0, 0, 0};
+          const int n = low ? MX : -1;
+          out = coarse_ghost<real, MX>(D, cm, e.n0, tlevel, alpha, X ? n : t, X ? t : n);
+        }
+      } else {
+        const real* q = patch_ptr(viaT ? D.qT : D.buf[D.cur[e.lev]], e.n0, S);
+        q0 = q[o];
+        in = q[o + d];
+        out = q[o - d];
+        lo = q[ol];
+        hi = q[oh];
+      }
+      if (t == 0) lo = cells[f];
+      if (t == MX - 1) hi = cells[f];
+      // slopes towards higher index, across the face and along it
+      const real sc = low ? minmod(out - q0, q0 - in) : minmod(in - q0, q0 - out);
+      const real sl = minmod(hi - q0, q0 - lo);
+      const real sx = X ? sc : sl, sy = X ? sl : sc;
+      real* w = g + 2 * li * st;
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        w[(k & 1) + (k >> 1) * S] = fine_value(q0, sx, sy, k & 1, k >> 1);
+    }
+  }
+#pragma unroll 1
+  for (int k = li; k < 16; k += MX) {  // the corners
+    const int r = 4 + (k >> 2), x = k & 1, y = (k >> 1) & 1;
+    const NbrEntry& e = E[r];
+    real v;
+    if (e.kind == NB_FINE) {
+      const real* w = D.buf[D.cur[e.lev]] + (size_t)e.n0 * SS +
+                      (((r & 2) ? 0 : MX - 4) + 2 * y + kMbc) * S + ((r & 1) ? 0 : MX - 4) + 2 * x +
+                      kMbc;
+      v = real(0.25) * (((w[0] + w[1]) + w[S]) + w[S + 1]);
+    } else if (e.kind == NB_COARSE) {
+      const real* c = cells + 4 + 5 * (r - 4);
+      const real sx = minmod(c[1] - c[0], c[0] - c[2]), sy = minmod(c[3] - c[0], c[0] - c[4]);
+      v = fine_value(c[0], sx, sy, x, y);
+    } else {
+      continue;
+    }
+    T[(((r & 2) ? MX : -2) + y + kMbc) * S + ((r & 1) ? MX : -2) + x + kMbc] = v;
+  }
+}
+
+template <typename real, int MX>
+struct WalkShape {
+  static constexpr int PK = Packed<real>::N;        // cells a lane works on at once
+  static constexpr bool SPLIT = PK == 2 && MX == 32;  // of one patch (two halves of its rows)
+  static constexpr int NPS = SPLIT ? 1 : PK;        // patches of a segment of MX lanes
+  static constexpr int PPW = (32 / MX) * NPS;       // patches of a warp
+  static constexpr int R = SPLIT ? MX / 2 : MX;     // rows a lane walks
+};
+
+// CTAs an SM is to hold of 8 warps each: FP32 24 warps of at most 80
+// registers, FP64 16 of 128 (its pipe, not latency, bounds it)
+template <typename real, int MX, bool SWIRL, bool FULL>
+__global__ void __launch_bounds__(256, sizeof(real) == 4 ? 3 : 2)
+    advance_walk_kernel(const __grid_constant__ DevForest<real> D, int p0, int p1,
+                        const __grid_constant__ AdvArgs a, AdvConst<real> ac, int* err) {
+  using W = WalkShape<real, MX>;
+  using PV = Packed<real>;
+  using V = typename PV::V;
+  using SL = Slot<real, MX>;
+  constexpr int S = MX + 4, TILE = S * S, PPW = W::PPW, NSEG = 32 / MX;
   constexpr unsigned kAll = 0xffffffffu;
+  constexpr uint32_t tbytes = sizeof(real) * TILE, nbytes = 8 * sizeof(NbrEntry);
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  __shared__ __align__(8) uint64_t bars[NW][2];
+  __shared__ __align__(8) uint64_t bars[8];
   __shared__ real ucoef_s;
-  __shared__ NbrStage nst[NW][PPW];
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, NW = blockDim.x >> 5;
   const int seg = lane / MX, li = lane % MX;
-  real* wbase = reinterpret_cast<real*>(smem_raw) + (size_t)warp * warp_reals<real, MX, NB>();
-  real* side = wbase + NB * PPW * TS + seg * side_reals<MX>();
-  real* TyS = side;           // sin(pi (y_r + y_{r+1})), r = -1..MX+1 at [r+1]
-  real* SyS = TyS + NS;       // sin^2(pi y_r), r = -1..MX+1 at [r+1]
-  real* FeN = SyS + NS;       // x-edge MX: normal flux, rows -1..MX at [r+1]
-  real* FeU = FeN + (MX + 2);  //            speed
-  real* XMe = FeU + (MX + 2);  //            fluctuation into cell MX-1
-  real* YPm = XMe + (MX + 2);  // y-edges of column -1, rows 0..MX
-  real* YMm = YPm + (MX + 1);
-  real* YPp = YMm + (MX + 1);  // y-edges of column MX, rows 0..MX
-  real* YMp = YPp + (MX + 1);
+  unsigned char* wbase = smem_raw + (size_t)warp * PPW * SL::bytes;
+  auto slot = [&](int s) { return wbase + s * SL::bytes; };
 
   if (threadIdx.x == 0 && SWIRL) {
     const double t = a.t0_dev ? *a.t0_dev + a.t_off : a.t_half;
     ucoef_s = cospi_ratio<real>(t, a.period) * real(a.sfac * 0.5 * a.nu);
   }
-  if (lane == 0) {
-    mbar_init(&bars[warp][0], 1);
-    mbar_init(&bars[warp][1], 1);
-  }
+  if (lane == 0) mbar_init(&bars[warp], 1);
   __syncthreads();
 
   const real ucoef = SWIRL ? ucoef_s : real(0);
-  const real cu = ac.cu, cv = ac.cv, h = ac.h;
   const Scheme<real, FULL> sc = make_scheme<real, FULL>(D.order, D.limiter, D.transverse);
+  const real h = ac.h;
+  const real* tab = static_cast<const real*>(a.trig);
+  auto sin2 = [&](int z) -> real {  // sin^2(pi x) at node z
+    if (tab) return tab[z + 1];
+    const real s = sinpi_r(real(z) * h);
+    return s * s;
+  };
+  auto sin1 = [&](int z) -> real {  // sin(pi (x_z + x_{z+1}))
+    return tab ? tab[a.trig_len + z + 1] : sinpi_r(real(2 * z + 1) * h);
+  };
 
   const int ngroups = (p1 - p0 + PPW - 1) / PPW;
   const int TW = gridDim.x * NW;
-  auto tile = [&](int b, int s) { return wbase + (b * PPW + s) * TS; };
-  auto issue = [&](int g, int b) {  // lane 0: TMA loads of group g into buffer b
-    const int nvalid = min(PPW, p1 - p0 - g * PPW);
-    fence_proxy_async();
-    mbar_expect_tx(&bars[warp][b], (uint32_t)(nvalid * TILE * sizeof(real)));
-    for (int s = 0; s < nvalid; ++s) {
-      const int p = p0 + g * PPW + s;
-      const real* src = D.buf[D.cur[D.meta[p].level]] + (size_t)p * TILE;
-      bulk_load(tile(b, s), src, (uint32_t)(TILE * sizeof(real)), &bars[warp][b]);
+  uint32_t par = 0;
+  for (int g = blockIdx.x * NW + warp; g < ngroups; g += TW) {
+    const int pg = p0 + g * PPW, nvalid = min(PPW, p1 - pg);
+    if (lane == 0) {
+      fence_proxy_async();
+      mbar_expect_tx(&bars[warp], nvalid * (tbytes + (a.gather ? nbytes : 0)));
+      for (int s = 0; s < nvalid; ++s) {
+        const int p = pg + s;
+        bulk_load(slot(s) + SL::tile, D.buf[D.cur[a.level]] + (size_t)p * TILE, tbytes, &bars[warp]);
+        if (a.gather) bulk_load(slot(s) + SL::nbr, D.nbr + (size_t)p * 8, nbytes, &bars[warp]);
+      }
     }
-  };
-
-  uint32_t par0 = 0, par1 = 0;
-  int b = 0;
-  const int g_first = blockIdx.x * NW + warp;
-  int g = g_first;
-  if (g < ngroups && lane == 0) issue(g, 0);
-  for (; g < ngroups; g += TW, b ^= (NB - 1)) {
-    const bool prefetch = NB == 2 && g + TW < ngroups;
-    // one buffer: the group's copy starts once the warp left the previous one
-    if (NB == 1 && g != g_first && lane == 0) issue(g, 0);
-    if (prefetch && lane == 0) issue(g + TW, b ^ 1);
-    const int p = p0 + g * PPW + seg;
-    const bool valid = p < p1;
-    const int pc = valid ? p : p0 + g * PPW;
-    const PatchMeta pm = D.meta[pc];
-    real* dst = D.buf[D.cur[pm.level] ^ 1] + (size_t)pc * TILE;
-    const int x0 = pm.x * MX, y0 = pm.y * MX;
-    // column factors of this lane's edges (streamfunction tables)
-    real Sx_i = 0, Tx_i = 0, SxE = 0, TxM = 0, TxP = 0;
-    if (SWIRL) {
-      real s = sinpi_r(real(x0 + li) * h);
-      Sx_i = s * s;
-      Tx_i = sinpi_r(real(2 * (x0 + li) + 1) * h);
-      s = sinpi_r(real(x0 + MX) * h);
-      SxE = s * s;
-      TxM = sinpi_r(real(2 * (x0 - 1) + 1) * h);
-      TxP = sinpi_r(real(2 * (x0 + MX) + 1) * h);
+    // this lane's patches (beyond the range: the group's first, not stored)
+    int pk[W::NPS];
+    bool ok[W::NPS];
+    real ux[W::NPS], vy[W::NPS];          // factors of the lane's x- and y-edges
+    real uxE[W::NPS], vyM[W::NPS], vyP[W::NPS];  // of x-edge MX and of columns -1, MX
+#pragma unroll
+    for (int k = 0; k < W::NPS; ++k) {
+      const int s = k * NSEG + seg;
+      ok[k] = s < nvalid;
+      pk[k] = ok[k] ? pg + s : pg;
+      ux[k] = vy[k] = uxE[k] = vyM[k] = vyP[k] = real(0);
+      if (SWIRL) {
+        const PatchMeta pm = D.meta[pk[k]];
+        const int x0 = pm.x * MX, y0 = pm.y * MX;
+        ux[k] = ucoef * sin2(x0 + li);
+        vy[k] = -ucoef * sin1(x0 + li);
+        uxE[k] = ucoef * sin2(x0 + MX);
+        vyM[k] = -ucoef * sin1(x0 - 1);
+        vyP[k] = -ucoef * sin1(x0 + MX);
+        // row r: factor of its x-edges, and of the y-edges above it
+        real* rw = reinterpret_cast<real*>(slot(ok[k] ? s : 0) + SL::rows);
+        if (ok[k])
+          for (int r = li - 1; r <= MX; r += MX) {
+            rw[2 * (r + 1)] = sin1(y0 + r);
+            rw[2 * (r + 1) + 1] = sin2(y0 + r + 1);
+          }
+      }
     }
-    uint32_t& par = b ? par1 : par0;
-    const bool ok = mbar_wait(&bars[warp][b], par, a.wait_limit);
-    if (!__all_sync(kAll, ok)) {
+    const bool landed = mbar_wait(&bars[warp], par, a.wait_limit);
+    if (!__all_sync(kAll, landed)) {
       if (lane == 0) atomicOr(err, kErrTimeout);
-      // let every copy in flight land before leaving
-      mbar_wait(&bars[warp][b], par, kWaitLimit);
-      if (prefetch) mbar_wait(&bars[warp][b ^ 1], b ? par0 : par1, kWaitLimit);
+      mbar_wait(&bars[warp], par, kWaitLimit);  // let the copies in flight land before leaving
       return;
     }
     par ^= 1;
-    real* T = tile(b, seg);
-    if (a.gather) {  // Alg. 1 for this segment's patch, into the tile's ghost ring
-      stage_neighbours(D.meta, D.nbr, pc, nst[warp][seg], li);
-      __syncwarp();
-      // every ghost by its own rule in one pass (the phases of Alg. 1 write
-      // different ghosts, and an interpolation reads the coarse patch, not
-      // this tile), then the wall condition once: the bits of the phased fill
-      const NbrStage& ns = nst[warp][seg];
-      for (int k = li; k < num_ghosts<MX>(); k += MX) {
-        int i, j;
-        ghost_ij<MX>(k, i, j);
-        const NbrEntry& e = ns.e[region_of<MX>(i, j)];
-        real v;
-        if (copy_or_average_entry<real, MX>(D, e, pm, a.tlevel, ac.alpha, i, j, v) ||
-            interpolate_entry<real, MX>(D, e, pm, a.tlevel, i, j, v))
-          T[(j + kMbc) * S + i + kMbc] = v;
+    if (a.gather) {  // Alg. 1 for the warp's patches, into their tiles' ghost rings
+      bool mixed = false, wall = false;
+#pragma unroll
+      for (int k = 0; k < W::NPS; ++k) {
+        const int s = k * NSEG + seg;
+        if (s < nvalid)
+          for (int r = li; r < 8; r += MX) {
+            const int kind = reinterpret_cast<const NbrEntry*>(slot(s) + SL::nbr)[r].kind;
+            mixed |= kind == NB_FINE || kind == NB_COARSE;
+            wall |= kind == NB_EXTERIOR;
+          }
+      }
+      mixed = __any_sync(kAll, mixed);
+      wall = __any_sync(kAll, wall);
+#pragma unroll 1
+      for (int k = 0; k < W::NPS; ++k) {
+        const int s = k * NSEG + seg;
+        if (s < nvalid)
+          gather_part1<real, MX>(D, reinterpret_cast<const NbrEntry*>(slot(s) + SL::nbr),
+                                 D.meta[pg + s], pg + s, a.tlevel, ac.alpha, a.direct != 0, mixed,
+                                 reinterpret_cast<real*>(slot(s) + SL::tile),
+                                 reinterpret_cast<real*>(slot(s) + SL::ye), li);
       }
       __syncwarp();
-      if (D.domain == FC_DOMAIN_WALLS) {
-        wall_bc<real, MX>(pm, T, li, MX);
+      if (mixed) {
+#pragma unroll 1
+        for (int k = 0; k < W::NPS; ++k) {
+          const int s = k * NSEG + seg;
+          if (s < nvalid)
+            gather_part2<real, MX>(D, reinterpret_cast<const NbrEntry*>(slot(s) + SL::nbr),
+                                   D.meta[pg + s], pg + s, a.tlevel, ac.alpha, a.direct != 0,
+                                   reinterpret_cast<real*>(slot(s) + SL::tile),
+                                   reinterpret_cast<const real*>(slot(s) + SL::ye), li);
+        }
         __syncwarp();
       }
+      if (wall && D.domain == FC_DOMAIN_WALLS) {
+#pragma unroll 1
+        for (int k = 0; k < W::NPS; ++k) {
+          const int s = k * NSEG + seg;
+          if (s < nvalid)
+            wall_bc<real, MX>(D.meta[pg + s], reinterpret_cast<real*>(slot(s) + SL::tile), li, MX);
+        }
+        __syncwarp();
+      }
+    } else {
+      __syncwarp();  // the rows' factors
     }
-    if (a.keep && valid) {  // the adjoint's replay keeps the ghost-filled input tile
-      real* kp = static_cast<real*>(a.keep) + (size_t)(p - a.keep_p0) * TILE;
-      for (int k = li; k < TILE; k += MX) kp[k] = T[k];
-    }
-    auto Q = [&](int i, int j) -> real { return T[(j + 2) * S + (i + 2)]; };
+    if (a.keep)  // the adjoint's replay keeps the ghost-filled input tile
+      for (int k = 0; k < W::NPS; ++k) {
+        const int s = k * NSEG + seg;
+        if (s >= nvalid) continue;
+        const real* T = reinterpret_cast<const real*>(slot(s) + SL::tile);
+        real* kp = static_cast<real*>(a.keep) + (size_t)(pg + s - a.keep_p0) * TILE;
+        for (int c = li; c < TILE; c += MX) kp[c] = T[c];
+      }
+    // packed views: component k of a lane reads slot sk at row offset rk
+    const unsigned char* b0 = slot(ok[0] ? seg : 0);
+    const unsigned char* b1 =
+        W::SPLIT ? b0 : W::NPS == 2 ? slot(ok[W::NPS - 1] ? NSEG + seg : 0) : b0;
+    const real* T0 = reinterpret_cast<const real*>(b0 + SL::tile);
+    const real* T1 = reinterpret_cast<const real*>(b1 + SL::tile);
+    constexpr int r1 = W::SPLIT ? W::R : 0;  // row offset of component 1
+    constexpr int kl = W::NPS - 1;           // patch of component 1
 
-    // side pass: lanes own rows r = -1..MX+1
-    for (int r = li - 1; r <= MX + 1; r += MX) {
-      const real ty = SWIRL ? sinpi_r(real(2 * (y0 + r) + 1) * h) : real(0);
-      real sy = SWIRL ? sinpi_r(real(y0 + r) * h) : real(0);
-      sy *= sy;
-      TyS[r + 1] = ty;
-      SyS[r + 1] = sy;
-      real Fn, P, M;
-      if (r <= MX) {  // x-edge MX of row r
-        const real c = SWIRL ? (ucoef * SxE) * ty : cu;
-        edge(c, Q(MX - 2, r), Q(MX - 1, r), Q(MX, r), Q(MX + 1, r), corr_factor(c, sc), sc, Fn, P,
-             M);
-        FeN[r + 1] = Fn;
-        FeU[r + 1] = c;
-        XMe[r + 1] = M;
+    // the edges beside the lanes: x-edge MX of rows -1..MX, y-edges of ghost
+    // columns -1 and MX at rows 0..MX, one (packed: two) a lane and round; in
+    // the split form a lane takes edges t and t + NT, else edge t of both patches
+    {
+      constexpr int NTASK = 3 * MX + 4;
+      constexpr int NT = W::SPLIT ? (NTASK + 1) / 2 : NTASK;
+      for (int t = li; t < NT; t += MX) {
+        V c, qa, qb, qc, qd;
+        const int ts[2] = {t, W::SPLIT ? t + NT : t};
+        real cc[2], v[2][4];
+#pragma unroll
+        for (int k = 0; k < PV::N; ++k) {
+          const int q = min(ts[k], NTASK - 1);
+          const bool x = q < MX + 2;
+          const bool right = q >= 2 * MX + 3;
+          const int r = x ? q - 1 : q - (right ? 2 * MX + 3 : MX + 2);
+          const real* T = k ? T1 : T0;
+          const real* rw = reinterpret_cast<const real*>((k ? b1 : b0) + SL::rows);
+          const real* o = T + (r + kMbc) * S + ((x || right) ? MX : -1) + kMbc;
+          const int st = x ? 1 : S;
+          const int w = k ? kl : 0;
+          // (y-edge row r takes the factor stored with row r - 1)
+          cc[k] = SWIRL ? (x ? uxE[w] * rw[2 * (r + 1)]
+                             : (right ? vyP[w] : vyM[w]) * rw[2 * r + 1])
+                        : (x ? ac.cu : ac.cv);
+          v[k][0] = o[-2 * st];
+          v[k][1] = o[-st];
+          v[k][2] = o[0];
+          v[k][3] = o[st];
+        }
+        constexpr int z = PV::N - 1;
+        c = PV::make(cc[0], cc[z]);
+        qa = PV::make(v[0][0], v[z][0]);
+        qb = PV::make(v[0][1], v[z][1]);
+        qc = PV::make(v[0][2], v[z][2]);
+        qd = PV::make(v[0][3], v[z][3]);
+        V F, nP, M;
+        const Speed<V> sp(c);
+        vedge(sp, vsub(qc, qb), vupwind(c, qa, qb, qc, qd), qb, qc, sc, F, nP, M);
+#pragma unroll
+        for (int k = 0; k < PV::N; ++k) {
+          const int q = ts[k];
+          if (q >= NTASK || !ok[W::SPLIT ? 0 : k]) continue;
+          unsigned char* b = const_cast<unsigned char*>(k ? b1 : b0);
+          if (q < MX + 2) {
+            EdgeRec<real>* e = reinterpret_cast<EdgeRec<real>*>(b + SL::rec) + q;
+            e->M = PV::get(M, k);
+            e->F = PV::get(F, k);
+            e->c = PV::get(c, k);
+          } else {
+            const bool right = q >= 2 * MX + 3;
+            const int r = q - (right ? 2 * MX + 3 : MX + 2);
+            real* y = reinterpret_cast<real*>(b + SL::ye) + (right ? 2 * (MX + 1) : 0);
+            y[r] = PV::get(nP, k);
+            y[MX + 1 + r] = PV::get(M, k);
+          }
+        }
       }
-      if (r >= 0 && r <= MX) {  // y-edges of ghost columns -1 and MX at row r
-        const real cl = SWIRL ? (-ucoef * TxM) * sy : cv;
-        edge(cl, Q(-1, r - 2), Q(-1, r - 1), Q(-1, r), Q(-1, r + 1), corr_factor(cl, sc), sc, Fn,
-             P, M);
-        YPm[r] = P;
-        YMm[r] = M;
-        const real cr = SWIRL ? (-ucoef * TxP) * sy : cv;
-        edge(cr, Q(MX, r - 2), Q(MX, r - 1), Q(MX, r), Q(MX, r + 1), corr_factor(cr, sc), sc, Fn,
-             P, M);
-        YPp[r] = P;
-        YMp[r] = M;
+      __syncwarp();
+#pragma unroll
+      for (int k = 0; k < W::NPS; ++k) {
+        if (!ok[k]) continue;
+        unsigned char* b = const_cast<unsigned char*>(k ? b1 : b0);
+        const real* y = reinterpret_cast<const real*>(b + SL::ye);
+        reinterpret_cast<real*>(b + SL::yl)[li + 1] = y[li] - y[MX + 1 + li + 1];
+        reinterpret_cast<EdgeRec<real>*>(b + SL::rec)[li + 1].nY =
+            y[2 * (MX + 1) + li] - y[3 * (MX + 1) + li + 1];
       }
+      __syncwarp();
     }
-    __syncwarp();
 
-    // main walk: lane li owns column li; iteration r computes x-edge (li, r)
-    // and y-edge (li, r+1), finishes the fluxes of row r and updates row r-1
-    const real ux = ucoef * Sx_i, vy = -ucoef * Tx_i;
-    real qa = Q(li, -2), qb = Q(li, -1), qc = Q(li, 0), qd = 0;
-    real Wa = qb - qa, Wb = qc - qb;  // jumps of y-edges (li, r), (li, r + 1)
-    real X_prev = 0, Gn_cur = 0, v_cur = 0, YP_cur = 0, Gf_prev = 0, dF_prev = 0;
-#pragma unroll 2  // fully unrolled, the row walk overflowed the instruction cache
-    for (int r = -1; r <= MX; ++r) {
-      if (r + 2 <= MX + 1) qd = Q(li, r + 2);
-      const real Wc = qd - qc;  // jump of y-edge (li, r + 2)
-      // x-edge (li, r): cells (li-1, r) | (li, r)
-      const real cx = SWIRL ? ux * TyS[r + 1] : cu;
-      real Fn_r, XP_r, XM_r;
-      edge(cx, Q(li - 2, r), Q(li - 1, r), qb, Q(li + 1, r), corr_factor(cx, sc), sc, Fn_r, XP_r,
-           XM_r);
-      real XMn = __shfl_down_sync(kAll, XM_r, 1, MX);
-      if (li == MX - 1) XMn = XMe[r + 1];
-      const real X_r = XP_r + XMn;  // x-fluctuation into cell (li, r)
-      // y-edge (li, r+1): cells (li, r) | (li, r+1)
-      real Gn_n = 0, YP_n = 0, YM_n = 0, v_n = 0;
-      if (r + 1 <= MX) {
-        v_n = SWIRL ? vy * SyS[r + 2] : cv;
-        edge_flux(v_n, Wb, upwind_left(v_n) ? Wa : Wc, qb, qc, corr_factor(v_n, sc), sc, Gn_n,
-                  YP_n, YM_n);
+    // the walk: iteration it works on row r = it - 1 (of each component's
+    // rows): x-edge (li, r), y-edge (li, r + 1), the final fluxes of row r
+    // and the update of row r - 1.  Rows outside the patch's are computed
+    // from whatever shared memory holds there and used by no stored cell.
+    auto col = [&](int i, int r) -> V {  // cell (li + i, r) of each component
+      const int o = (r + kMbc) * S + li + i + kMbc;
+      return PV::make(T0[o], T1[o + r1 * S]);
+    };
+    const V uxv = PV::make(ux[0], ux[kl]), vyv = PV::make(vy[0], vy[kl]);
+    const real* rw0 = reinterpret_cast<const real*>(b0 + SL::rows);
+    const real* rw1 = reinterpret_cast<const real*>(b1 + SL::rows) + 2 * r1;
+    const EdgeRec<real>* ec0 = reinterpret_cast<const EdgeRec<real>*>(b0 + SL::rec);
+    const EdgeRec<real>* ec1 = reinterpret_cast<const EdgeRec<real>*>(b1 + SL::rec) + r1;
+    const real* yl0 = reinterpret_cast<const real*>(b0 + SL::yl);
+    const real* yl1 = reinterpret_cast<const real*>(b1 + SL::yl) + r1;
+    real* dst = D.buf[D.cur[a.level] ^ 1];
+    real* dst0 = dst + (size_t)pk[0] * TILE + li + kMbc;
+    real* dst1 = dst + (size_t)pk[kl] * TILE + r1 * S + li + kMbc;
+    const bool okl = ok[kl];
+    auto up = [&](V v) -> V {  // of the lane to the left
+      return PV::make(__shfl_up_sync(kAll, PV::get(v, 0), 1, MX),
+                      PV::N == 2 ? __shfl_up_sync(kAll, PV::get(v, 1), 1, MX) : real(0));
+    };
+    auto down = [&](V v) -> V {
+      return PV::make(__shfl_down_sync(kAll, PV::get(v, 0), 1, MX),
+                      PV::N == 2 ? __shfl_down_sync(kAll, PV::get(v, 1), 1, MX) : real(0));
+    };
+    const bool first = li == 0, last = li == MX - 1;
+    V qa = col(0, -2), qb = col(0, -1), qc = col(0, 0);
+    V Wa = vsub(qb, qa), Wb = vsub(qc, qb);
+    const V zero = PV::all(real(0));
+    V nX_prev = zero, G_cur = zero, nP_cur = zero, Gf_prev = zero, dF_prev = zero;
+    Speed<V> v_cur(zero);
+#pragma unroll 2
+    for (int it = 0; it < W::R + 2; ++it) {
+      const int r = it - 1;
+      const V qd = col(0, r + 2);
+      const V Wc = vsub(qd, qc);
+      V fx, fy;  // speeds of x-edge (li, r) and y-edge (li, r + 1)
+      if (SWIRL) {
+        using V2 = typename Vec2<real>::T;
+        const V2 f0 = reinterpret_cast<const V2*>(rw0)[it], f1 = reinterpret_cast<const V2*>(rw1)[it];
+        fx = vmul(uxv, PV::make(f0.x, f1.x));
+        fy = vmul(vyv, PV::make(f0.y, f1.y));
+      } else {
+        fx = PV::all(ac.cu);
+        fy = PV::all(ac.cv);
       }
-      // final flux at y-edge (li, r)
-      real Gf_r = 0;
-      if (r >= 0) Gf_r = final_flux(v_cur, X_prev, X_r, Gn_cur, sc);
-      // final fluxes at x-edges (li, r) and (li+1, r)
-      real dF_r = 0;
-      if (r >= 0 && r < MX) {
-        const real Y_r = YP_cur + YM_n;  // y-fluctuation into cell (li, r)
-        real Yl = __shfl_up_sync(kAll, Y_r, 1, MX);
-        if (li == 0) Yl = YPm[r] + YMm[r + 1];
-        const real Ff = final_flux(cx, Yl, Y_r, Fn_r, sc);
-        real Fr = __shfl_down_sync(kAll, Ff, 1, MX);
-        if (li == MX - 1)
-          Fr = final_flux(FeU[r + 1], Y_r, YPp[r] + YMp[r + 1], FeN[r + 1], sc);
-        dF_r = Fr - Ff;
+      const Speed<V> sx(fx), sy(fy);
+      V F, nP, M;
+      {
+        const V ql = col(-1, r);
+        vedge(sx, vsub(qb, ql), vupwind(fx, col(-2, r), ql, qb, col(1, r)), ql, qb, sc, F, nP, M);
       }
-      // conservative update of cell (li, r-1)
-      if (r >= 1 && valid)
-        dst[(r + 1) * S + (li + 2)] = fma(real(-2), dF_prev + (Gf_r - Gf_prev), qa);
-      X_prev = X_r;
-      Gn_cur = Gn_n;
-      v_cur = v_n;
-      YP_cur = YP_n;
-      Gf_prev = Gf_r;
-      dF_prev = dF_r;
+      V Mr = down(M);
+      EdgeRec<real> e0, e1;
+      if (last) {
+        e0 = ec0[it];
+        e1 = ec1[it];
+        Mr = PV::make(e0.M, e1.M);
+      }
+      const V nX = vsub(nP, Mr);  // turned x-fluctuation sum of cell (li, r)
+      V Gn, nPn, Mn;
+      vedge(sy, Wb, vselect(fy, Wa, Wc), qb, qc, sc, Gn, nPn, Mn);
+      // final flux of y-edge (li, r)
+      const V Gf = vfinal(v_cur, nX_prev, nX, G_cur, sc);
+      // final fluxes of x-edges (li, r) and (li + 1, r)
+      const V nY = vsub(nP_cur, Mn);  // turned y-fluctuation sum of cell (li, r)
+      V nYl = up(nY);
+      if (first) nYl = PV::make(yl0[it], yl1[it]);
+      const V Ff = vfinal(sx, nYl, nY, F, sc);
+      V Fr = down(Ff);
+      if (last) {
+        const V ce = PV::make(e0.c, e1.c);
+        Fr = vfinal(Speed<V>(ce), nY, PV::make(e0.nY, e1.nY), PV::make(e0.F, e1.F), sc);
+      }
+      const V dF = vsub(Fr, Ff);
+      if (it >= 2) {  // the update of cell (li, r - 1)
+        const V n = vfma(PV::all(real(-2)), vadd(dF_prev, vsub(Gf, Gf_prev)), qa);
+        if (ok[0]) dst0[(r + 1) * S] = PV::get(n, 0);
+        if (PV::N == 2 && okl) dst1[(r + 1) * S] = PV::get(n, PV::N - 1);
+      }
+      nX_prev = nX;
+      G_cur = Gn;
+      v_cur = sy;
+      nP_cur = nPn;
+      Gf_prev = Gf;
+      dF_prev = dF;
       qa = qb;
       qb = qc;
       qc = qd;
       Wa = Wb;
       Wb = Wc;
     }
-    __syncwarp();
+    __syncwarp();  // the next group's copies overwrite the slots
   }
 }
 
-template <typename real, int MX, int NW, bool SWIRL, int NB, bool FULL>
+template <typename real, int MX, bool SWIRL, bool FULL>
 cudaError_t walk_launch(const DevForest<real>& D, int p0, int p1, const AdvArgs& a, int* err,
                         cudaStream_t s) {
-  // computed once per process; concurrent first calls compute the same value
-  static std::atomic<int> max_ctas_once{0};
-  int max_ctas = max_ctas_once.load(std::memory_order_acquire);
-  constexpr size_t smem = sizeof(real) * (size_t)NW * warp_reals<real, MX, NB>();
-  auto kern = advance_walk_kernel<real, MX, NW, SWIRL, NB, FULL>;
-  if (max_ctas == 0) {
-    cudaError_t e =
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  using W = WalkShape<real, MX>;
+  auto kern = advance_walk_kernel<real, MX, SWIRL, FULL>;
+  // warps of a CTA: those asked for, at most what shared memory holds
+  constexpr size_t per_warp = (size_t)W::PPW * Slot<real, MX>::bytes;
+  constexpr int most = (int)(227 * 1024 / per_warp) < 8 ? (int)(227 * 1024 / per_warp) : 8;
+  const int nw = a.warps < most ? a.warps : most;
+  const size_t smem = nw * per_warp;
+  // set once per process; concurrent first calls set the same
+  static std::atomic<int> max_ctas[9];
+  int cap = max_ctas[nw].load(std::memory_order_acquire);
+  if (cap == 0) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)(most * per_warp));
     if (e != cudaSuccess) return e;
     int dev = 0, nsm = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NW * 32, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, nw * 32, smem);
     if (e != cudaSuccess) return e;
-    max_ctas = nsm * (per_sm > 0 ? per_sm : 1);
-    max_ctas_once.store(max_ctas, std::memory_order_release);
+    cap = nsm * (per_sm > 0 ? per_sm : 1);
+    max_ctas[nw].store(cap, std::memory_order_release);
   }
-  constexpr int PPW = 32 / MX;
-  const int groups = (p1 - p0 + PPW - 1) / PPW;
-  int ctas = (groups + NW - 1) / NW;
-  const int cap = a.ctas > 0 ? a.ctas : max_ctas;
+  const int groups = (p1 - p0 + W::PPW - 1) / W::PPW;
+  int ctas = (groups + nw - 1) / nw;
+  if (a.ctas > 0) cap = a.ctas;
   if (ctas > cap) ctas = cap;
-  kern<<<ctas, NW * 32, smem, s>>>(D, p0, p1, a, adv_const(D, a), err);
+  kern<<<ctas, nw * 32, smem, s>>>(D, p0, p1, a, adv_const(D, a), err);
   ++launch_counter();
   return cudaGetLastError();
 }
 
-template <typename real, int MX, int NW, bool FULL>
-cudaError_t walk_vel(const DevForest<real>& D, int p0, int p1, const AdvArgs& a, int* err,
-                     cudaStream_t s) {
-  const bool one = a.variant == ADV_WALK1;
-  if (D.vel_kind == FC_VEL_SWIRL)
-    return one ? walk_launch<real, MX, NW, true, 1, FULL>(D, p0, p1, a, err, s)
-               : walk_launch<real, MX, NW, true, 2, FULL>(D, p0, p1, a, err, s);
-  return one ? walk_launch<real, MX, NW, false, 1, FULL>(D, p0, p1, a, err, s)
-             : walk_launch<real, MX, NW, false, 2, FULL>(D, p0, p1, a, err, s);
-}
-
-template <typename real, int MX, int NW>
+template <typename real, int MX>
 cudaError_t walk_opt(const DevForest<real>& D, int p0, int p1, const AdvArgs& a, int* err,
                      cudaStream_t s) {
-  return full_scheme(D.order, D.limiter, D.transverse)
-             ? walk_vel<real, MX, NW, true>(D, p0, p1, a, err, s)
-             : walk_vel<real, MX, NW, false>(D, p0, p1, a, err, s);
-}
-
-template <typename real, int MX>
-cudaError_t walk_nw(const DevForest<real>& D, int p0, int p1, const AdvArgs& a, int* err,
-                    cudaStream_t s) {
-  switch (a.warps) {
-    case 2: return walk_opt<real, MX, 2>(D, p0, p1, a, err, s);
-    case 8: return walk_opt<real, MX, 8>(D, p0, p1, a, err, s);
-    default: return walk_opt<real, MX, 4>(D, p0, p1, a, err, s);
-  }
+  const bool full = full_scheme(D.order, D.limiter, D.transverse);
+  if (D.vel_kind == FC_VEL_SWIRL)
+    return full ? walk_launch<real, MX, true, true>(D, p0, p1, a, err, s)
+                : walk_launch<real, MX, true, false>(D, p0, p1, a, err, s);
+  return full ? walk_launch<real, MX, false, true>(D, p0, p1, a, err, s)
+              : walk_launch<real, MX, false, false>(D, p0, p1, a, err, s);
 }
 
 }  // namespace
@@ -323,9 +677,9 @@ template <typename real>
 cudaError_t launch_advance_walk(const DevForest<real>& D, int p0, int p1, const AdvArgs& a,
                                 int* err, cudaStream_t s) {
   switch (D.mx) {
-    case 8: return walk_nw<real, 8>(D, p0, p1, a, err, s);
-    case 16: return walk_nw<real, 16>(D, p0, p1, a, err, s);
-    case 32: return walk_nw<real, 32>(D, p0, p1, a, err, s);
+    case 8: return walk_opt<real, 8>(D, p0, p1, a, err, s);
+    case 16: return walk_opt<real, 16>(D, p0, p1, a, err, s);
+    case 32: return walk_opt<real, 32>(D, p0, p1, a, err, s);
     default: return cudaErrorInvalidValue;
   }
 }

@@ -327,6 +327,21 @@ __global__ void remap_kernel(DevForest<real> Old, DevForest<real> New, const Rem
   }
 }
 
+// ------------------------------------------------------------------ trig
+
+// the swirl streamfunction's factors along one axis of a level, once per
+// forest (a patch needs 4 (mx + 3) of them each update: in FP64 that was a
+// third of the update's FP64 instructions)
+template <typename real>
+__global__ void trig_kernel(real* out, int len, real h) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= len) return;
+  const int z = k - 1;
+  const real s = sinpi_r(real(z) * h);
+  out[k] = s * s;
+  out[len + k] = sinpi_r(real(2 * z + 1) * h);
+}
+
 inline int grid_for(int n) { return n < 1 ? 1 : (n < 65535 * 8 ? n : 65535 * 8); }
 
 // Refluxing (Berger and Colella's correction; the paper's scheme has none):
@@ -438,6 +453,13 @@ cudaError_t launch_reflux(const DevForest<real>& D, int p0, int p1, const real* 
       break;
     default: return cudaErrorInvalidValue;
   }
+  ++launch_counter();
+  return cudaGetLastError();
+}
+
+template <typename real>
+cudaError_t launch_trig(real* out, int len, double h, cudaStream_t s) {
+  trig_kernel<real><<<(len + 255) / 256, 256, 0, s>>>(out, len, real(h));
   ++launch_counter();
   return cudaGetLastError();
 }
@@ -568,6 +590,7 @@ cudaError_t launch_reflux_pairs(const DevForest<real>& D, int p0, int p1, const 
 }
 
 #define FC_INSTANTIATE(real)                                                                   \
+  template cudaError_t launch_trig<real>(real*, int, double, cudaStream_t);                    \
   template cudaError_t launch_tag<real>(const DevForest<real>&, int, double*, cudaStream_t);        \
   template cudaError_t launch_reflux<real>(const DevForest<real>&, int, int, const real*, int, int, \
                                            double, double, cudaStream_t);                          \

@@ -236,6 +236,12 @@ struct fc_forest {
   int walk_ctas = 0;                    // cap on the walk grid (0: residency)
   uint32_t wait_polls = kWaitLimit;     // polls of the update kernels' bounded waits
   double vel_scale = 1.0;                 // multiplies every edge speed
+  // the swirl's streamfunction factors per level (AdvArgs::trig), made once:
+  // they depend on the level and mx alone
+  void* d_trig = nullptr;
+  size_t trig_bytes = 0;
+  size_t trig_off[kMaxLevel + 1] = {};  // in values
+  int trig_len[kMaxLevel + 1] = {};     // 0: not held
   double* d_metric = nullptr;             // cubed sphere: FP64 metric blocks per patch
   double* d_corner = nullptr;             // deformational flow: grid corners per patch
   void* lam[2] = {nullptr, nullptr};      // adjoint tiles (patch-store layout), lazily allocated
@@ -407,6 +413,8 @@ void free_device(fc_forest* F) {
   dfree(F->d_remap);
   dfree(F->d_err);
   dfree(F->d_t0);
+  dfree(F->d_trig);
+  F->trig_bytes = 0;
   dfree(F->lam[0]);
   dfree(F->lam[1]);
   for (auto& b : F->madj) dfree(b);
@@ -449,6 +457,37 @@ fc_status update_metrics(fc_forest* F, const RemapEntry* rm = nullptr,
   }
   FC_CUDA(launch_sphere_metrics(F->d_meta, n, H.desc.mx, w, F->d_metric, rm, old, F->d_corner,
                                 g_alloc_stream));
+  return FC_OK;
+}
+
+// the tables of the swirl's streamfunction for the levels of up to 32768
+// cells along the domain (256 KB of FP32 a table; beyond, the kernels
+// compute the factors)
+fc_status make_trig(fc_forest* F) {
+  const fc_forest_desc& d = F->host.desc;
+  if (d.vel_kind != FC_VEL_SWIRL || F->d_trig) return FC_OK;
+  size_t off = 0;
+  for (int l = d.lmin; l <= d.lmax; ++l) {
+    F->trig_len[l] = 0;
+    if (((size_t)d.mx << l) > 32768) continue;
+    F->trig_off[l] = off;
+    F->trig_len[l] = (d.mx << l) + 4;
+    off += 2 * (size_t)F->trig_len[l];
+  }
+  if (off == 0) return FC_OK;
+  F->trig_bytes = off * F->esize;
+  if (dmalloc_bytes(&F->d_trig, F->trig_bytes) != cudaSuccess)
+    return fail(FC_ERR_OOM, "streamfunction table allocation failed");
+  for (int l = d.lmin; l <= d.lmax; ++l) {
+    if (!F->trig_len[l]) continue;
+    const double h = std::ldexp(1.0, -l) / d.mx;
+    if (F->esize == 4)
+      FC_CUDA(launch_trig(static_cast<float*>(F->d_trig) + F->trig_off[l], F->trig_len[l], h,
+                          g_alloc_stream));
+    else
+      FC_CUDA(launch_trig(static_cast<double*>(F->d_trig) + F->trig_off[l], F->trig_len[l], h,
+                          g_alloc_stream));
+  }
   return FC_OK;
 }
 
@@ -631,6 +670,11 @@ AdvArgs adv_args(const fc_forest* F, int L, double t, double dt, int n) {
   a.alpha = 0.0;
   a.bflux = F->bflux;
   a.bslot = 0;
+  a.level = L;
+  if (F->d_trig && F->trig_len[L]) {
+    a.trig = static_cast<const char*>(F->d_trig) + F->trig_off[L] * F->esize;
+    a.trig_len = F->trig_len[L];
+  }
   choose_variant(F, n, &a);
   return a;
 }
@@ -641,23 +685,46 @@ int size_bucket(int n) {
   return b;
 }
 
+// From how many patches a launch of a planar level is the walk's: where its
+// one-level step (uniform forests, one GB300) passes the band's.
+//   us, band / walk   n = 640        1280         2560         6400
+//   FP32 mx = 32   15.3 / 16.6  20.8 / 18.7  31.2 / 22.9  66.0 / 39.3
+//        mx = 16   12.2 / 18.7  14.7 / 18.7  18.8 / 20.8  35.1 / 23.0
+//        mx = 8    10.6 / 16.7  10.6 / 16.8  14.5 / 16.8  23.0 / 18.7
+//   FP64 mx = 32   90.5 / 74.3   156 / 115    289 / 217    721 / 496
+//        mx = 16   35.2 / 39.2  49.4 / 45.9  88.6 / 69.9   203 / 148
+//        mx = 8    18.7 / 27.1  29.1 / 28.9  49.8 / 33.1   103 / 53.5
+// (FP64 mx = 32 at 320: 57.7 / 61.8)
+int walk_from(int mx, size_t esize) {
+  if (esize == 4) return mx == 32 ? 768 : mx == 16 ? 3072 : 4096;
+  return mx == 32 ? 384 : mx == 16 ? 1024 : 1280;
+}
+
 // the patch-update configuration for a launch of n patches: the autotuned
 // choice when this size was tuned, else walk for launches that fill the GPU
 // (planar grids) and band for the others
 void choose_variant(const fc_forest* F, int n, AdvArgs* a) {
   const fc_forest::Tune& t = F->tune[size_bucket(n)];
+  const int mx = F->host.desc.mx;
   if (F->forced_variant >= 0) {
     a->variant = F->forced_variant;
     a->warps = F->forced_warps;
   } else if (t.tuned) {
     a->variant = t.variant;
     a->warps = t.warps;
-  } else if (n >= 1024 && !F->d_metric && F->host.desc.domain != FC_DOMAIN_SPHERE) {
-    a->variant = ADV_WALK;  // (it has no capacity form)
-    a->warps = F->esize == 4 ? 4 : 2;
+  } else if (n >= walk_from(mx, F->esize) && !F->d_metric &&
+             F->host.desc.domain != FC_DOMAIN_SPHERE) {
+    // (it has no capacity form).  FP64: CTAs of two warps spread a launch of
+    // few groups over the SMs, whose FP64 pipes are what it waits for
+    a->variant = ADV_WALK;
+    a->warps = F->esize == 4 ? 8 : 2;
   } else {
+    // rows a band, by warps: at mx = 16 one row of a patch a warp segment (8
+    // warps) computes every x-edge three times; FP64, 320 patches: 31.0 us,
+    // two rows 23.0, four 20.9 (64 patches: 16.7, 16.6, 18.7); FP32, 1280
+    // patches: 16.7, 14.7, 14.7 (64: the same)
     a->variant = ADV_BAND;
-    a->warps = 8;
+    a->warps = mx == 16 ? (F->esize == 8 && n >= 128 ? 2 : 4) : 8;
   }
   // only the staged and band updates record the face fluxes
   if (F->bflux && a->variant != ADV_STAGED && a->variant != ADV_BAND) {
@@ -789,10 +856,11 @@ fc_status advance_level_t(fc_forest* F, int L, double t, double dt, cudaStream_t
       // the level's chain (at alpha = 0 from the coarser level's older
       // state, which its running update does not write); in the adjoint's
       // replay they also store those cells in the kept time-interpolated
-      // tiles, all the reverse reads of them.  The walk keeps the fill: with
-      // one warp per patch, computing those cells in the update measured
-      // slower on the ensemble (5.5e10 vs 7.4e10 cell-updates/s)
-      const bool direct = tlevel >= 0 && (a.variant == ADV_STAGED || a.variant == ADV_BAND);
+      // tiles, all the reverse reads of them.  The walk computes each coarse
+      // cell beside a face once for its four ghosts; in the adjoint's replay
+      // it keeps the fill, which leaves the tiles the reverse reads
+      const bool walk = a.variant == ADV_WALK || a.variant == ADV_WALK1;
+      const bool direct = tlevel >= 0 && !(walk && F->keep_qT);
       if (direct) A.ntargets = 0;
       a.direct = direct ? 1 : 0;
       if (direct && F->keep_qT) {
@@ -1010,6 +1078,7 @@ fc_status fc_forest_info(const fc_forest* F, fc_info* out) {
   if (F->d_corner) bytes += sizeof(double) * n * 3 * (S + 1) * (S + 1);
   for (void* b : F->lam) bytes += b ? store : 0;
   for (void* b : F->madj) bytes += b ? store : 0;
+  bytes += F->trig_bytes;
   if (F->mio) bytes += n * H.desc.mx * H.desc.mx * F->esize;
   bytes += F->msnap_bytes;
   for (const auto& t : F->tapes) bytes += t.bytes;
@@ -1054,6 +1123,7 @@ fc_status fc_forest_create(const fc_forest_desc* desc, int nleaves, const int* l
   }
   keep_pool_memory();
   st = upload(F, true);  // on the legacy default stream
+  if (st == FC_OK) st = make_trig(F);
   if (st == FC_OK && cudaStreamSynchronize(0) != cudaSuccess) st = cuda_fail(cudaGetLastError(), "create");
   if (st != FC_OK) {
     free_device(F);
@@ -1187,8 +1257,8 @@ fc_status fc_autotune(fc_forest* F, int* report, void* stream) {
   // (band with 16 warps is left out: timed a level at a time it can win,
   // but beside the other levels' branches of a captured step it measured
   // slower than with 8)
-  } cand[] = {{ADV_STAGED, 4}, {ADV_BAND, 4}, {ADV_BAND, 8},  {ADV_WALK, 2},
-              {ADV_WALK, 4},   {ADV_WALK, 8}, {ADV_WALK1, 4}, {ADV_WALK1, 8}};
+  } cand[] = {{ADV_STAGED, 4}, {ADV_BAND, 4}, {ADV_BAND, 8},
+              {ADV_WALK, 2},   {ADV_WALK, 4}, {ADV_WALK, 8}};
   constexpr int ncand = sizeof(cand) / sizeof(cand[0]);
   cudaEvent_t e0, e1;
   FC_CUDA(cudaEventCreate(&e0));
@@ -1225,13 +1295,13 @@ fc_status fc_autotune(fc_forest* F, int* report, void* stream) {
       a.variant = c.variant;
       a.warps = c.warps;
       a.gather = fused;
-      a.tlevel = -1;
+      // as in a step: the update computes its coarse neighbours' cells itself
+      a.direct = fused && L > H.desc.lmin ? 1 : 0;
+      a.tlevel = a.direct ? L - 1 : -1;
+      a.alpha = a.direct ? 0.5 : 0.0;
       auto run = [&]() {
-        cudaError_t e;
-        if (fused) {
-          FillArgs A{F->d_lists + F->off_t[L], (int)H.list_t[L].size(), -1, 0.0};
-          e = F->esize == 4 ? launch_fill_coarse(Df, A, s) : launch_fill_coarse(Dd, A, s);
-        } else {
+        cudaError_t e = cudaSuccess;
+        if (!fused) {
           FillArgs A{F->d_lists + F->off_a[L], (int)H.list_a[L].size(), -1, 0.0};
           FillArgs B{F->d_lists + F->off_b[L], (int)H.list_b[L].size(), -1, 0.0};
           e = F->esize == 4 ? launch_fill_coarse(Df, A, s) : launch_fill_coarse(Dd, A, s);
@@ -2277,7 +2347,12 @@ fc_status fc_tag_regrid(fc_forest* F, double tau_refine, double tau_coarsen,
   retire_graphs(F);
   F->d_err = nullptr;  // (G holds them)
   F->d_t0 = nullptr;
+  void* const trig = F->d_trig;  // (of the levels, not of the layout)
+  const size_t trig_bytes = F->trig_bytes;
+  F->d_trig = nullptr;
   free_device(F);
+  F->d_trig = trig;
+  F->trig_bytes = trig_bytes;
   F->spare_nbr.swap(F->host.nbr);  // the next regrid's build writes here
   F->spare_meta.swap(F->host.meta);
   F->host = std::move(G->host);
@@ -2444,6 +2519,7 @@ fc_status fc_forest_create_part(const fc_forest_desc* desc, int nleaves, const i
   keep_pool_memory();
   const HostForest& H = F->host;
   st = upload(F, true);
+  if (st == FC_OK) st = make_trig(F);
   // the exchange lists, one block: per (level or all, rank) the send list,
   // then the receive list
   std::vector<int> lists;

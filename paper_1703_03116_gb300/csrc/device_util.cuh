@@ -5,11 +5,21 @@
 
 namespace fc {
 
-template <typename real>
-__device__ __forceinline__ real minmod(real a, real b) {
-  // by the signs: a product of two small slopes underflows
-  if ((a <= real(0) && b >= real(0)) || (a >= real(0) && b <= real(0))) return real(0);
-  return fabs(a) < fabs(b) ? a : b;
+// the smaller of two slopes of one sign, else 0 (decided by the signs: a
+// product of two small slopes underflows)
+__device__ __forceinline__ float minmod(float a, float b) {
+  if ((a <= 0.f && b >= 0.f) || (a >= 0.f && b <= 0.f)) return 0.f;
+  return fabsf(a) < fabsf(b) ? a : b;
+}
+// the same on the bits: no FP64 instruction (the FP64 pipe issues 1/64 of an
+// SM's slots); a NaN gives b, as the comparisons do
+__device__ __forceinline__ double minmod(double a, double b) {
+  constexpr long long kMag = 0x7fffffffffffffffll, kInf = 0x7ff0000000000000ll;
+  const long long x = __double_as_longlong(a), y = __double_as_longlong(b);
+  const long long ax = x & kMag, ay = y & kMag;
+  if (ax > kInf || ay > kInf) return b;
+  if ((x ^ y) < 0 || ax == 0 || ay == 0) return 0.0;
+  return ax < ay ? a : b;
 }
 
 // Signed permutation A of Eq. (transform): bit 0 swaps the axes, bits 1 and

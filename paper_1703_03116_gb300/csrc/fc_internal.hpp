@@ -479,6 +479,12 @@ struct AdvArgs {
   // bflux + ((p * 2 + bslot) * 4 + face) * mx (faces -x, +x, -y, +y; null: off)
   void* bflux;
   int bslot;
+  int level;  // of the launch's patches
+  // the streamfunction's factors at the level's nodes z = -1..N + 2 (N cells
+  // along the domain), in the field's precision: sin^2(pi z h) at [z + 1],
+  // sin(pi (2 z + 1) h) at [trig_len + z + 1]; null: the kernel computes them
+  const void* trig;
+  int trig_len;
 };
 
 // Patch-update kernel variants (chosen per level launch by the autotuner):
@@ -497,6 +503,10 @@ cudaError_t launch_advance_walk(const DevForest<real>& D, int p0, int p1, const 
 template <typename real>
 cudaError_t launch_advance_band(const DevForest<real>& D, int p0, int p1, const AdvArgs& a,
                                 int* err, cudaStream_t s);
+
+// the table of AdvArgs::trig for cell width h: 2 len values at out
+template <typename real>
+cudaError_t launch_trig(real* out, int len, double h, cudaStream_t s);
 
 cudaError_t launch_set_time(double* t0_dev, double t0, cudaStream_t s);
 // *dst += *src (one thread; device doubles)

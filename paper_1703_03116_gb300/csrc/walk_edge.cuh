@@ -12,7 +12,7 @@
 //   correction        1/2 |s| (1 - |s| dt/h) lim   ->  |c| (1/2 - |c|) lim
 //   transverse share  1/2 dt/h s X                 ->  c X
 //   update            q - dt/h (dF + dG)           ->  q - 2 (dF + dG)
-// and 2 lim = min(|W + Wup|, 4 |W|, 4 |Wup|) takes the limiter's factors.
+// and the limiter's factors go into the correction's.
 // The FP64 pipe issues 1/64 of an SM's slots, so what bounds the FP64 update
 // is its count of FP64 instructions: about 25 a cell in this form, of 66 in
 // the speeds' own units with min, max and compares in FP64 -- the minima,
@@ -32,15 +32,18 @@ namespace fc {
 // holds no selection by option (8 instructions a cell in FP32).
 template <typename real, bool FULL>
 struct Scheme {
-  real k0 = real(0.25);  // correction |c| (k0 - k1 |c|) m, m = 2 lim (MC) or W (unlimited):
-  real k1 = real(0.5);   //   1/4, 1/2 with MC; 1/2, 1 unlimited; 0, 0 first order
+  // the correction's factor |c| (k0 - k1 |c|) of the limited wave, k1 = 2 k0:
+  // MC in FP32 of lim / 2 (k0 = 1), in FP64 of 2 lim (1/4: fewer FP64
+  // instructions, see limited()); unlimited of W (1/2); first order 0
+  static constexpr real kMC = sizeof(real) == 4 ? real(1) : real(0.25);
+  real k0 = kMC, k1 = real(2) * kMC;
   bool mc_ = true;       // MC limiter
   bool t1_ = true, t2_ = true;  // transverse fluctuations; their corrections too
   __device__ __forceinline__ bool mc() const { return FULL || mc_; }
   __device__ __forceinline__ bool t1() const { return FULL || t1_; }
   __device__ __forceinline__ bool t2() const { return FULL || t2_; }
-  __device__ __forceinline__ real c0() const { return FULL ? real(0.25) : k0; }
-  __device__ __forceinline__ real c1() const { return FULL ? real(0.5) : k1; }
+  __device__ __forceinline__ real c0() const { return FULL ? kMC : k0; }
+  __device__ __forceinline__ real c1() const { return FULL ? real(2) * kMC : k1; }
 };
 
 inline bool full_scheme(int order, int limiter, int transverse) {
@@ -53,7 +56,7 @@ __device__ __forceinline__ Scheme<real, FULL> make_scheme(int order, int limiter
   Scheme<real, FULL> sc;
   if (!FULL) {
     sc.mc_ = limiter != 0;
-    sc.k0 = order > 1 ? (sc.mc_ ? real(0.25) : real(0.5)) : real(0);
+    sc.k0 = order > 1 ? (sc.mc_ ? sc.kMC : real(0.5)) : real(0);
     sc.k1 = real(2) * sc.k0;
     sc.t1_ = transverse > 0;
     sc.t2_ = transverse > 1;
@@ -89,16 +92,16 @@ inline AdvConst<real> adv_const(const DevForest<real>& D, const AdvArgs& a) {
 __device__ __forceinline__ bool upwind_left(float c) { return c >= 0.f; }
 __device__ __forceinline__ bool upwind_left(double c) { return __double2hiint(c) >= 0; }
 
-// twice the MC-limited wave: 0 unless W and Wup share a sign, else
-// sign(W) min(|W + Wup|, 4 |W|, 4 |Wup|).  (A zero wave gives a zero minimum,
-// so the signs' bits decide.)
-__device__ __forceinline__ float mc_twice(float W, float Wup) {
-  const float m = fminf(fabsf(W + Wup), 4.f * fminf(fabsf(W), fabsf(Wup)));
+// The MC-limited wave, 0 unless W and Wup share a sign, else sign(W)
+// min(|W + Wup| / 2, 2 |W|, 2 |Wup|), up to the factor above: half of it in
+// FP32, twice it in FP64.
+__device__ __forceinline__ float limited(float W, float Wup) {
+  const float m = fminf(fabsf(0.25f * (W + Wup)), fminf(fabsf(W), fabsf(Wup)));
   return (__float_as_int(W) ^ __float_as_int(Wup)) >= 0 ? copysignf(m, W) : 0.f;
 }
 // one FP64 instruction (the sum): magnitudes compare as integers, 4 x adds 2
 // to the exponent; a minimum below the normal range counts as zero
-__device__ __forceinline__ double mc_twice(double W, double Wup) {
+__device__ __forceinline__ double limited(double W, double Wup) {
   constexpr unsigned long long kMag = 0x7fffffffffffffffull;
   const unsigned long long w = (unsigned long long)__double_as_longlong(W);
   const unsigned long long u = (unsigned long long)__double_as_longlong(Wup);
@@ -124,32 +127,35 @@ __device__ __forceinline__ real corr_factor_cap(real c, real w, const Scheme<rea
   return a * fma(-sc.c0() * a, w, sc.c0());
 }
 
-// the edge between cells qb and qc (W = qc - qb, Wup the upwind edge's jump,
-// k the correction's factor): normal flux and the fluctuations entering the
-// right / upper (P) and the left / lower (M) cell
+// The edge between cells qb and qc (W = qc - qb, Wup the upwind edge's jump,
+// k the correction's factor): normal flux F and the fluctuations P entering
+// the right / upper cell, as nP = -P, and M entering the left / lower cell.
+// Sums of fluctuations are carried with their sign turned (nX = -X): every
+// step is then an addition or a fused multiply-add without a negation of its
+// own (an FP64 instruction in FP64, two integer ones in the packed form).
 template <bool FULL>
 __device__ __forceinline__ void edge_flux(float c, float W, float Wup, float qb, float qc, float k,
-                                          const Scheme<float, FULL>& sc, float& Fn, float& P, float& M) {
+                                          const Scheme<float, FULL>& sc, float& F, float& nP,
+                                          float& M) {
   const float cp = fmaxf(c, 0.f), cm = fminf(c, 0.f);
-  const float Ft = k * (sc.mc() ? mc_twice(W, Wup) : W);
+  const float Ft = k * (sc.mc() ? limited(W, Wup) : W);
   const float T = sc.t2() ? Ft : 0.f;
-  Fn = fmaf(cp, qb, fmaf(cm, qc, Ft));
-  P = fmaf(cp, W, -T);
+  F = fmaf(cp, qb, fmaf(cm, qc, Ft));
+  nP = fmaf(-cp, W, T);
   M = fmaf(cm, W, T);
 }
-// (one of the two products with max(c, 0), min(c, 0) is zero: selected)
+// (one of the two fluctuations is the correction alone: selected)
 template <bool FULL>
 __device__ __forceinline__ void edge_flux(double c, double W, double Wup, double qb, double qc,
-                                          double k, const Scheme<double, FULL>& sc, double& Fn,
-                                          double& P, double& M) {
+                                          double k, const Scheme<double, FULL>& sc, double& F,
+                                          double& nP, double& M) {
   const bool up = upwind_left(c);
-  const double Ft = k * (sc.mc() ? mc_twice(W, Wup) : W);
+  const double Ft = k * (sc.mc() ? limited(W, Wup) : W);
   const double T = sc.t2() ? Ft : 0.0;
-  Fn = fma(c, up ? qb : qc, Ft);
-  const double Ts = up ? -T : T;
-  const double A = fma(c, W, Ts);
-  P = up ? A : -T;
-  M = up ? T : A;
+  F = fma(c, up ? qb : qc, Ft);
+  const double B = fma(-fabs(c), W, T);
+  nP = up ? B : T;
+  M = up ? T : B;
 }
 
 // the jump on the upwind side of an edge from its four cells
@@ -165,23 +171,146 @@ __device__ __forceinline__ double upwind_jump(double c, double qa, double qb, do
 // an edge from its four cells qa..qd
 template <typename real, bool FULL>
 __device__ __forceinline__ void edge(real c, real qa, real qb, real qc, real qd, real k,
-                                     const Scheme<real, FULL>& sc, real& Fn, real& P, real& M) {
-  edge_flux(c, qc - qb, upwind_jump(c, qa, qb, qc, qd), qb, qc, k, sc, Fn, P, M);
+                                     const Scheme<real, FULL>& sc, real& F, real& nP, real& M) {
+  edge_flux(c, qc - qb, upwind_jump(c, qa, qb, qc, qd), qb, qc, k, sc, F, nP, M);
 }
 
 // final flux: the normal flux F less the transverse shares of the fluctuation
-// sums Xm, Xp in the cells before and beyond the edge
+// sums in the cells before and beyond the edge (nXm, nXp: turned)
 template <bool FULL>
-__device__ __forceinline__ float final_flux(float c, float Xm, float Xp, float F,
+__device__ __forceinline__ float final_flux(float c, float nXm, float nXp, float F,
                                             const Scheme<float, FULL>& sc) {
   const float ct = sc.t1() ? c : 0.f;
-  return fmaf(-fmaxf(ct, 0.f), Xm, fmaf(-fminf(ct, 0.f), Xp, F));
+  return fmaf(fmaxf(ct, 0.f), nXm, fmaf(fminf(ct, 0.f), nXp, F));
 }
 template <bool FULL>
-__device__ __forceinline__ double final_flux(double c, double Xm, double Xp, double F,
+__device__ __forceinline__ double final_flux(double c, double nXm, double nXp, double F,
                                              const Scheme<double, FULL>& sc) {
-  const double X = upwind_left(c) ? Xm : Xp;
-  return fma(-c, sc.t1() ? X : 0.0, F);
+  const double X = upwind_left(c) ? nXm : nXp;
+  return fma(c, sc.t1() ? X : 0.0, F);
+}
+
+}  // namespace fc
+
+// ------------------------------------------------ the walk's packed form
+//
+// The FP32 walk computes two cells at a time in packed registers (float2:
+// add, sub, mul and fma are one instruction for both), the FP64 walk one
+// (double).
+namespace fc {
+
+__device__ __forceinline__ float2 vadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 vmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 vfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 vsub(float2 a, float2 b) {
+  float2 r;
+  asm("{\n .reg .b64 a, b, c;\n mov.b64 a, {%2, %3};\n mov.b64 b, {%4, %5};\n"
+      " sub.rn.f32x2 c, a, b;\n mov.b64 {%0, %1}, c;\n}"
+      : "=f"(r.x), "=f"(r.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return r;
+}
+__device__ __forceinline__ double vadd(double a, double b) { return a + b; }
+__device__ __forceinline__ double vsub(double a, double b) { return a - b; }
+__device__ __forceinline__ double vmul(double a, double b) { return a * b; }
+__device__ __forceinline__ double vfma(double a, double b, double c) { return fma(a, b, c); }
+
+template <typename real>
+struct Packed;
+template <>
+struct Packed<float> {
+  using V = float2;
+  static constexpr int N = 2;
+  static __device__ __forceinline__ V all(float a) { return make_float2(a, a); }
+  static __device__ __forceinline__ V make(float a, float b) { return make_float2(a, b); }
+  static __device__ __forceinline__ float get(V v, int k) { return k ? v.y : v.x; }
+};
+template <>
+struct Packed<double> {
+  using V = double;
+  static constexpr int N = 1;
+  static __device__ __forceinline__ V all(double a) { return a; }
+  static __device__ __forceinline__ V make(double a, double) { return a; }
+  static __device__ __forceinline__ double get(V v, int) { return v; }
+};
+
+// a half Courant number, split by sign where the products with both parts
+// are cheaper than a selection (FP32)
+template <typename V>
+struct Speed;
+template <>
+struct Speed<float2> {
+  float2 c, p, m;  // p + m = c
+  Speed() = default;
+  __device__ __forceinline__ explicit Speed(float2 v) : c(v) {
+    p = make_float2(fmaxf(v.x, 0.f), fmaxf(v.y, 0.f));
+    m = vsub(v, p);
+  }
+};
+template <>
+struct Speed<double> {
+  double c;
+  Speed() = default;
+  __device__ __forceinline__ explicit Speed(double v) : c(v) {}
+};
+
+// limited() of both packed cells: the same value, by ordering (fewer
+// instructions; the form above has the shorter chain, which the band update
+// with its few warps waits for: 0.139 against 0.123 ms a coarse step)
+__device__ __forceinline__ float2 limited(float2 W, float2 U) {
+  const float2 s4 = vmul(vadd(W, U), make_float2(0.25f, 0.25f));
+  const float2 lo = make_float2(fmaxf(fminf(fminf(s4.x, W.x), U.x), 0.f),
+                                fmaxf(fminf(fminf(s4.y, W.y), U.y), 0.f));
+  const float2 hi = make_float2(fminf(fmaxf(fmaxf(s4.x, W.x), U.x), 0.f),
+                                fminf(fmaxf(fmaxf(s4.y, W.y), U.y), 0.f));
+  return vadd(lo, hi);
+}
+
+// one edge for both packed cells: normal flux F, nP = -P and M
+template <bool FULL>
+__device__ __forceinline__ void vedge(const Speed<float2>& s, float2 W, float2 U, float2 qb,
+                                      float2 qc, const Scheme<float, FULL>& sc, float2& F,
+                                      float2& nP, float2& M) {
+  const float2 ab = vsub(s.p, s.m);  // |c|
+  const float c0 = sc.c0(), c1 = -sc.c1();
+  const float2 k = vmul(ab, vfma(make_float2(c1, c1), ab, make_float2(c0, c0)));
+  const float2 Ft = vmul(k, sc.mc() ? limited(W, U) : W);
+  const float2 T = sc.t2() ? Ft : make_float2(0.f, 0.f);
+  F = vfma(s.p, qb, vfma(s.m, qc, Ft));
+  nP = vfma(s.p, vsub(qb, qc), T);
+  M = vfma(s.m, W, T);
+}
+template <bool FULL>
+__device__ __forceinline__ void vedge(const Speed<double>& s, double W, double U, double qb,
+                                      double qc, const Scheme<double, FULL>& sc, double& F,
+                                      double& nP, double& M) {
+  edge_flux(s.c, W, U, qb, qc, corr_factor(s.c, sc), sc, F, nP, M);
+}
+
+__device__ __forceinline__ float2 vselect(float2 c, float2 a, float2 b) {
+  return make_float2(upwind_left(c.x) ? a.x : b.x, upwind_left(c.y) ? a.y : b.y);
+}
+__device__ __forceinline__ double vselect(double c, double a, double b) {
+  return upwind_left(c) ? a : b;
+}
+// the jump on the upwind side from an edge's four cells
+__device__ __forceinline__ float2 vupwind(float2 c, float2 qa, float2 qb, float2 qc, float2 qd) {
+  return vselect(c, vsub(qb, qa), vsub(qd, qc));
+}
+__device__ __forceinline__ double vupwind(double c, double qa, double qb, double qc, double qd) {
+  return upwind_jump(c, qa, qb, qc, qd);
+}
+
+// final flux from the turned sums nXm, nXp
+template <bool FULL>
+__device__ __forceinline__ float2 vfinal(const Speed<float2>& s, float2 nXm, float2 nXp, float2 F,
+                                         const Scheme<float, FULL>& sc) {
+  return sc.t1() ? vfma(s.p, nXm, vfma(s.m, nXp, F)) : F;
+}
+template <bool FULL>
+__device__ __forceinline__ double vfinal(const Speed<double>& s, double nXm, double nXp, double F,
+                                         const Scheme<double, FULL>& sc) {
+  return final_flux(s.c, nXm, nXp, F, sc);
 }
 
 }  // namespace fc
