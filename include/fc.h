@@ -88,7 +88,8 @@ typedef enum { FC_VEL_CONST = 0, FC_VEL_SWIRL = 1, FC_VEL_ROTATION = 2, FC_VEL_D
  *               psi differences between the edges' end points, formed as
  *               k c (s_b - s_a)(s_b + s_a) - (2 pi/T_f)(Z_b - Z_a) with
  *               s = Y cos(2 pi t/T) - X sin(2 pi t/T), c = cos(pi t/T),
- *               from the grid corners kept per patch (3 (mx+5)^2 doubles);
+ *               from coefficients kept per edge (8 (mx+4)(mx+5) doubles a
+ *               patch);
  *               times the velocity scale.
  *               FC_VEL_ROTATION (sphere only): solid-body rotation
  *               u = omega x X, omega = (vel[0], vel[1], vel[2]).  The sphere

@@ -14,8 +14,8 @@
 // then reads its four fluxes.  Every thread works on every phase, so a patch
 // finishes quickly -- the better choice when a launch has few patches.
 //
-// Capacity form (CAP, the cubed sphere, Sec. 5.3): the patch's FP64 metric
-// block arrives by a second bulk copy.  Edge speeds become edge volume fluxes
+// Capacity form (CAP, the cubed sphere, Sec. 5.3): the patch's metric block
+// (field precision) arrives by a second bulk copy.  Edge speeds become edge volume fluxes
 // phi, and every 1/h becomes 1/kappa of the cell concerned: the correction
 // 1/2 |phi| (1 - dt |phi| (1/kappa_L + 1/kappa_R)/2) phi(theta) W, the
 // transverse increments 1/2 dt/kappa_cell phi^-+ (fluctuation entering that
@@ -49,7 +49,7 @@ __global__ void __launch_bounds__(NT, NT >= 512 ? (sizeof(real) == 4 ? 3 : 2)
   constexpr int S = MX + 4;
   constexpr int NE = (MX + 1) * (MX + 2);
   constexpr int NV = MX + 3;  // corner nodes -1..MX+1
-  constexpr int MS = CAP ? metric_stride(S) : 0;
+  constexpr int MS = CAP ? umetric_stride(S) : 0;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t bar;
   __shared__ real ucoef_s;
@@ -69,9 +69,9 @@ __global__ void __launch_bounds__(NT, NT >= 512 ? (sizeof(real) == 4 ? 3 : 2)
   constexpr int NCHUNK = (2 * NI + 31) / 32;  // warp-sized chunks of them
   constexpr int NB = 6 * MX + 2;              // boundary edges per direction
   __shared__ int chunk_next;
-  // capacity form: kappa, phi_x, phi_y of the patch (MS doubles) come first
-  const double* Ms = reinterpret_cast<const double*>(smem_raw);
-  real* Q = reinterpret_cast<real*>(smem_raw + sizeof(double) * MS);
+  // capacity form: 1/kappa, phi_x, phi_y of the patch (MS values) come first
+  const real* Ms = reinterpret_cast<const real*>(smem_raw);
+  real* Q = reinterpret_cast<real*>(smem_raw + sizeof(real) * MS);
   real* Fn = Q + S * S;
   real* XP = Fn + NE;
   real* XM = XP + NE;
@@ -87,7 +87,7 @@ __global__ void __launch_bounds__(NT, NT >= 512 ? (sizeof(real) == 4 ? 3 : 2)
   const real cu = real(D.vel[0]), cv = real(D.vel[1]);
   const real nu = real(a.nu), half_nu = real(0.5 * a.nu), h = real(a.h);
   constexpr uint32_t bytes = sizeof(real) * S * S;
-  constexpr uint32_t mbytes = sizeof(double) * MS;
+  constexpr uint32_t mbytes = sizeof(real) * MS;
   const real dt = real(a.dt), half_dt = real(0.5 * a.dt);
 
   if (threadIdx.x == 0) {
@@ -107,29 +107,29 @@ __global__ void __launch_bounds__(NT, NT >= 512 ? (sizeof(real) == 4 ? 3 : 2)
       fence_proxy_async();
       mbar_expect_tx(&bar, bytes + mbytes);
       bulk_load(Q, src, bytes, &bar);
-      if (CAP) bulk_load(smem_raw, D.metric + (size_t)p * MS, mbytes, &bar);
+      if (CAP) bulk_load(smem_raw, D.umetric + (size_t)p * MS, mbytes, &bar);
     }
     if (swirl && threadIdx.x == NT - 1 && p == p0 + (int)blockIdx.x) {
       const double t = a.t0_dev ? *a.t0_dev + a.t_off : a.t_half;
       ucoef_s = cospi_ratio<real>(t, a.period) * real(a.sfac);
     }
     auto q = [&](int i, int j) -> real { return Q[(j + 2) * S + (i + 2)]; };
-    // capacity form: kappa of cell (i,j), flux through x-edge / y-edge (i,j)
-    auto kap = [&](int i, int j) -> real { return real(Ms[(j + 2) * S + (i + 2)]); };
+    // capacity form: 1/kappa of cell (i,j), flux through x-edge / y-edge (i,j)
+    auto ik = [&](int i, int j) -> real { return Ms[(j + 2) * S + (i + 2)]; };
     auto uvel = [&](int i, int j) -> real {
-      if (CAP) return real(Ms[S * S + (j + 2) * (S + 1) + (i + 2)]);
+      if (CAP) return Ms[S * S + (j + 2) * (S + 1) + (i + 2)];
       return swirl ? ucoef * Sx[i + 1] * Ty[j + 1] : cu;
     };
     auto vvel = [&](int i, int j) -> real {
-      if (CAP) return real(Ms[S * S + S * (S + 1) + (j + 2) * S + (i + 2)]);
+      if (CAP) return Ms[S * S + S * (S + 1) + (j + 2) * S + (i + 2)];
       return swirl ? -ucoef * Sy[j + 1] * Tx[i + 1] : cv;
     };
     // dt |phi| (1/kappa_L + 1/kappa_R)/2 = nu_e |phi| in the correction
     auto nu_x = [&](int i, int j) -> real {
-      return CAP ? dt * (real(0.5) * (real(1) / kap(i - 1, j) + real(1) / kap(i, j))) : nu;
+      return CAP ? dt * (real(0.5) * (ik(i - 1, j) + ik(i, j))) : nu;
     };
     auto nu_y = [&](int i, int j) -> real {
-      return CAP ? dt * (real(0.5) * (real(1) / kap(i, j - 1) + real(1) / kap(i, j))) : nu;
+      return CAP ? dt * (real(0.5) * (ik(i, j - 1) + ik(i, j))) : nu;
     };
     // normal flux and fluctuations of x-edge (i, j) (cells (i-1,j) | (i,j))
     // and of y-edge (i, j) (cells (i,j-1) | (i,j))
@@ -311,7 +311,7 @@ __global__ void __launch_bounds__(NT, NT >= 512 ? (sizeof(real) == 4 ? 3 : 2)
           const real yl = YP[ye(i - 1, j)] + YM[ye(i - 1, j + 1)];  // into cell (i-1,j)
           const real yr = YP[ye(i, j)] + YM[ye(i, j + 1)];          // into cell (i,j)
           if (CAP)
-            Fn[xe(i, j)] -= half_dt * (sp * yl / kap(i - 1, j) + sm * yr / kap(i, j));
+            Fn[xe(i, j)] -= half_dt * (sp * yl * ik(i - 1, j) + sm * yr * ik(i, j));
           else
             Fn[xe(i, j)] -= half_nu * (sp * yl + sm * yr);
         } else {  // y-edges j in [0,MX], interior columns
@@ -322,7 +322,7 @@ __global__ void __launch_bounds__(NT, NT >= 512 ? (sizeof(real) == 4 ? 3 : 2)
           const real xb = XP[xe(i, j - 1)] + XM[xe(i + 1, j - 1)];  // into cell (i,j-1)
           const real xt = XP[xe(i, j)] + XM[xe(i + 1, j)];          // into cell (i,j)
           if (CAP)
-            Gn[ye(i, j)] -= half_dt * (sp * xb / kap(i, j - 1) + sm * xt / kap(i, j));
+            Gn[ye(i, j)] -= half_dt * (sp * xb * ik(i, j - 1) + sm * xt * ik(i, j));
           else
             Gn[ye(i, j)] -= half_nu * (sp * xb + sm * xt);
         }
@@ -340,7 +340,7 @@ __global__ void __launch_bounds__(NT, NT >= 512 ? (sizeof(real) == 4 ? 3 : 2)
       const int i = k % MX, j = k / MX;
       real v;
       if (CAP)
-        v = q(i, j) - dt / kap(i, j) *
+        v = q(i, j) - dt * ik(i, j) *
                           ((Fn[xe(i + 1, j)] - Fn[xe(i, j)]) + (Gn[ye(i, j + 1)] - Gn[ye(i, j)]));
       else
         v = q(i, j) - nu * (Fn[xe(i + 1, j)] - Fn[xe(i, j)]) -
@@ -353,7 +353,7 @@ __global__ void __launch_bounds__(NT, NT >= 512 ? (sizeof(real) == 4 ? 3 : 2)
 
 template <typename real, int MX, bool CAP>
 constexpr size_t staged_smem() {
-  return sizeof(double) * (size_t)(CAP ? metric_stride(MX + 4) : 0) +
+  return sizeof(real) * (size_t)(CAP ? umetric_stride(MX + 4) : 0) +
          sizeof(real) * (size_t)((MX + 4) * (MX + 4) + 6 * (MX + 1) * (MX + 2) + 4 * (MX + 3));
 }
 

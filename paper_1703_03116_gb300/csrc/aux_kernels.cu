@@ -85,7 +85,7 @@ __global__ void patch_sum_kernel(DevForest<real> D, double* sums) {
     const real* Q = D.buf[D.cur[pm.level]] + (size_t)p * S * S;
     double s = 0.0;
     if (D.metric) {  // mapped grid: sum of kappa q
-      const double* K = D.metric + (size_t)p * metric_stride(S);
+      const double* K = D.metric + (size_t)p * S * S;
       for (int k = threadIdx.x; k < mx * mx; k += blockDim.x) {
         const int o = (k / mx + 2) * S + k % mx + 2;
         s += K[o] * (double)Q[o];
@@ -238,7 +238,7 @@ __global__ void pack_capacity_kernel(DevForest<real> D, const int* api_to_dev, d
     const int k = (int)(g / (mx * mx)), r = (int)(g % (mx * mx));
     const int p = api_to_dev[k];
     if (D.metric) {
-      out[g] = D.metric[(size_t)p * metric_stride(S) + (r / mx + 2) * S + r % mx + 2];
+      out[g] = D.metric[(size_t)p * S * S + (r / mx + 2) * S + r % mx + 2];
     } else {
       const double h = ldexp(1.0, -D.meta[p].level) / mx;
       out[g] = h * h;
@@ -310,7 +310,7 @@ __global__ void remap_kernel(DevForest<real> Old, DevForest<real> New, const Rem
         const real* C = Old.buf[Old.cur[Old.meta[s].level]] + (size_t)s * S * S;
         const int fi = 2 * i - cx * mx + 2, fj = 2 * j - cy * mx + 2;
         if (Old.metric) {  // mapped grid: area-weighted, as the ghost average
-          const double* K = Old.metric + (size_t)s * metric_stride(S);
+          const double* K = Old.metric + (size_t)s * S * S;
           const double k0 = K[fj * S + fi], k1 = K[fj * S + fi + 1];
           const double k2 = K[(fj + 1) * S + fi], k3 = K[(fj + 1) * S + fi + 1];
           v = real((((k0 * double(C[fj * S + fi]) + k1 * double(C[fj * S + fi + 1])) +
@@ -400,7 +400,7 @@ __global__ void reflux_pairs_kernel(DevForest<real> D, int p0, int p1,
   if (p >= p1) return;  // whole warps leave together
   const int S = D.S;
   real* Q = D.buf[D.cur[D.meta[p].level]] + (size_t)p * S * S;
-  const double* K = D.metric + (size_t)p * metric_stride(S);
+  const double* K = D.metric + (size_t)p * S * S;
   for (int dir = 0; dir < 4; ++dir) {
     if (lane < MX) {
       const int* e = pairs + (((size_t)p * 4 + dir) * MX + lane) * 5;

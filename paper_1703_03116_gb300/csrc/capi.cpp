@@ -242,8 +242,9 @@ struct fc_forest {
   size_t trig_bytes = 0;
   size_t trig_off[kMaxLevel + 1] = {};  // in values
   int trig_len[kMaxLevel + 1] = {};     // 0: not held
-  double* d_metric = nullptr;             // cubed sphere: FP64 metric blocks per patch
-  double* d_corner = nullptr;             // deformational flow: grid corners per patch
+  double* d_metric = nullptr;             // cubed sphere: FP64 cell areas per patch
+  void* d_umetric = nullptr;              // and the update's block in the field's precision
+  double* d_coef = nullptr;               // deformational flow: edge coefficients per patch
   void* lam[2] = {nullptr, nullptr};      // adjoint tiles (patch-store layout), lazily allocated
   void* madj[3] = {nullptr, nullptr, nullptr};  // multirate adjoint: current, previous, qT tiles
   void* mio = nullptr;                    // multirate adjoint: lam in field layout (graph input)
@@ -425,7 +426,8 @@ void free_device(fc_forest* F) {
   for (auto& t : F->tapes) dfree(t.pool);
   F->tapes.clear();
   dfree(F->d_metric);
-  dfree(F->d_corner);
+  dfree(F->d_umetric);
+  dfree(F->d_coef);
   dfree(F->d_halo);
   dfree(F->d_pairs);
 }
@@ -433,21 +435,24 @@ void free_device(fc_forest* F) {
 // cubed sphere: (re)compute the metric blocks of the current layout for the
 // rotation vector times the velocity scale (synchronous); after a regrid the
 // kept patches copy theirs from the old layout (rm, old: device).  The
-// deformational flow keeps every patch's grid corners instead of fixed edge
-// fluxes (its fluxes are refreshed per substep): all patches are computed.
+// deformational flow keeps every patch's edge coefficients instead of fixed
+// edge fluxes (its fluxes are refreshed per substep): all patches are
+// computed.
 fc_status update_metrics(fc_forest* F, const RemapEntry* rm = nullptr,
-                         const double* old = nullptr) {
+                         const fc_forest* old = nullptr) {
   const HostForest& H = F->host;
   if (H.desc.domain != FC_DOMAIN_SPHERE) return FC_OK;
   const int n = H.npatch();
   const int S = H.desc.mx + 2 * kMbc;
   const bool deform = H.desc.vel_kind == FC_VEL_DEFORM;
   dfree(F->d_metric);
-  dfree(F->d_corner);
-  if (dmalloc(&F->d_metric, (size_t)n * metric_stride(S)) != cudaSuccess)
+  dfree(F->d_umetric);
+  dfree(F->d_coef);
+  if (dmalloc(&F->d_metric, (size_t)n * S * S) != cudaSuccess ||
+      dmalloc_bytes(&F->d_umetric, (size_t)n * umetric_stride(S) * F->esize) != cudaSuccess)
     return fail(FC_ERR_OOM, "metric allocation failed");
-  if (deform && dmalloc(&F->d_corner, (size_t)n * 3 * (S + 1) * (S + 1)) != cudaSuccess)
-    return fail(FC_ERR_OOM, "corner allocation failed");
+  if (deform && dmalloc(&F->d_coef, (size_t)n * coef_stride(S)) != cudaSuccess)
+    return fail(FC_ERR_OOM, "edge coefficient allocation failed");
   double w[3] = {F->vel_scale * H.desc.vel[0], F->vel_scale * H.desc.vel[1],
                  F->vel_scale * H.desc.vel[2]};
   if (deform) {
@@ -455,8 +460,18 @@ fc_status update_metrics(fc_forest* F, const RemapEntry* rm = nullptr,
     rm = nullptr;
     old = nullptr;
   }
-  FC_CUDA(launch_sphere_metrics(F->d_meta, n, H.desc.mx, w, F->d_metric, rm, old, F->d_corner,
-                                g_alloc_stream));
+  if (F->esize == 4)
+    FC_CUDA(launch_sphere_metrics(F->d_meta, n, H.desc.mx, w, F->d_metric,
+                                  static_cast<float*>(F->d_umetric), rm,
+                                  old ? old->d_metric : nullptr,
+                                  old ? static_cast<const float*>(old->d_umetric) : nullptr,
+                                  F->d_coef, g_alloc_stream));
+  else
+    FC_CUDA(launch_sphere_metrics(F->d_meta, n, H.desc.mx, w, F->d_metric,
+                                  static_cast<double*>(F->d_umetric), rm,
+                                  old ? old->d_metric : nullptr,
+                                  old ? static_cast<const double*>(old->d_umetric) : nullptr,
+                                  F->d_coef, g_alloc_stream));
   return FC_OK;
 }
 
@@ -497,8 +512,12 @@ fc_status deform_fluxes(fc_forest* F, int p0, int p1, const AdvArgs& a, cudaStre
   const fc_forest_desc& d = F->host.desc;
   if (d.vel_kind != FC_VEL_DEFORM || p1 <= p0) return FC_OK;
   const double kc = d.vel[0] * F->vel_scale, rot = 2.0 * M_PI / d.vel[2] * F->vel_scale;
-  FC_CUDA(launch_deform_fluxes(p0, p1, d.mx, F->d_corner, F->d_metric, kc, d.vel[1], rot,
-                               a.t_half, a.t0_dev, a.t_off, s));
+  if (F->esize == 4)
+    FC_CUDA(launch_deform_fluxes(p0, p1, d.mx, F->d_coef, static_cast<float*>(F->d_umetric), kc,
+                                 d.vel[1], rot, a.t_half, a.t0_dev, a.t_off, s));
+  else
+    FC_CUDA(launch_deform_fluxes(p0, p1, d.mx, F->d_coef, static_cast<double*>(F->d_umetric), kc,
+                                 d.vel[1], rot, a.t_half, a.t0_dev, a.t_off, s));
   return FC_OK;
 }
 
@@ -630,6 +649,7 @@ DevForest<real> dev(const fc_forest* F) {
   D.meta = F->d_meta;
   D.nbr = F->d_nbr;
   D.metric = F->d_metric;
+  D.umetric = static_cast<const real*>(F->d_umetric);
   D.buf[0] = static_cast<real*>(F->buf[0]);
   D.buf[1] = static_cast<real*>(F->buf[1]);
   D.qT = static_cast<real*>(F->qT);
@@ -754,8 +774,9 @@ double ghost_bytes(const fc_forest* F) {
 double advance_bytes(const fc_forest* F, int n) {
   const double mx = F->host.desc.mx;
   // read the patch with its ghosts, write the interior; a mapped grid also
-  // reads its FP64 metric block
-  const double metric = F->d_metric ? 8.0 * metric_stride(F->host.desc.mx + 2 * kMbc) : 0.0;
+  // reads its metric block
+  const double metric =
+      F->d_metric ? (double)F->esize * umetric_stride(F->host.desc.mx + 2 * kMbc) : 0.0;
   return (double)n * (((mx + 4) * (mx + 4) + mx * mx) * (double)F->esize + metric);
 }
 
@@ -1074,8 +1095,8 @@ fc_status fc_forest_info(const fc_forest* F, fc_info* out) {
   size_t bytes = 4 * store;  // two state buffers, the time-interpolated tiles, the stage
   if (F->bflux) bytes += n * 2 * 4 * H.desc.mx * F->esize;
   bytes += sizeof(NbrEntry) * n * 8 + sizeof(PatchMeta) * n + 3 * sizeof(double) * n;
-  if (F->d_metric) bytes += sizeof(double) * n * metric_stride((int)S);
-  if (F->d_corner) bytes += sizeof(double) * n * 3 * (S + 1) * (S + 1);
+  if (F->d_metric) bytes += n * (sizeof(double) * S * S + F->esize * umetric_stride((int)S));
+  if (F->d_coef) bytes += sizeof(double) * n * coef_stride((int)S);
   for (void* b : F->lam) bytes += b ? store : 0;
   for (void* b : F->madj) bytes += b ? store : 0;
   bytes += F->trig_bytes;
@@ -2346,7 +2367,7 @@ fc_status fc_tag_regrid(fc_forest* F, double tau_refine, double tau_coarsen,
                                   cudaMemcpyHostToDevice, s);
   if (e != cudaSuccess) return abandon(cuda_fail(e, "remap list copy"));
   if (F->d_metric) {  // the new layout's metrics: kept patches copy theirs
-    st = update_metrics(G, G->d_remap, F->d_metric);
+    st = update_metrics(G, G->d_remap, F);
     if (st != FC_OK) return abandon(st);
   }
   {
@@ -2391,7 +2412,8 @@ fc_status fc_tag_regrid(fc_forest* F, double tau_refine, double tau_coarsen,
   F->d_err = G->d_err;
   F->d_t0 = G->d_t0;
   F->d_metric = G->d_metric;
-  F->d_corner = G->d_corner;
+  F->d_umetric = G->d_umetric;
+  F->d_coef = G->d_coef;
   F->d_pairs = G->d_pairs;
   std::memcpy(F->pair_level, G->pair_level, sizeof F->pair_level);
   for (int l = 0; l <= kMaxLevel; ++l) F->cur[l] = 0;

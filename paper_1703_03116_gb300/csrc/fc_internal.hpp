@@ -391,12 +391,17 @@ void sort_leaves(std::vector<Leaf>* v);
 
 // ---------------------------------------------------------------- device side
 
-// Cubed-sphere metric block of one patch, FP64 over the extended index range
-// (cells -2..mx+1): capacity kappa[S*S] (spherical cell area), then the
-// volume flux of the velocity field through every x-edge, phix[S*(S+1)]
-// (edge i-1/2 of row j at j*(S+1) + i, shifted by 2), then through every
-// y-edge, phiy[(S+1)*S] (edge j-1/2 of column i at j*S + i, shifted by 2).
-__host__ __device__ constexpr int metric_stride(int S) { return S * S + 2 * S * (S + 1); }
+// Cubed-sphere metrics of one patch over the extended index range (cells
+// -2..mx+1): the capacities kappa[S*S] (spherical cell areas) in FP64, for
+// averages, masses and corrections; and the update's block in the field's
+// precision, formed from the FP64 values: 1 / kappa[S*S], the volume flux
+// of the velocity field through every x-edge, phix[S*(S+1)] (edge i-1/2 of
+// row j at j*(S+1) + i, shifted by 2), then through every y-edge,
+// phiy[(S+1)*S] (edge j-1/2 of column i at j*S + i, shifted by 2).
+__host__ __device__ constexpr int umetric_stride(int S) { return S * S + 2 * S * (S + 1); }
+// The deformational flow's four time-independent coefficients per edge (FP64,
+// planes over the x-edges, then the y-edges).
+__host__ __device__ constexpr int coef_stride(int S) { return 4 * 2 * S * (S + 1); }
 
 // Cubed sphere (FC_DOMAIN_SPHERE): block b is the face of the cube [-1,1]^3
 // with outward normal n; its block coordinates (x, y) in [0,1]^2 sit at
@@ -417,7 +422,8 @@ template <typename real>
 struct DevForest {
   int mx, S, npatch, domain;
   int napi;  // leaves in the field layout (get/set, mass): npatch, or the owned ones
-  const double* metric;  // cubed sphere: metric_stride(S) doubles per patch; else null
+  const double* metric;  // cubed sphere: kappa, S*S doubles per patch; else null
+  const real* umetric;   // and the update's block, umetric_stride(S) per patch
   const PatchMeta* meta;
   const NbrEntry* nbr;
   real* buf[2];
@@ -613,23 +619,25 @@ uint64_t& launch_counter();
 cudaError_t launch_coarse_sources(NbrEntry* nbr, const PatchMeta* meta, int n, int mx, int walls,
                                   cudaStream_t s);
 
-// Cubed-sphere metric blocks of patches [0, npatch) for the solid-body
-// rotation omega (already scaled): equiangular gnomonic mapping of each
-// face, capacities from two spherical triangles per cell, edge fluxes from
-// the stream function -omega . X (Sec. 5.3 mapped grids).  With a remap list
-// (rm, device, one entry per patch), RM_COPY patches copy their block from
-// old_metric (same omega) instead.
-// With corner_out set, every patch's grid corners (three planes of
-// (mx+5)^2 unit-sphere components) are also written there.
+// Cubed-sphere metrics of patches [0, npatch) for the solid-body rotation
+// omega (already scaled): equiangular gnomonic mapping of each face,
+// capacities from two spherical triangles per cell, edge fluxes from the
+// stream function -omega . X (Sec. 5.3 mapped grids).  With a remap list (rm,
+// device, one entry per patch), RM_COPY patches copy their blocks from the old
+// layout's (same omega) instead.  With coef set, every patch's edge
+// coefficients of the deformational flow are written there.
+template <typename real>
 cudaError_t launch_sphere_metrics(const PatchMeta* meta, int npatch, int mx, const double* omega,
-                                  double* metric, const RemapEntry* rm, const double* old_metric,
-                                  double* corner_out, cudaStream_t s);
+                                  double* metric, real* umetric, const RemapEntry* rm,
+                                  const double* old_metric, const real* old_umetric, double* coef,
+                                  cudaStream_t s);
 
 // The deformational flow (FC_VEL_DEFORM): the edge volume fluxes of the
-// metric blocks of patches [p0, p1) for time t (t0_dev ? *t0_dev + t_off :
-// t_half) from their kept corners; coefficients already scaled:
-// kc = k * scale, rot = 2 pi / T_f * scale.
-cudaError_t launch_deform_fluxes(int p0, int p1, int mx, const double* corner, double* metric,
+// update's blocks of patches [p0, p1) for time t (t0_dev ? *t0_dev + t_off :
+// t_half) from their edge coefficients; kc = k * scale, rot = 2 pi / T_f *
+// scale.
+template <typename real>
+cudaError_t launch_deform_fluxes(int p0, int p1, int mx, const double* coef, real* umetric,
                                  double kc, double T, double rot, double t_half,
                                  const double* t0_dev, double t_off, cudaStream_t s);
 

@@ -87,7 +87,7 @@ __device__ __forceinline__ bool copy_or_average_entry(const DevForest<real>& D, 
   for (int q = 0; q < 4; ++q)
     s[q] = src_interior(D, tlevel, alpha, n, e.lev, lx + (q & 1), ly + (q >> 1));
   if (D.metric) {  // mapped grid: weighted by the fine cells' areas
-    const double* K = D.metric + (size_t)n * metric_stride(D.S) + (ly + kMbc) * D.S + lx + kMbc;
+    const double* K = D.metric + (size_t)n * D.S * D.S + (ly + kMbc) * D.S + lx + kMbc;
     const double k0 = K[0], k1 = K[1], k2 = K[D.S], k3 = K[D.S + 1];
     v = real((((k0 * double(s[0]) + k1 * double(s[1])) + k2 * double(s[2])) + k3 * double(s[3])) /
              (((k0 + k1) + k2) + k3));
@@ -195,7 +195,7 @@ __device__ __forceinline__ real fill_rule(const DevForest<real>& D, int tlevel, 
   for (int q = 0; q < 4; ++q)
     s[q] = src_interior(D, tlevel, alpha, n, tlevel + 1, lx + (q & 1), ly + (q >> 1));
   if (D.metric) {
-    const double* K = D.metric + (size_t)n * metric_stride(D.S) + (ly + kMbc) * D.S + lx + kMbc;
+    const double* K = D.metric + (size_t)n * D.S * D.S + (ly + kMbc) * D.S + lx + kMbc;
     const double k0 = K[0], k1 = K[1], k2 = K[D.S], k3 = K[D.S + 1];
     return real((((k0 * double(s[0]) + k1 * double(s[1])) + k2 * double(s[2])) +
                  k3 * double(s[3])) /
