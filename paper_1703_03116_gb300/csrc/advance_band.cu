@@ -24,7 +24,7 @@
 #include <atomic>
 #include <cstdint>
 
-#include "ghost_gather.cuh"
+#include "ghost_ring.cuh"
 #include "walk_edge.cuh"
 
 namespace fc {
@@ -72,13 +72,15 @@ __global__ void __launch_bounds__(band_threads<real, MX, R>(), band_min_blocks<r
   constexpr int NG = num_ghosts<MX>();
   constexpr unsigned kAll = 0xffffffffu;
   constexpr uint32_t bytes = sizeof(real) * S * S;
-  static_assert(NT >= 4 * NV, "a thread per table entry");
+  static_assert(NT >= 4 * NV && NT >= ring_threads<MX>(), "a thread per table entry and task");
   static_assert(MX % R == 0 && NW % 32 == 0 && NT % 32 == 0, "bands of R rows, whole warps");
   __shared__ __align__(128) real Q[S * S];
   __shared__ __align__(8) uint64_t bar;
   __shared__ real ucoef_s;
-  __shared__ real ring[NG];    // ghost values gathered while the tile loads
-  __shared__ bool ring_w[NG];
+  // ghost values gathered while the tile loads: the sphere's whole ring, else
+  // the cells beyond coarse patches' interiors (ghost_ring.cuh)
+  __shared__ real ring[CAP ? NG : 24];
+  __shared__ bool ring_w[CAP ? NG : 1];
   // streamfunction tables over corner nodes k = 0..MX+2 (index k - 1):
   // Sx = sin^2(pi x_node), Tx = sin(pi (x_{c} + x_{c+1})) of column c = k - 1
   __shared__ real Sx[NV], Sy[NV], Tx[NV], Ty[NV];
@@ -112,8 +114,9 @@ __global__ void __launch_bounds__(band_threads<real, MX, R>(), band_min_blocks<r
   uint32_t parity = 0;
   for (int p = p0 + blockIdx.x; p < p1; p += gridDim.x, parity ^= 1) {
     const PatchMeta pm = D.meta[p];
-    const real* src = D.buf[D.cur[pm.level]] + (size_t)p * S * S;
-    real* dst = D.buf[D.cur[pm.level] ^ 1] + (size_t)p * S * S;
+    // (the launch's level: the copy does not wait for the patch's record)
+    const real* src = D.buf[D.cur[a.level]] + (size_t)p * S * S;
+    real* dst = D.buf[D.cur[a.level] ^ 1] + (size_t)p * S * S;
     if (tid == 0) {
       fence_proxy_async();
       mbar_expect_tx(&bar, bytes + mbytes);
@@ -130,8 +133,9 @@ __global__ void __launch_bounds__(band_threads<real, MX, R>(), band_min_blocks<r
     // than the read by 1%) now, stored after the gather, whose reads are not
     // to wait for this one's
     real tv = real(0);
-    if (SWIRL && tid < 4 * NV) {
-      const int tb = tid / NV, c = tid % NV;
+    const int tk = NT - 1 - tid;  // (the first threads start the gather's longest reads)
+    if (SWIRL && tk < 4 * NV) {
+      const int tb = tk / NV, c = tk % NV;
       const int z = (tb & 1 ? pm.y : pm.x) * MX + c - 1;
       if (sizeof(real) == 8 && tab) {
         tv = tab[(tb < 2 ? 0 : a.trig_len) + z + 1];
@@ -142,14 +146,20 @@ __global__ void __launch_bounds__(band_threads<real, MX, R>(), band_min_blocks<r
         tv = sinpi_r(real(2 * z + 1) * h);
       }
     }
-    // each gathering thread reads the entry of its ghost's region from the
-    // table itself: no staging pass, no barrier before the gather
-    if (a.gather)
-      gather_ring<real, MX>(
-          D, [&](int r) { return D.nbr[(size_t)p * 8 + r]; }, p, pm, a.tlevel, ac.alpha,
-          a.direct != 0, ring, ring_w, tid, NT, static_cast<real*>(a.keep_t), a.keep_t_p0);
-    if (SWIRL && tid < 4 * NV) {
-      const int tb = tid / NV, c = tid % NV;
+    // each gathering thread reads its region's entry from the table itself: no
+    // staging pass, no barrier before the gather
+    RingPart<real> part;
+    if (a.gather) {
+      if (CAP)
+        gather_ring<real, MX>(
+            D, [&](int r) { return D.nbr[(size_t)p * 8 + r]; }, p, pm, a.tlevel, ac.alpha,
+            a.direct != 0, ring, ring_w, tid, NT, static_cast<real*>(a.keep_t), a.keep_t_p0);
+      else
+        part = ring_read<real, MX>(D, p, pm, a.level, a.tlevel, ac.alpha, a.direct != 0, ring,
+                                   tid, static_cast<real*>(a.keep_t), a.keep_t_p0);
+    }
+    if (SWIRL && tk < 4 * NV) {
+      const int tb = tk / NV, c = tk % NV;
       (tb == 0 ? Sx : tb == 1 ? Sy : tb == 2 ? Tx : Ty)[c] = tv;
     }
     // thread 0 observes the copy's completion (bounded), the others after the
@@ -162,9 +172,16 @@ __global__ void __launch_bounds__(band_threads<real, MX, R>(), band_min_blocks<r
     }
     if (tid != 0) mbar_wait(&bar, parity, kWaitLimit);
     if (a.gather) {
-      store_ring<real, MX>(Q, ring, ring_w, tid, NT);
+      if (CAP)
+        store_ring<real, MX>(Q, ring, ring_w, tid, NT);
+      else
+        ring_store<real, MX>(D, part, a.level, a.tlevel, ac.alpha, a.direct != 0, Q, ring, tid,
+                             static_cast<real*>(a.keep_t), a.keep_t_p0, p);
       __syncthreads();
-      if (D.domain == FC_DOMAIN_WALLS) {
+      // (uniform over the CTA: does the patch touch a wall?)
+      const int last_q = (1 << a.level) - 1;
+      if (D.domain == FC_DOMAIN_WALLS &&
+          (pm.x == 0 || pm.y == 0 || pm.x == last_q || pm.y == last_q)) {
         wall_bc<real, MX>(pm, Q, tid, NT);
         __syncthreads();
       }
