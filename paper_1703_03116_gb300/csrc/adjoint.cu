@@ -33,6 +33,7 @@
 // The adjoint tiles use the patch-store layout ((mx+4)^2 per patch).
 #include <atomic>
 
+#include "adjoint_fp64.cuh"
 #include "ghost_gather.cuh"
 
 namespace fc {
@@ -501,6 +502,18 @@ struct AdjGhosts {
   int coarse_p0, tlevel;
 };
 
+// Per-level scalars of a launch, in the field's precision (one launch covers
+// every level of a global step): cell width, dt/h, a constant velocity, and
+// the swirl coefficient's factor; in FP64 the velocities are half Courant
+// numbers (adjoint_fp64.cuh).
+template <typename real>
+struct AdjLevels {
+  real h[kMaxLevel + 1], nu[kMaxLevel + 1], hn[kMaxLevel + 1];
+  real cu[kMaxLevel + 1], cv[kMaxLevel + 1], usc[kMaxLevel + 1];
+  double period, t_half, t_off;
+  const double* t0_dev;
+};
+
 // The forward tile of patch p is read from the store, or from
 // tiles + (p - tiles_p0) tiles when `tiles` is given (kept copies).  acc
 // (multirate accumulators, with g): lam_in's tile is cleared once read, the
@@ -511,7 +524,7 @@ struct AdjGhosts {
 // patches run in one wave)
 template <typename real, int MX, int R, int NT, int NS>
 __global__ void __launch_bounds__(NT, sizeof(real) == 4 && NT >= 384 ? 2 : 1)
-    adj_advance_kernel(DevForest<real> D, AdvArgs a,
+    adj_advance_kernel(DevForest<real> D, AdjLevels<real> a,
                                                          real* lam_in, real* lam_out,
                                                          double* dscale, double dfac, int p0,
                                                          int p1, const real* tiles, int tiles_p0,
@@ -537,15 +550,7 @@ __global__ void __launch_bounds__(NT, sizeof(real) == 4 && NT >= 384 ? 2 : 1)
   __shared__ NbrStage st;  // acc: the patch's neighbour entries
   const int order = D.order, limiter = D.limiter, transverse = D.transverse;
   const bool swirl = D.vel_kind == FC_VEL_SWIRL;
-  const real cu = real(D.vel[0]), cv = real(D.vel[1]);
-  const real nu = real(a.nu), hn = real(0.5 * a.nu), h = real(a.h);
-  // the swirl coefficient, by the last thread while the first patch's data
-  // load (graph replay: the time is on the device); read after the barrier
-  if (threadIdx.x == NT - 1 && swirl) {
-    const double t = a.t0_dev ? *a.t0_dev + a.t_off : a.t_half;
-    ucoef_s = cospi_ratio<real>(t, a.period) * real(a.sfac);
-  }
-  real ucoef = real(0);
+  constexpr bool kHalf = sizeof(real) == 8;
   // velocity-scale derivative: per-thread partial sums in the field's
   // precision (FP64 arithmetic is scarce on this GPU), FP64 from the block
   // reduction on
@@ -553,6 +558,14 @@ __global__ void __launch_bounds__(NT, sizeof(real) == 4 && NT >= 384 ? 2 : 1)
 
   for (int p = p0 + blockIdx.x; p < p1; p += gridDim.x) {
     const PatchMeta pm = D.meta[p];
+    const real h = a.h[pm.level], nu = a.nu[pm.level], hn = a.hn[pm.level];
+    const real cu = a.cu[pm.level], cv = a.cv[pm.level];
+    // the swirl coefficient, by the last thread while the data load (graph
+    // replay: the time is on the device); read after the barrier
+    if (threadIdx.x == NT - 1 && swirl) {
+      const double t = a.t0_dev ? *a.t0_dev + a.t_off : a.t_half;
+      ucoef_s = cospi_ratio<real>(t, a.period) * a.usc[pm.level];
+    }
     const real* src = tiles ? tiles + (size_t)(p - tiles_p0) * S * S
                             : D.buf[D.cur[pm.level]] + (size_t)p * S * S;
     real* lin = lam_in + (size_t)p * S * S;
@@ -595,39 +608,63 @@ __global__ void __launch_bounds__(NT, sizeof(real) == 4 && NT >= 384 ? 2 : 1)
     for (int u = 0; u < NL; ++u) {
       const int k = (int)threadIdx.x + u * NT;
       if (k < MX * MX) {
-        LN[k] = vl[u];
+        LN[k] = kHalf ? vl[u] + vl[u] : vl[u];
         if (acc) lin[(k / MX + 2) * S + (k % MX) + 2] = real(0);  // consumed: next state from zero
       }
     }
     __syncthreads();
-    ucoef = swirl ? ucoef_s : real(0);
+    const real ucoef = swirl ? ucoef_s : real(0);
     auto q = [&](int i, int j) -> real { return Q[(j + 2) * S + (i + 2)]; };
     auto lq = [&](int i, int j) -> real* { return &LQ[(j + 2) * S + (i + 2)]; };
     auto uvel = [&](int i, int j) -> real { return swirl ? ucoef * Sx[i + 1] * Ty[j + 1] : cu; };
     auto vvel = [&](int i, int j) -> real { return swirl ? -ucoef * Sy[j + 1] * Tx[i + 1] : cv; };
     // the side quantities the band walk reads, then the walk (rows of
     // bands) and the edges beside it (columns MX and -1)
-    for (int k = threadIdx.x; k < 2 * MX + 3; k += NT) {
-      if (k < MX + 2) {
-        const int j = k - 1;
-        XMe[k] = edge_fw(order, limiter, transverse, uvel(MX, j), q(MX - 2, j), q(MX - 1, j),
-                         q(MX, j), q(MX + 1, j), nu)
-                     .M;
-      } else {
-        const int j = k - (MX + 2);
-        const EdgeFw<real> e = edge_fw(order, limiter, transverse, vvel(-1, j), q(-1, j - 2),
-                                       q(-1, j - 1), q(-1, j), q(-1, j + 1), nu);
-        YPm[j] = e.P;
-        YMm[j] = e.M;
+    if constexpr (kHalf) {
+      const half::AdjScheme sc{order > 1, limiter != 0, transverse > 0, transverse > 1};
+      for (int k = threadIdx.x; k < 2 * MX + 3; k += NT) {
+        if (k < MX + 2) {
+          const int j = k - 1;
+          XMe[k] = half::edge_fw(sc, uvel(MX, j), q(MX - 2, j), q(MX - 1, j), q(MX, j),
+                                 q(MX + 1, j))
+                       .M;
+        } else {
+          const int j = k - (MX + 2);
+          const half::EdgeFw<real> e = half::edge_fw(sc, vvel(-1, j), q(-1, j - 2), q(-1, j - 1),
+                                                     q(-1, j), q(-1, j + 1));
+          YPm[j] = e.nP;
+          YMm[j] = e.M;
+        }
       }
+      __syncthreads();
+      if (threadIdx.x < NW)
+        dsum += half::band_transpose<real, MX, R>(Q, LQ, LN, XMe, YPm, YMm, sc, uvel, vvel,
+                                                  threadIdx.x);
+      else
+        dsum += half::side_transpose<real, MX>(Q, LQ, LN, sc, uvel, vvel, threadIdx.x - NW, NS);
+    } else {
+      for (int k = threadIdx.x; k < 2 * MX + 3; k += NT) {
+        if (k < MX + 2) {
+          const int j = k - 1;
+          XMe[k] = edge_fw(order, limiter, transverse, uvel(MX, j), q(MX - 2, j), q(MX - 1, j),
+                           q(MX, j), q(MX + 1, j), nu)
+                       .M;
+        } else {
+          const int j = k - (MX + 2);
+          const EdgeFw<real> e = edge_fw(order, limiter, transverse, vvel(-1, j), q(-1, j - 2),
+                                         q(-1, j - 1), q(-1, j), q(-1, j + 1), nu);
+          YPm[j] = e.P;
+          YMm[j] = e.M;
+        }
+      }
+      __syncthreads();
+      if (threadIdx.x < NW)
+        dsum += band_transpose<real, MX, R>(Q, LQ, LN, XMe, YPm, YMm, order, limiter, transverse, nu,
+                                            hn, uvel, vvel, threadIdx.x);
+      else
+        dsum += side_transpose<real, MX>(Q, LQ, LN, order, limiter, transverse, nu, hn, uvel, vvel,
+                                         threadIdx.x - NW, NS);
     }
-    __syncthreads();
-    if (threadIdx.x < NW)
-      dsum += band_transpose<real, MX, R>(Q, LQ, LN, XMe, YPm, YMm, order, limiter, transverse, nu,
-                                          hn, uvel, vvel, threadIdx.x);
-    else
-      dsum += side_transpose<real, MX>(Q, LQ, LN, order, limiter, transverse, nu, hn, uvel, vvel,
-                                       threadIdx.x - NW, NS);
     __syncthreads();
     // transpose of the second wall-BC pass
     if (D.domain == FC_DOMAIN_WALLS) {
@@ -785,14 +822,28 @@ constexpr size_t adj_smem() {
 
 inline int grid_for(int n) { return n < 1 ? 1 : (n < 65535 * 8 ? n : 65535 * 8); }
 
-// transpose of the update of level L's patches [p0, p1) over (t, t + dt)
+// level L's scalars of a step dt
 template <typename real, int MX>
-cudaError_t adj_advance_level(const DevForest<real>& D, int L, int p0, int p1, double t, double dt,
-                              double period, double scale, double dfac, real* lam_in,
-                              real* lam_out, double* dscale, cudaStream_t s,
-                              const double* t0_dev = nullptr, const real* tiles = nullptr,
-                              int tiles_p0 = 0, int acc = 0,
-                              AdjGhosts<real> g = AdjGhosts<real>{}) {
+void adj_level(const DevForest<real>& D, int L, double dt, double scale, AdjLevels<real>* a) {
+  const double h = ldexp(1.0, -L) / MX, nu = dt / h;
+  const double unit = sizeof(real) == 8 ? 0.5 * nu : 1.0;
+  const double sfac = D.vel_kind == FC_VEL_SWIRL ? scale * sin(M_PI * h) / (M_PI * h) : 0.0;
+  a->h[L] = real(h);
+  a->nu[L] = real(nu);
+  a->hn[L] = real(0.5 * nu);
+  a->cu[L] = real(D.vel[0] * unit);
+  a->cv[L] = real(D.vel[1] * unit);
+  a->usc[L] = real(sfac * unit);
+}
+
+// transpose of the update of patches [p0, p1) over (t, t + dt); a: the
+// scalars of their levels
+template <typename real, int MX>
+cudaError_t adj_advance(const DevForest<real>& D, AdjLevels<real>& a, int p0, int p1, double t,
+                        double dt, double period, double dfac, real* lam_in, real* lam_out,
+                        double* dscale, cudaStream_t s, const double* t0_dev = nullptr,
+                        const real* tiles = nullptr, int tiles_p0 = 0, int acc = 0,
+                        AdjGhosts<real> g = AdjGhosts<real>{}) {
   // a whole CTA per patch whose warps walk bands of R rows (4 at mx = 32,
   // 2 below) while more warps transpose the side edges
   constexpr int R = MX == 32 ? 4 : 2;
@@ -808,16 +859,12 @@ cudaError_t adj_advance_level(const DevForest<real>& D, int L, int p0, int p1, d
     attr.store(true, std::memory_order_release);
   }
   if (p1 <= p0) return cudaSuccess;
-  AdvArgs al{};
-  al.h = ldexp(1.0, -L) / MX;
-  al.nu = dt / al.h;
-  al.period = period;
-  al.t_half = t + 0.5 * dt;
-  al.t_off = t + 0.5 * dt;  // with t0_dev: t is relative to the replayed step's start
-  al.t0_dev = t0_dev;
-  al.sfac = D.vel_kind == FC_VEL_SWIRL ? scale * sin(M_PI * al.h) / (M_PI * al.h) : 0.0;
+  a.period = period;
+  a.t_half = t + 0.5 * dt;
+  a.t_off = t + 0.5 * dt;  // with t0_dev: t is relative to the replayed step's start
+  a.t0_dev = t0_dev;
   adj_advance_kernel<real, MX, R, NT, NS><<<p1 - p0, NT, smem, s>>>(
-      D, al, lam_in, lam_out, dscale, dfac, p0, p1, tiles, tiles_p0, acc, g);
+      D, a, lam_in, lam_out, dscale, dfac, p0, p1, tiles, tiles_p0, acc, g);
   ++launch_counter();
   return cudaGetLastError();
 }
@@ -826,10 +873,13 @@ template <typename real, int MX>
 cudaError_t adjoint_mx(const DevForest<real>& D, const AdjArgs& g, const real* lam_in,
                        real* lam_out, double* dscale, cudaStream_t s) {
   // one launch per level (per-level h and dt/h); all read the pre-step state
+  AdjLevels<real> a{};
   for (int L = 0; L <= kMaxLevel; ++L) {
-    cudaError_t e = adj_advance_level<real, MX>(D, L, g.lev_start[L], g.lev_start[L + 1], g.t,
-                                                g.dt, g.period, g.scale, g.dscale_factor,
-                                                const_cast<real*>(lam_in), lam_out, dscale, s);
+    if (g.lev_start[L + 1] <= g.lev_start[L]) continue;
+    adj_level<real, MX>(D, L, g.dt, g.scale, &a);
+    cudaError_t e = adj_advance<real, MX>(D, a, g.lev_start[L], g.lev_start[L + 1], g.t, g.dt,
+                                          g.period, g.dscale_factor, const_cast<real*>(lam_in),
+                                          lam_out, dscale, s);
     if (e != cudaSuccess) return e;
   }
   if (g.ncoarse > 0) {
@@ -853,9 +903,11 @@ cudaError_t adjoint_sub_mx(const DevForest<real>& D, const AdjSubArgs& g, const 
   const int n = g.p1 - g.p0;
   if (n <= 0) return cudaSuccess;
   const real alpha = real(g.alpha);
-  cudaError_t e = adj_advance_level<real, MX>(
-      D, g.L, g.p0, g.p1, g.t, g.dt, g.period, g.scale, g.dscale_factor, c.lam_in, c.lam_out,
-      dscale, s, g.t0_dev, static_cast<const real*>(g.tiles), g.tiles_p0, 1,
+  AdjLevels<real> a{};
+  adj_level<real, MX>(D, g.L, g.dt, g.scale, &a);
+  cudaError_t e = adj_advance<real, MX>(
+      D, a, g.p0, g.p1, g.t, g.dt, g.period, g.dscale_factor, c.lam_in, c.lam_out, dscale, s,
+      g.t0_dev, static_cast<const real*>(g.tiles), g.tiles_p0, 1,
       AdjGhosts<real>{c.lam_fine, c.lamT, static_cast<const real*>(g.coarse), g.coarse_p0,
                       g.tlevel});
   if (e != cudaSuccess) return e;
