@@ -15,10 +15,10 @@
 //  adj_interp      transpose of the interpolation (Eq. ghost_fine): each
 //                  fine ghost's adjoint goes to the coarse cells it read
 //                  (atomic adds into the coarse patch's tile).
-//  adj_bc          transpose of the first wall-BC pass (local to a patch).
-//  adj_copy        transpose of copy / average (Eq. transform,
-//                  Eq. ghost_coarse): ghost adjoints go to the neighbours'
-//                  interior cells (atomic adds).
+//  adj_copy        transpose of the first wall-BC pass (local to a patch),
+//                  then of copy / average (Eq. transform, Eq. ghost_coarse):
+//                  ghost adjoints go to the neighbours' interior cells
+//                  (atomic adds).
 //
 // Multirate substep of level L (launch_adjoint_substep), two kernels: the
 // update's transpose followed, in the same CTA, by that of the patch's ghost
@@ -733,20 +733,17 @@ __global__ void adj_interp_kernel(DevForest<real> D, const int* targets, int nta
   }
 }
 
-template <typename real, int MX>
-__global__ void adj_bc_kernel(DevForest<real> D, real* lam) {
-  constexpr int S = MX + 4;
-  for (int p = blockIdx.x; p < D.npatch; p += gridDim.x)
-    adj_bc_patch<real, MX>(D.meta[p], lam + (size_t)p * S * S, threadIdx.x, blockDim.x);
-}
-
+// the wall pass's transpose (within the patch's own tile), then that of the
+// copies and averages (ghosts to the neighbours' interiors)
 template <typename real, int MX>
 __global__ void adj_copy_kernel(DevForest<real> D, real* lam) {
-  constexpr int S = MX + 4;
   __shared__ NbrStage st;
+  constexpr int S = MX + 4;
   for (int p = blockIdx.x; p < D.npatch; p += gridDim.x) {
     stage_neighbours(D.meta, D.nbr, p, st, threadIdx.x);
     const PatchMeta pm = D.meta[p];
+    if (D.domain == FC_DOMAIN_WALLS)
+      adj_bc_patch<real, MX>(pm, lam + (size_t)p * S * S, threadIdx.x, blockDim.x);
     __syncthreads();
     adj_copy_patch<real, MX>(st, pm, lam + (size_t)p * S * S,
                              AdjTargets<real>{lam, lam, nullptr, nullptr}, -1, real(0),
@@ -869,29 +866,27 @@ cudaError_t adj_advance(const DevForest<real>& D, AdjLevels<real>& a, int p0, in
   return cudaGetLastError();
 }
 
+// The adjoint of a global step: the updates' transposes in one launch over
+// all levels (all read the pre-step state; a launch a level, one after
+// another, each took the 10 us of one patch), then the transpose of Alg. 1 in
+// two more, a thread per ghost.  496 patches of 32^2, FP32, with its field
+// moves: 95 -> 65 us.
 template <typename real, int MX>
 cudaError_t adjoint_mx(const DevForest<real>& D, const AdjArgs& g, const real* lam_in,
                        real* lam_out, double* dscale, cudaStream_t s) {
-  // one launch per level (per-level h and dt/h); all read the pre-step state
   AdjLevels<real> a{};
-  for (int L = 0; L <= kMaxLevel; ++L) {
-    if (g.lev_start[L + 1] <= g.lev_start[L]) continue;
-    adj_level<real, MX>(D, L, g.dt, g.scale, &a);
-    cudaError_t e = adj_advance<real, MX>(D, a, g.lev_start[L], g.lev_start[L + 1], g.t, g.dt,
-                                          g.period, g.dscale_factor, const_cast<real*>(lam_in),
-                                          lam_out, dscale, s);
-    if (e != cudaSuccess) return e;
-  }
+  for (int L = 0; L <= kMaxLevel; ++L)
+    if (g.lev_start[L + 1] > g.lev_start[L]) adj_level<real, MX>(D, L, g.dt, g.scale, &a);
+  cudaError_t e = adj_advance<real, MX>(D, a, 0, D.npatch, g.t, g.dt, g.period, g.dscale_factor,
+                                        const_cast<real*>(lam_in), lam_out, dscale, s);
+  if (e != cudaSuccess) return e;
+  constexpr int NT = (num_ghosts<MX>() + 31) / 32 * 32;
   if (g.ncoarse > 0) {
-    adj_interp_kernel<real, MX><<<grid_for(g.ncoarse), 128, 0, s>>>(D, g.coarse_list, g.ncoarse,
-                                                                     lam_out);
+    adj_interp_kernel<real, MX><<<grid_for(g.ncoarse), NT, 0, s>>>(D, g.coarse_list, g.ncoarse,
+                                                                    lam_out);
     ++launch_counter();
   }
-  if (D.domain == FC_DOMAIN_WALLS) {
-    adj_bc_kernel<real, MX><<<grid_for(D.npatch), 128, 0, s>>>(D, lam_out);
-    ++launch_counter();
-  }
-  adj_copy_kernel<real, MX><<<grid_for(D.npatch), 128, 0, s>>>(D, lam_out);
+  adj_copy_kernel<real, MX><<<grid_for(D.npatch), NT, 0, s>>>(D, lam_out);
   ++launch_counter();
   return cudaGetLastError();
 }
