@@ -77,8 +77,8 @@ __global__ void __launch_bounds__(band_threads<real, MX, R>(), band_min_blocks<r
   __shared__ __align__(128) real Q[S * S];
   __shared__ __align__(8) uint64_t bar;
   __shared__ real ucoef_s;
-  // ghost values gathered while the tile loads: the sphere's whole ring, else
-  // the cells beyond coarse patches' interiors (ghost_ring.cuh)
+  // ghost values gathered while the tile loads: the whole ring, or the cells
+  // beyond coarse patches' interiors (ghost_ring.cuh)
   __shared__ real ring[CAP ? NG : 24];
   __shared__ bool ring_w[CAP ? NG : 1];
   // streamfunction tables over corner nodes k = 0..MX+2 (index k - 1):
@@ -149,13 +149,14 @@ __global__ void __launch_bounds__(band_threads<real, MX, R>(), band_min_blocks<r
     // each gathering thread reads its region's entry from the table itself: no
     // staging pass, no barrier before the gather
     RingPart<real> part;
+    const bool each = CAP && (pm.flags & 2);  // ghost by ghost: a neighbour's axes are turned
     if (a.gather) {
-      if (CAP)
+      if (each)
         gather_ring<real, MX>(
             D, [&](int r) { return D.nbr[(size_t)p * 8 + r]; }, p, pm, a.tlevel, ac.alpha,
             a.direct != 0, ring, ring_w, tid, NT, static_cast<real*>(a.keep_t), a.keep_t_p0);
       else
-        part = ring_read<real, MX>(D, p, pm, a.level, a.tlevel, ac.alpha, a.direct != 0, ring,
+        part = ring_read<real, MX, CAP>(D, p, pm, a.level, a.tlevel, ac.alpha, a.direct != 0, ring,
                                    tid, static_cast<real*>(a.keep_t), a.keep_t_p0);
     }
     if (SWIRL && tk < 4 * NV) {
@@ -172,10 +173,10 @@ __global__ void __launch_bounds__(band_threads<real, MX, R>(), band_min_blocks<r
     }
     if (tid != 0) mbar_wait(&bar, parity, kWaitLimit);
     if (a.gather) {
-      if (CAP)
+      if (each)
         store_ring<real, MX>(Q, ring, ring_w, tid, NT);
       else
-        ring_store<real, MX>(D, part, a.level, a.tlevel, ac.alpha, a.direct != 0, Q, ring, tid,
+        ring_store<real, MX, CAP>(D, part, a.level, a.tlevel, ac.alpha, a.direct != 0, Q, ring, tid,
                              static_cast<real*>(a.keep_t), a.keep_t_p0, p);
       __syncthreads();
       // (uniform over the CTA: does the patch touch a wall?)
@@ -185,7 +186,7 @@ __global__ void __launch_bounds__(band_threads<real, MX, R>(), band_min_blocks<r
         wall_bc<real, MX>(pm, Q, tid, NT);
         __syncthreads();
       }
-      if (CAP && D.domain == FC_DOMAIN_SPHERE) {  // corners beyond a cube vertex
+      if (each) {  // corners beyond a cube vertex
         corner3_fill_k<real, MX>([&](int r) { return D.nbr[(size_t)p * 8 + r].kind; }, Q, tid,
                                  NT);
         __syncthreads();

@@ -131,7 +131,9 @@ inline void parallel_chunks(int n, int min_per_piece, Fn fn) {
 }
 
 struct PatchMeta {
-  int level, x, y, block, forest, flags;  // flags bit 0: has a coarser neighbour
+  // flags bit 0: has a coarser neighbour; bit 1: a neighbour's axes are turned
+  // against this patch's, or a corner lies beyond a cube vertex
+  int level, x, y, block, forest, flags;
 };
 
 struct Leaf {

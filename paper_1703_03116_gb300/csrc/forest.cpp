@@ -584,6 +584,8 @@ std::string HostForest::neighbour_rows(int kb, int ke) {
         e.x1 = n1.x;
         e.y1 = n1.y;
       }
+      // (the updates' face-by-face gather is for neighbours of one orientation)
+      if (e.a != 0 || e.kind == NB_CORNER3) meta[p].flags |= 2;
       nbr[(size_t)p * 8 + dir] = e;
     }
   }

@@ -1,5 +1,7 @@
-// The ghost ring of one patch by a CTA, side by side (square domains, whose
-// neighbours keep orientation): the band update's gather.
+// The ghost ring of one patch by a CTA, side by side: the band update's
+// gather for patches whose neighbours keep orientation (every patch of a
+// square domain; on the cubed sphere those away from the cube's edges, the
+// others take the ring ghost by ghost).
 //
 // A launch of a few hundred patches waits for each patch's chain of dependent
 // reads and instructions, not for bandwidth.  Ghost by ghost, with each
@@ -10,7 +12,8 @@
 // interpolation needs beyond the coarse patch's interior are found by threads
 // of their own at the same time.  Measured (one GB300): the update of 248
 // patches of 32^2 in FP32 10.4 -> 7.2 us, a coarse step of the swirl forest
-// (496 patches, 16 finest substeps one after another) 0.124 -> 0.104 ms.
+// (496 patches, 16 finest substeps one after another) 0.124 -> 0.104 ms; on
+// the sphere (1806 patches, levels 1-7) 1.66 -> 1.21 ms.
 //
 // Threads: [0, 4 MX) ghosts (or coarse cells) of the faces; [4 MX, 4 MX + 16)
 // corner ghosts; from the next whole warp on 24 cells beyond coarse interiors:
@@ -37,9 +40,22 @@ template <typename real>
 struct RingPart {
   int kind;             // of its region's neighbour; 0: nothing to store
   real v0, v1, v2, v3;  // two ghosts, or the coarse cell, its neighbours in, lo, hi
+  real v4;              // coarse, mapped grid: the cell towards the owner
   int t, n0;            // coarse: index along the face, patch
   bool own;             // coarse: the cell towards the owner is the owner's average
 };
+
+// Eq. ghost_coarse of four cells, the first at offset o of patch n (mapped
+// grid: weighted by their areas)
+template <bool CAP, typename real>
+__device__ __forceinline__ real ring_average(const DevForest<real>& D, int n, int o, real s0,
+                                             real s1, real s2, real s3) {
+  if (!CAP) return real(0.25) * (((s0 + s1) + s2) + s3);
+  const double* K = D.metric + (size_t)n * D.S * D.S + o;
+  const double k0 = K[0], k1 = K[1], k2 = K[D.S], k3 = K[D.S + 1];
+  return real((((k0 * double(s0) + k1 * double(s1)) + k2 * double(s2)) + k3 * double(s3)) /
+              (((k0 + k1) + k2) + k3));
+}
 
 // interior cell at offset o of a patch at qo / qn (older / newer state) of
 // the level read at weight alpha (0 and 1: one state alone, see src_interior)
@@ -55,7 +71,7 @@ __device__ __forceinline__ real ring_time(const real* qo, const real* qn, real a
 // alpha (interpolate_direct_entry), else from its filled tile (D.qT at
 // tlevel, else the store).  cells: 24 values in shared memory.  keep_t: the
 // cells an interpolation reads are also stored in the kept coarse tiles.
-template <typename real, int MX>
+template <typename real, int MX, bool CAP>
 __device__ __forceinline__ RingPart<real> ring_read(const DevForest<real>& D, int p,
                                                     const PatchMeta& pm, int L, int tlevel,
                                                     real alpha, bool direct, real* cells, int tid,
@@ -80,13 +96,14 @@ __device__ __forceinline__ RingPart<real> ring_read(const DevForest<real>& D, in
       // summed in the order (0,0), (1,0), (0,1), (1,1)
       w.kind = NB_SAME;
       const int half = li >= MX / 2 ? 1 : 0;
-      const real* c = D.buf[D.cur[L + 1]] + (size_t)(half ? e.n1 : e.n0) * SS +
-                      (2 * li - half * MX + kMbc) * st + (low ? MX - 2 : 2) * sn;
+      const int n = half ? e.n1 : e.n0;
+      const int o = (2 * li - half * MX + kMbc) * st + (low ? MX - 2 : 2) * sn;
+      const real* c = D.buf[D.cur[L + 1]] + (size_t)n * SS + o;
       real u[8];
 #pragma unroll
       for (int k = 0; k < 8; ++k) u[k] = c[(k >> 2) * 2 * sn + (k & 1) + ((k >> 1) & 1) * S];
-      w.v0 = real(0.25) * (((u[0] + u[1]) + u[2]) + u[3]);
-      w.v1 = real(0.25) * (((u[4] + u[5]) + u[6]) + u[7]);
+      w.v0 = ring_average<CAP>(D, n, o, u[0], u[1], u[2], u[3]);
+      w.v1 = ring_average<CAP>(D, n, o + 2 * sn, u[4], u[5], u[6], u[7]);
     } else if (e.kind == NB_COARSE && li < MX / 2) {
       w.kind = NB_COARSE;
       const int t0 = X ? ((pm.y * MX + e.fy) >> 1) - e.y0 * MX
@@ -106,6 +123,11 @@ __device__ __forceinline__ RingPart<real> ring_read(const DevForest<real>& D, in
         w.v1 = ring_time(qo, qn, alpha, one, o + d);
         w.v2 = ring_time(qo, qn, alpha, one, ol);
         w.v3 = ring_time(qo, qn, alpha, one, oh);
+        if (CAP && w.own) {
+          const int b = (2 * li + kMbc) * st + (low ? kMbc : MX) * sn;
+          const real* u = D.buf[D.cur[L]] + (size_t)p * SS + b;
+          w.v4 = ring_average<CAP>(D, p, b, u[0], u[1], u[S], u[S + 1]);
+        }
       } else {
         const real* q = patch_ptr(tlevel == L - 1 ? D.qT : D.buf[c], e.n0, S);
         w.v0 = q[o];
@@ -123,10 +145,10 @@ __device__ __forceinline__ RingPart<real> ring_read(const DevForest<real>& D, in
                              ((r & 1) ? 0 : MX - 2) + x + kMbc];
     } else if (e.kind == NB_FINE) {
       w.kind = NB_SAME;
-      const real* c = D.buf[D.cur[L + 1]] + (size_t)e.n0 * SS +
-                      (((r & 2) ? 0 : MX - 4) + 2 * y + kMbc) * S + ((r & 1) ? 0 : MX - 4) +
-                      2 * x + kMbc;
-      w.v0 = real(0.25) * (((c[0] + c[1]) + c[S]) + c[S + 1]);
+      const int o = (((r & 2) ? 0 : MX - 4) + 2 * y + kMbc) * S + ((r & 1) ? 0 : MX - 4) + 2 * x +
+                    kMbc;
+      const real* c = D.buf[D.cur[L + 1]] + (size_t)e.n0 * SS + o;
+      w.v0 = ring_average<CAP>(D, e.n0, o, c[0], c[1], c[S], c[S + 1]);
     } else if (e.kind == NB_COARSE) {
       w.kind = NB_COARSE;
     }
@@ -174,7 +196,7 @@ __device__ __forceinline__ RingPart<real> ring_read(const DevForest<real>& D, in
 }
 
 // The stores into the landed tile T (cells and T's interior visible to all).
-template <typename real, int MX>
+template <typename real, int MX, bool CAP>
 __device__ __forceinline__ void ring_store(const DevForest<real>& D, const RingPart<real>& w,
                                            int L, int tlevel, real alpha, bool direct, real* T,
                                            const real* cells, int tid, real* keep_t,
@@ -205,7 +227,9 @@ __device__ __forceinline__ void ring_store(const DevForest<real>& D, const RingP
   const real q0 = w.v0, in = w.v1;
   const real lo = t == 0 ? cells[f] : w.v2, hi = t == MX - 1 ? cells[f] : w.v3;
   real out;
-  if (w.own) {  // towards the owner: the average of its own cells
+  if (CAP && w.own) {
+    out = w.v4;
+  } else if (w.own) {  // towards the owner: the average of its own cells
     const real* u = T + (2 * li + kMbc) * st + (low ? kMbc : MX) * sn;
     out = real(0.25) * (((u[0] + u[1]) + u[S]) + u[S + 1]);
   } else if (direct) {
