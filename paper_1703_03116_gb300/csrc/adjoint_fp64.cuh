@@ -8,7 +8,7 @@
 // signs and selections are taken on the bits, and an edge's forward values
 // and its transpose together take about 27 FP64 instructions, half of what
 // the form in the speeds' own units takes.  4 coarse steps of 229 patches of
-// 32^2 and their gradient: 5.0 -> 3.9 ms.
+// 32^2 and their gradient: 5.0 -> 3.7 ms.
 //
 // FP32 keeps that form (adjoint.cu): its instructions are not what bounds it
 // (2% of the adjoint of a global step), and its velocity-scale derivative is
@@ -43,11 +43,11 @@ __device__ __forceinline__ double turned(double a) {
 
 // Forward values of an edge that its transpose reads: jump W, limited wave L
 // and its partials dW, dU with respect to W and the upwind jump on the piece
-// the data select, correction kap L, the correction as the fluctuations
-// carry it (T), and the fluctuations (P turned).
+// the data select, the correction's factor kap and the correction Ft = kap L,
+// and the fluctuations (P turned).
 template <typename real>
 struct EdgeFw {
-  real W, L, dW, dU, kap, nP, M;
+  real W, L, dW, dU, kap, Ft, nP, M;
   bool up;
 };
 
@@ -75,7 +75,8 @@ __device__ __forceinline__ EdgeFw<real> edge_fw(const AdjScheme& sc, real c, rea
   }
   e.kap = a * (real(0.5) - a);
   if (!sc.o2) e.kap = e.L = real(0);
-  const real T = sc.t2 ? e.kap * e.L : real(0);
+  e.Ft = e.kap * e.L;
+  const real T = sc.t2 ? e.Ft : real(0);
   const real B = fma(-a, e.W, T);
   e.nP = e.up ? B : T;
   e.M = e.up ? T : B;
@@ -85,17 +86,17 @@ __device__ __forceinline__ EdgeFw<real> edge_fw(const AdjScheme& sc, real c, rea
 // One edge's transpose: e is the forward edge at half Courant number c between
 // cells a, b, c, d along its normal (qb, qc the middle two); lF, lP, lM the
 // adjoints of its normal flux and of the fluctuations it sends into c's and
-// b's side.  Returns the four cells' adjoint contributions, the derivative
-// with respect to the edge speed times the speed (ds), and c lF.
+// b's side.  Returns the four cells' adjoint contributions and c lF, and adds
+// the derivative with respect to the edge speed times the speed to ds.
 template <typename real>
 struct EdgeAdj {
-  real a, b, c, d, ds, cF;
+  real a, b, c, d, cF;
 };
 
 template <typename real>
 __device__ __forceinline__ EdgeAdj<real> edge_transpose(const EdgeFw<real>& e, const AdjScheme& sc,
                                                        real c, real qb, real qc, real lF,
-                                                       real lP, real lM) {
+                                                       real lP, real lM, real& ds) {
   const real lFt = sc.t2 ? lF + (lM - lP) : lF;
   const real a = fabs(c);
   const real lsel = sc.t1 ? (e.up ? lP : lM) : real(0);
@@ -110,8 +111,8 @@ __device__ __forceinline__ EdgeAdj<real> edge_transpose(const EdgeFw<real>& e, c
   o.a = e.up ? nU : real(0);
   o.d = e.up ? real(0) : lU;
   // d(kap)/dc c = |c| (1/2 - 2 |c|) = kap - |c|^2
-  const real u = fma(-a, a * e.L, e.kap * e.L);
-  o.ds = fma(lFt, u, fma(cl, e.W, o.cF * (e.up ? qb : qc)));
+  const real u = fma(-a, a * e.L, e.Ft);
+  ds = fma(lFt, u, fma(cl, e.W, fma(o.cF, e.up ? qb : qc, ds)));
   return o;
 }
 
@@ -200,9 +201,8 @@ __device__ __forceinline__ real band_transpose(const real* Q, real* LQ, const re
     real nY_l = __shfl_up_sync(kAll, nY, 1, MX);
     if (li == 0) nY_l = frow ? YPm[j] - YMm[j + 1] : real(0);
     // x-edge (li, j)
-    EdgeAdj<real> ox = edge_transpose(ex, sc, su, ql, qb, lFf, lX, lX_l);
-    if (!xrow) ox = EdgeAdj<real>{0, 0, 0, 0, 0, 0};
-    dsum += ox.ds;
+    EdgeAdj<real> ox{0, 0, 0, 0, 0};
+    if (xrow) ox = edge_transpose(ex, sc, su, ql, qb, lFf, lX, lX_l, dsum);
     if (sc.t1 && xrow && frow) dsum = fma(ox.cF, ex.up ? nY_l : nY, dsum);
     real T = ox.c;
     {
@@ -224,8 +224,8 @@ __device__ __forceinline__ real band_transpose(const real* Q, real* LQ, const re
     // y-edge (li, j)
     if (yrow) {
       const EdgeAdj<real> oy = edge_transpose(ey, sc, v_cur, qa, qb, lGf_cur,
-                                              j < MX ? lY : real(0), j > 0 ? lY_prev : real(0));
-      dsum += oy.ds;
+                                              j < MX ? lY : real(0), j > 0 ? lY_prev : real(0),
+                                              dsum);
       if (sc.t1) dsum = fma(oy.cF, ey.up ? nX_prev : nX, dsum);
       A0 += oy.a;
       A1 += oy.b;
@@ -294,12 +294,11 @@ __device__ __forceinline__ real side_transpose(const real* Q, real* LQ, const re
         nlM = (j + 1 <= MX ? pos(vvel(MX - 1, j + 1)) * lGf(MX - 1, j + 1) : real(0)) +
               (j >= 0 ? neg(vvel(MX - 1, j)) * lGf(MX - 1, j) : real(0));
       const EdgeAdj<real> o =
-          edge_transpose(e, sc, s, q(MX - 1, j), q(MX, j), lF, real(0), turned(nlM));
+          edge_transpose(e, sc, s, q(MX - 1, j), q(MX, j), lF, real(0), turned(nlM), dsum);
       add(MX - 2, j, o.a);
       add(MX - 1, j, o.b);
       add(MX, j, o.c);
       add(MX + 1, j, o.d);
-      dsum += o.ds;
       if (sc.t1 && j >= 0 && j < MX) {  // its transverse increment's speed
         const int c = e.up ? MX - 1 : MX;
         dsum = fma(o.cF, yedge(c, j).nP - yedge(c, j + 1).M, dsum);
@@ -316,12 +315,11 @@ __device__ __forceinline__ real side_transpose(const real* Q, real* LQ, const re
         return turned(right ? neg(uvel(MX, r)) * lFf(MX, r) : pos(uvel(0, r)) * lFf(0, r));
       };
       const EdgeAdj<real> o =
-          edge_transpose(e, sc, s, q(c, j - 1), q(c, j), real(0), lY(j), lY(j - 1));
+          edge_transpose(e, sc, s, q(c, j - 1), q(c, j), real(0), lY(j), lY(j - 1), dsum);
       add(c, j - 2, o.a);
       add(c, j - 1, o.b);
       add(c, j, o.c);
       add(c, j + 1, o.d);
-      dsum += o.ds;
     }
   }
   return dsum;
