@@ -561,7 +561,7 @@ __global__ void __launch_bounds__(256, sizeof(real) == 4 ? 3 : 2)
     const V zero = PV::all(real(0));
     V nX_prev = zero, G_cur = zero, nP_cur = zero, Gf_prev = zero, dF_prev = zero;
     Speed<V> v_cur(zero);
-#pragma unroll 2
+#pragma unroll(sizeof(real) == 4 ? 6 : 2)  // (FP32: 2.72, 2.71, 2.68 ms by 2, 3, 6; 1: 2.99)
     for (int it = 0; it < W::R + 2; ++it) {
       const int r = it - 1;
       const V qd = col(0, r + 2);
