@@ -344,43 +344,60 @@ __global__ void trig_kernel(real* out, int len, real h) {
 
 inline int grid_for(int n) { return n < 1 ? 1 : (n < 65535 * 8 ? n : 65535 * 8); }
 
-// Refluxing (Berger and Colella's correction; the paper's scheme has none):
-// one warp per level-L patch, lane k on face cell k.  A face whose other side
+// Refluxing (Berger and Colella's correction; the paper's scheme has none): a
+// thread per boundary cell of the level-L patches.  A face whose other side
 // is finer (an NB_FINE face entry: n0 holds the half of the face at cells
 // 0..MX/2-1, n1 the other half, the square domains' identity orientation)
 // gives coarse cell k the fine fluxes of fine cells 2k - half*MX and the next
 // through the fine patch's opposite face, summed over nfs substep slots and
-// scaled by w, in place of its own flux Fc of slot cslot.  The faces go one
-// after the other (-x, +x, -y, +y): a corner cell takes two corrections, from
-// two lanes, ordered by the warp barrier between faces.
+// scaled by w, in place of its own flux Fc of slot cslot.  A cell takes its
+// faces' corrections in the order -x, +x, -y, +y (a corner cell two), each
+// face's reads issued before any is used: the launches are small and wait
+// for their chain of dependent reads (229 patches of 8^2, a coarse step 85 ->
+// 75 us against a warp a patch, face after face).
 template <typename real, int MX>
-__global__ void reflux_kernel(DevForest<real> D, int p0, int p1, const real* __restrict__ bflux,
-                              int cslot, int nfs, real w, real nu) {
-  const int lane = threadIdx.x & 31;
-  const int p = p0 + blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (p >= p1) return;  // whole warps leave together
-  real* Q = D.buf[D.cur[D.meta[p].level]] + (size_t)p * D.S * D.S;
-  for (int dir = 0; dir < 4; ++dir) {
-    const NbrEntry& e = D.nbr[(size_t)p * 8 + dir];
-    if (e.kind == NB_FINE && lane < MX) {
-      const int k = lane, half = k >= MX / 2 ? 1 : 0;
-      const int n = half ? e.n1 : e.n0;
-      const int jf = 2 * k - half * MX;
-      const int ff = dir ^ 1;  // the fine patch's face on the shared edge
-      real acc = real(0);
-      for (int s = 0; s < nfs; ++s) {
-        const real* b = bflux + (((size_t)n * 2 + s) * 4 + ff) * MX + jf;
-        acc += b[0] + b[1];
-      }
-      const real Fbar = w * acc;
-      const real Fc = bflux[(((size_t)p * 2 + cslot) * 4 + dir) * MX + k];
-      const int i = dir == 0 ? 0 : (dir == 1 ? MX - 1 : k);
-      const int j = dir == 2 ? 0 : (dir == 3 ? MX - 1 : k);
-      real* c = Q + (size_t)(j + kMbc) * D.S + (i + kMbc);
-      *c = (dir == 0 || dir == 2) ? *c + nu * (Fbar - Fc) : *c + nu * (Fc - Fbar);
+__global__ void __launch_bounds__(128) reflux_kernel(DevForest<real> D, int p0, int p1,
+                                                     const real* __restrict__ bflux, int cslot,
+                                                     int nfs, real w, real nu) {
+  constexpr int NB = 4 * MX - 4;                          // boundary cells
+  constexpr int TP = NB <= 32 ? 32 : NB <= 64 ? 64 : 128;  // threads a patch
+  const int p = p0 + blockIdx.x * (128 / TP) + threadIdx.x / TP, b = threadIdx.x % TP;
+  if (p >= p1 || b >= NB) return;
+  // cells of the rows 0 and MX-1, then of the columns 0 and MX-1 between
+  const int m = b - 2 * MX;
+  const int i = b < 2 * MX ? b % MX : (m & 1) * (MX - 1);
+  const int j = b < 2 * MX ? (b / MX) * (MX - 1) : 1 + (m >> 1);
+  const int fx = i == 0 ? 0 : i == MX - 1 ? 1 : -1, fy = j == 0 ? 2 : j == MX - 1 ? 3 : -1;
+  const int dir[2] = {fx, fy}, k[2] = {j, i};
+  int n[2] = {-1, -1};
+#pragma unroll
+  for (int c = 0; c < 2; ++c)
+    if (dir[c] >= 0) {
+      const NbrEntry& e = D.nbr[(size_t)p * 8 + dir[c]];
+      if (e.kind == NB_FINE) n[c] = k[c] >= MX / 2 ? e.n1 : e.n0;
     }
-    __syncwarp();
-  }
+  if (n[0] < 0 && n[1] < 0) return;
+  real Fbar[2] = {real(0), real(0)}, Fc[2] = {real(0), real(0)};
+#pragma unroll
+  for (int c = 0; c < 2; ++c)
+    if (n[c] >= 0) {
+      const int jf = 2 * k[c] - (k[c] >= MX / 2 ? MX : 0);
+      real acc = real(0);
+      for (int s = 0; s < nfs; ++s) {  // through the fine patch's face on the shared edge
+        const real* f = bflux + (((size_t)n[c] * 2 + s) * 4 + (dir[c] ^ 1)) * MX + jf;
+        acc += f[0] + f[1];
+      }
+      Fbar[c] = w * acc;
+      Fc[c] = bflux[(((size_t)p * 2 + cslot) * 4 + dir[c]) * MX + k[c]];
+    }
+  real* q = D.buf[D.cur[D.meta[p].level]] + (size_t)p * D.S * D.S + (size_t)(j + kMbc) * D.S + i +
+            kMbc;
+  real v = *q;
+#pragma unroll
+  for (int c = 0; c < 2; ++c)
+    if (n[c] >= 0)
+      v = (dir[c] & 1) == 0 ? v + nu * (Fbar[c] - Fc[c]) : v + nu * (Fc[c] - Fbar[c]);
+  *q = v;
 }
 
 // Refluxing on the cubed sphere, from the host's pairing (per patch, face
@@ -436,20 +453,18 @@ template <typename real>
 cudaError_t launch_reflux(const DevForest<real>& D, int p0, int p1, const real* bflux, int cslot,
                           int nfs, double w, double nu, cudaStream_t s) {
   if (p1 <= p0) return cudaSuccess;
-  constexpr int kWarps = 4;
-  const int grid = (p1 - p0 + kWarps - 1) / kWarps;
-  switch (D.mx) {
+  const int n = p1 - p0;
+  switch (D.mx) {  // (4, 2 or 1 patches a CTA of 128 threads)
     case 8:
-      reflux_kernel<real, 8><<<grid, 32 * kWarps, 0, s>>>(D, p0, p1, bflux, cslot, nfs, real(w),
-                                                           real(nu));
+      reflux_kernel<real, 8><<<(n + 3) / 4, 128, 0, s>>>(D, p0, p1, bflux, cslot, nfs, real(w),
+                                                         real(nu));
       break;
     case 16:
-      reflux_kernel<real, 16><<<grid, 32 * kWarps, 0, s>>>(D, p0, p1, bflux, cslot, nfs, real(w),
-                                                            real(nu));
+      reflux_kernel<real, 16><<<(n + 1) / 2, 128, 0, s>>>(D, p0, p1, bflux, cslot, nfs, real(w),
+                                                          real(nu));
       break;
     case 32:
-      reflux_kernel<real, 32><<<grid, 32 * kWarps, 0, s>>>(D, p0, p1, bflux, cslot, nfs, real(w),
-                                                            real(nu));
+      reflux_kernel<real, 32><<<n, 128, 0, s>>>(D, p0, p1, bflux, cslot, nfs, real(w), real(nu));
       break;
     default: return cudaErrorInvalidValue;
   }
