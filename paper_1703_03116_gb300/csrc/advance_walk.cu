@@ -25,7 +25,7 @@
 //
 // Measured on one GB300 against the form before it (ghost by ghost after a
 // fill launch, one cell a lane, two tile buffers a warp), a coarse step with
-// its field moves: 256 forests (67168 patches of 32^2, FP32) 6.0 -> 2.7 ms,
+// its field moves: 256 forests (67168 patches of 32^2, FP32) 6.0 -> 2.6 ms,
 // 64 forests (13852 patches of 16^2, FP64) 3.7 -> 2.5 ms; 16384 patches of
 // 32^2 at one level 94 -> 67 us.  About 3500 warp instructions a 32^2 patch
 // (of 6200), at 55% of the issue slots with 24 warps an SM; its sides are one
@@ -53,9 +53,11 @@ template <>
 struct Vec2<double> {
   using T = double2;
 };
+// x-edge MX of a row: fluctuation M into cell MX - 1 and the final flux as
+// A + B nY, nY the turned y-fluctuation sum of cell MX - 1
 template <typename real>
-struct alignas(16) EdgeRec {  // x-edge MX of a row: fluctuation into cell MX - 1, normal flux,
-  real M, F, c, nY;           // speed; turned y-fluctuation sum of ghost cell MX
+struct alignas(16) EdgeRec {
+  real M, A, B, pad;
 };
 
 // Shared memory of one patch: its tile, its eight neighbour entries, and per
@@ -504,8 +506,8 @@ __global__ void __launch_bounds__(256, sizeof(real) == 4 ? 3 : 2)
           if (q < MX + 2) {
             EdgeRec<real>* e = reinterpret_cast<EdgeRec<real>*>(b + SL::rec) + q;
             e->M = PV::get(M, k);
-            e->F = PV::get(F, k);
-            e->c = PV::get(c, k);
+            e->A = PV::get(F, k);  // (the normal flux and the speed, until both columns are known)
+            e->B = PV::get(c, k);
           } else {
             const bool right = q >= 2 * MX + 3;
             const int r = q - (right ? 2 * MX + 3 : MX + 2);
@@ -522,8 +524,9 @@ __global__ void __launch_bounds__(256, sizeof(real) == 4 ? 3 : 2)
         unsigned char* b = const_cast<unsigned char*>(k ? b1 : b0);
         const real* y = reinterpret_cast<const real*>(b + SL::ye);
         reinterpret_cast<real*>(b + SL::yl)[li + 1] = y[li] - y[MX + 1 + li + 1];
-        reinterpret_cast<EdgeRec<real>*>(b + SL::rec)[li + 1].nY =
-            y[2 * (MX + 1) + li] - y[3 * (MX + 1) + li + 1];
+        EdgeRec<real>& e = reinterpret_cast<EdgeRec<real>*>(b + SL::rec)[li + 1];
+        const real nYE = y[2 * (MX + 1) + li] - y[3 * (MX + 1) + li + 1];  // of ghost cell MX
+        edge_affine(e.B, nYE, e.A, sc, e.A, e.B);
       }
       __syncwarp();
     }
@@ -561,7 +564,7 @@ __global__ void __launch_bounds__(256, sizeof(real) == 4 ? 3 : 2)
     const V zero = PV::all(real(0));
     V nX_prev = zero, G_cur = zero, nP_cur = zero, Gf_prev = zero, dF_prev = zero;
     Speed<V> v_cur(zero);
-#pragma unroll(sizeof(real) == 4 ? 6 : 2)  // (FP32: 2.72, 2.71, 2.68 ms by 2, 3, 6; 1: 2.99)
+#pragma unroll(sizeof(real) == 4 ? 6 : 2)  // (FP32, 256 forests: 2.72 ms by 2, 2.68 by 6)
     for (int it = 0; it < W::R + 2; ++it) {
       const int r = it - 1;
       const V qd = col(0, r + 2);
@@ -583,28 +586,28 @@ __global__ void __launch_bounds__(256, sizeof(real) == 4 ? 3 : 2)
         vedge(sx, vsub(qb, ql), vupwind(fx, col(-2, r), ql, qb, col(1, r)), ql, qb, sc, F, nP, M);
       }
       V Mr = down(M);
-      EdgeRec<real> e0, e1;
-      if (last) {
-        e0 = ec0[it];
-        e1 = ec1[it];
-        Mr = PV::make(e0.M, e1.M);
-      }
+      const EdgeRec<real> e0 = ec0[it], e1 = ec1[it];
+      if (last) Mr = PV::make(e0.M, e1.M);
       const V nX = vsub(nP, Mr);  // turned x-fluctuation sum of cell (li, r)
-      V Gn, nPn, Mn;
-      vedge(sy, Wb, vselect(fy, Wa, Wc), qb, qc, sc, Gn, nPn, Mn);
+      // (FP64: the last row's y-edge and the first and last rows' x-fluxes,
+      // which nothing uses, are left out; FP32 has no branch here)
+      constexpr bool kAll2 = PV::N == 2;
+      V Gn = zero, nPn = zero, Mn = zero;
+      if (kAll2 || it <= W::R) vedge(sy, Wb, vselect(fy, Wa, Wc), qb, qc, sc, Gn, nPn, Mn);
       // final flux of y-edge (li, r)
       const V Gf = vfinal(v_cur, nX_prev, nX, G_cur, sc);
       // final fluxes of x-edges (li, r) and (li + 1, r)
-      const V nY = vsub(nP_cur, Mn);  // turned y-fluctuation sum of cell (li, r)
-      V nYl = up(nY);
-      if (first) nYl = PV::make(yl0[it], yl1[it]);
-      const V Ff = vfinal(sx, nYl, nY, F, sc);
-      V Fr = down(Ff);
-      if (last) {
-        const V ce = PV::make(e0.c, e1.c);
-        Fr = vfinal(Speed<V>(ce), nY, PV::make(e0.nY, e1.nY), PV::make(e0.F, e1.F), sc);
+      V dF = zero;
+      if (kAll2 || (it >= 1 && it <= W::R)) {
+        const V nY = vsub(nP_cur, Mn);  // turned y-fluctuation sum of cell (li, r)
+        V nYl = up(nY);
+        if (first) nYl = PV::make(yl0[it], yl1[it]);
+        const V Ff = vfinal(sx, nYl, nY, F, sc);
+        V Fr = down(Ff);
+        const V Fe = vfma(PV::make(e0.B, e1.B), nY, PV::make(e0.A, e1.A));
+        if (last) Fr = Fe;
+        dF = vsub(Fr, Ff);
       }
-      const V dF = vsub(Fr, Ff);
       if (it >= 2) {  // the update of cell (li, r - 1)
         const V n = vfma(PV::all(real(-2)), vadd(dF_prev, vsub(Gf, Gf_prev)), qa);
         if (ok[0]) dst0[(r + 1) * S] = PV::get(n, 0);

@@ -190,6 +190,23 @@ __device__ __forceinline__ double final_flux(double c, double nXm, double nXp, d
   return fma(c, sc.t1() ? X : 0.0, F);
 }
 
+// final_flux as A + B nXm, from the side that is known (nXp)
+template <bool FULL>
+__device__ __forceinline__ void edge_affine(float c, float nXp, float F,
+                                            const Scheme<float, FULL>& sc, float& A, float& B) {
+  const float ct = sc.t1() ? c : 0.f;
+  A = fmaf(fminf(ct, 0.f), nXp, F);
+  B = fmaxf(ct, 0.f);
+}
+template <bool FULL>
+__device__ __forceinline__ void edge_affine(double c, double nXp, double F,
+                                            const Scheme<double, FULL>& sc, double& A,
+                                            double& B) {
+  const bool up = upwind_left(c);
+  A = up || !sc.t1() ? F : fma(c, nXp, F);
+  B = up && sc.t1() ? c : 0.0;
+}
+
 }  // namespace fc
 
 // ------------------------------------------------ the walk's packed form
