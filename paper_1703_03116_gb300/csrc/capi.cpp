@@ -742,9 +742,11 @@ void choose_variant(const fc_forest* F, int n, AdvArgs* a) {
     // rows a band, by warps: at mx = 16 one row of a patch a warp segment (8
     // warps) computes every x-edge three times; FP64, 320 patches: 31.0 us,
     // two rows 23.0, four 20.9 (64 patches: 16.7, 16.6, 18.7); FP32, 1280
-    // patches: 16.7, 14.7, 14.7 (64: the same)
+    // patches: 16.7, 14.7, 14.7 (64: the same).  At mx = 32 FP64 takes 8 rows a
+    // band (4 warps) and two CTAs an SM: a step of the swirl forest's levels
+    // of 35 to 248 patches 718 us, 740 with 4 rows; FP32 473 and 416
     a->variant = ADV_BAND;
-    a->warps = mx == 16 ? (F->esize == 8 && n >= 128 ? 2 : 4) : 8;
+    a->warps = mx == 16 ? (F->esize == 8 && n >= 128 ? 2 : 4) : F->esize == 8 ? 4 : 8;
   }
   // only the staged and band updates record the face fluxes
   if (F->bflux && a->variant != ADV_STAGED && a->variant != ADV_BAND) {
