@@ -782,11 +782,20 @@ double advance_bytes(const fc_forest* F, int n) {
   return (double)n * (((mx + 4) * (mx + 4) + mx * mx) * (double)F->esize + metric);
 }
 
+// Alg. 1 on every level; delta: also the regrid indicator, tagged set if it
+// was taken (one launch for whole forests; a partition's mirrors hold only
+// what its owned patches read, and fused fills off means the separate kernels)
 template <typename real>
-fc_status fill_all_t(fc_forest* F, cudaStream_t s) {
+fc_status fill_all_t(fc_forest* F, cudaStream_t s, double* delta, bool* tagged) {
   DevForest<real> D = dev<real>(F);
   const HostForest& H = F->host;
   const double gb = ghost_bytes(F);
+  if (F->fuse && !H.partial) {
+    Timed tm(F, 1, s, gb * H.npatch());
+    FC_CUDA(launch_fill_tag(D, H.desc.indicator, delta, F->d_err, s));
+    if (tagged) *tagged = delta != nullptr;
+    return FC_OK;
+  }
   FillArgs A{F->d_lists + F->off_all, (int)H.list_all.size(), -1, 0.0};
   {
     Timed tm(F, 1, s, gb * A.ntargets);
@@ -800,8 +809,10 @@ fc_status fill_all_t(fc_forest* F, cudaStream_t s) {
   return FC_OK;
 }
 
-fc_status fill_all(fc_forest* F, cudaStream_t s) {
-  return F->esize == 4 ? fill_all_t<float>(F, s) : fill_all_t<double>(F, s);
+fc_status fill_all(fc_forest* F, cudaStream_t s, double* delta = nullptr,
+                   bool* tagged = nullptr) {
+  return F->esize == 4 ? fill_all_t<float>(F, s, delta, tagged)
+                       : fill_all_t<double>(F, s, delta, tagged);
 }
 
 // the adjoint's replay: copy the time-interpolated tiles of level L-1 (what
@@ -2244,15 +2255,16 @@ fc_status fc_tag(fc_forest* F, double* delta_host, void* stream) {
   if (!F || !delta_host) return fail(FC_ERR_INVALID_ARG, "null argument");
   cudaStream_t s = as_stream(stream);
   const int kind = F->host.desc.indicator;
+  bool tagged = false;
   {  // Alg. 1 first: central differences read the first ghost layer, and a
      // regrid's new children interpolate from their parent's cells with its
      // ghosts (the update kernels keep ghosts in shared memory only)
-    const fc_status st = fill_all(F, s);
+    const fc_status st = fill_all(F, s, F->d_delta, &tagged);
     if (st != FC_OK) return st;
   }
   const int n = F->host.npatch();
-  cudaError_t e;
-  {
+  cudaError_t e = cudaSuccess;
+  if (!tagged) {
     Timed tm(F, 2, s, (double)n * F->host.desc.mx * F->host.desc.mx * F->esize);
     e = F->esize == 4 ? launch_tag(dev<float>(F), kind, F->d_delta, s)
                       : launch_tag(dev<double>(F), kind, F->d_delta, s);

@@ -12,10 +12,107 @@
 //
 // The rules themselves live in ghost_gather.cuh, shared with the patch-update
 // kernels, which apply them to the tile they hold in shared memory.
-#include "ghost_gather.cuh"
+// fill_tag: the whole of Alg. 1 for every patch at one time, and the regrid
+//   indicator, in one launch: a coarser neighbour's cells are computed where
+//   they are read (as the updates do), so no patch waits for another's ghosts,
+//   and the indicator is taken from the tile in shared memory.
+#include "ghost_ring.cuh"
 
 namespace fc {
 namespace {
+
+// One CTA per patch: its tile by a bulk copy, its ghost ring (ghost_ring.cuh,
+// or ghost by ghost where a neighbour's axes are turned), the wall condition
+// and the corners beyond a cube vertex; the ghosts go back to the patch's
+// array, the indicator (kind 0: max over cells of |grad q| / 2, 1: max q - min
+// q; tag_kernel's values) to delta if it is set.  Three launches took their
+// latency one after another (496 patches of 32^2, FP32: 20 us and two gaps, now
+// 6 us; the tag with its copy to the host 47 -> 29 us).
+template <typename real, int MX, bool CAP>
+__global__ void __launch_bounds__(288) fill_tag_kernel(const __grid_constant__ DevForest<real> D,
+                                                       int kind, double* delta, int* err) {
+  constexpr int S = MX + 4, NT = 288, NG = num_ghosts<MX>();
+  constexpr uint32_t bytes = sizeof(real) * S * S;
+  __shared__ __align__(128) real Q[S * S];
+  __shared__ __align__(8) uint64_t bar;
+  __shared__ real ring[CAP ? NG : 24];
+  __shared__ bool ring_w[CAP ? NG : 1];
+  __shared__ real red[2][NT / 32];
+  const int tid = threadIdx.x, p = blockIdx.x;
+  if (tid == 0) mbar_init(&bar, 1);
+  const PatchMeta pm = D.meta[p];
+  const int L = pm.level;
+  real* P = D.buf[D.cur[L]] + (size_t)p * S * S;
+  if (tid == 0) {
+    fence_proxy_async();
+    mbar_expect_tx(&bar, bytes);
+    bulk_load(Q, P, bytes, &bar);
+  }
+  const bool each = CAP && (pm.flags & 2);
+  RingPart<real> part;
+  if (each)
+    gather_ring<real, MX>(D, [&](int r) { return D.nbr[(size_t)p * 8 + r]; }, p, pm, L - 1,
+                          real(1), true, ring, ring_w, tid, NT);
+  else
+    part = ring_read<real, MX, CAP>(D, p, pm, L, L - 1, real(1), true, ring, tid, nullptr, 0);
+  const bool landed = tid == 0 ? mbar_wait(&bar, 0, kWaitLimit) : true;
+  if (!__syncthreads_and(landed)) {
+    if (tid == 0) atomicOr(err, kErrTimeout);
+    mbar_wait(&bar, 0, kWaitLimit);
+    return;
+  }
+  if (tid != 0) mbar_wait(&bar, 0, kWaitLimit);
+  if (each)
+    store_ring<real, MX>(Q, ring, ring_w, tid, NT);
+  else
+    ring_store<real, MX, CAP>(D, part, L, L - 1, real(1), true, Q, ring, tid, nullptr, 0, p);
+  __syncthreads();
+  const int last_q = (1 << L) - 1;
+  if (D.domain == FC_DOMAIN_WALLS &&
+      (pm.x == 0 || pm.y == 0 || pm.x == last_q || pm.y == last_q)) {
+    wall_bc<real, MX>(pm, Q, tid, NT);
+    __syncthreads();
+  }
+  if (each) {
+    corner3_fill_k<real, MX>([&](int r) { return D.nbr[(size_t)p * 8 + r].kind; }, Q, tid, NT);
+    __syncthreads();
+  }
+  for (int k = tid; k < NG; k += NT) {
+    int i, j;
+    ghost_ij<MX>(k, i, j);
+    const int o = (j + kMbc) * S + i + kMbc;
+    P[o] = Q[o];
+  }
+  if (!delta) return;
+  real hi = kind == 1 ? Q[2 * S + 2] : real(0), lo = hi;
+  for (int k = tid; k < MX * MX; k += NT) {
+    const real* c = Q + (k / MX + 2) * S + k % MX + 2;
+    real v = c[0];
+    if (kind == 0) {
+      const real gx = c[1] - c[-1], gy = c[S] - c[-S];
+      v = gx * gx + gy * gy;
+    }
+    hi = v > hi ? v : hi;
+    lo = v < lo ? v : lo;
+  }
+  for (int w = 16; w > 0; w >>= 1) {
+    const real a = __shfl_down_sync(0xffffffffu, hi, w), b = __shfl_down_sync(0xffffffffu, lo, w);
+    hi = a > hi ? a : hi;
+    lo = b < lo ? b : lo;
+  }
+  if ((tid & 31) == 0) {
+    red[0][tid >> 5] = hi;
+    red[1][tid >> 5] = lo;
+  }
+  __syncthreads();
+  if (tid == 0) {
+    for (int w = 1; w < NT / 32; ++w) {
+      hi = red[0][w] > hi ? red[0][w] : hi;
+      lo = red[1][w] < lo ? red[1][w] : lo;
+    }
+    delta[p] = kind == 1 ? (double)hi - (double)lo : 0.5 * sqrt((double)hi);
+  }
+}
 
 template <typename real, int MX>
 __global__ void __launch_bounds__(256) fill_coarse_kernel(DevForest<real> D, FillArgs A) {
@@ -137,6 +234,40 @@ cudaError_t launch_fill_fine(const DevForest<real>& D, const FillArgs& A, cudaSt
   return fill_dispatch(D, A, true, s);
 }
 
+template <typename real>
+cudaError_t launch_fill_tag(const DevForest<real>& D, int kind, double* delta, int* err,
+                            cudaStream_t s) {
+  if (D.npatch <= 0) return cudaSuccess;
+  const bool cap = D.metric != nullptr;
+  switch (D.mx) {
+    case 8:
+      if (cap)
+        fill_tag_kernel<real, 8, true><<<D.npatch, 288, 0, s>>>(D, kind, delta, err);
+      else
+        fill_tag_kernel<real, 8, false><<<D.npatch, 288, 0, s>>>(D, kind, delta, err);
+      break;
+    case 16:
+      if (cap)
+        fill_tag_kernel<real, 16, true><<<D.npatch, 288, 0, s>>>(D, kind, delta, err);
+      else
+        fill_tag_kernel<real, 16, false><<<D.npatch, 288, 0, s>>>(D, kind, delta, err);
+      break;
+    case 32:
+      if (cap)
+        fill_tag_kernel<real, 32, true><<<D.npatch, 288, 0, s>>>(D, kind, delta, err);
+      else
+        fill_tag_kernel<real, 32, false><<<D.npatch, 288, 0, s>>>(D, kind, delta, err);
+      break;
+    default: return cudaErrorInvalidValue;
+  }
+  ++launch_counter();
+  return cudaGetLastError();
+}
+
+template cudaError_t launch_fill_tag<float>(const DevForest<float>&, int, double*, int*,
+                                            cudaStream_t);
+template cudaError_t launch_fill_tag<double>(const DevForest<double>&, int, double*, int*,
+                                             cudaStream_t);
 template cudaError_t launch_fill_coarse<float>(const DevForest<float>&, const FillArgs&,
                                                cudaStream_t);
 template cudaError_t launch_fill_coarse<double>(const DevForest<double>&, const FillArgs&,
