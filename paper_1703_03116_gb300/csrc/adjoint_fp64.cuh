@@ -28,14 +28,13 @@ __device__ __forceinline__ bool same_sign(double a, double b) {
   const long long x = __double_as_longlong(a), y = __double_as_longlong(b);
   return (x ^ y) >= 0 && (x << 1) != 0 && (y << 1) != 0;
 }
-// |a| <= |b|, |a| <= 4 |b|
-__device__ __forceinline__ bool mag_le(double a, double b) {
-  constexpr long long kMag = 0x7fffffffffffffffll;
-  return (__double_as_longlong(a) & kMag) <= (__double_as_longlong(b) & kMag);
+// |a| <= |b|, |a| <= 4 |b| (unsigned: 4 |b| may pass the largest double)
+__device__ __forceinline__ unsigned long long mag(double a) {
+  return (unsigned long long)__double_as_longlong(a) & 0x7fffffffffffffffull;
 }
+__device__ __forceinline__ bool mag_le(double a, double b) { return mag(a) <= mag(b); }
 __device__ __forceinline__ bool mag_le4(double a, double b) {
-  constexpr long long kMag = 0x7fffffffffffffffll;
-  return (__double_as_longlong(a) & kMag) <= (__double_as_longlong(b) & kMag) + (2ll << 52);
+  return mag(a) <= mag(b) + (2ull << 52);
 }
 __device__ __forceinline__ double turned(double a) {
   return __longlong_as_double(__double_as_longlong(a) ^ (long long)0x8000000000000000ull);

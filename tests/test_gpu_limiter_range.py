@@ -37,3 +37,26 @@ def test_limited_waves_over_the_range(variant, mx):
             gpu.set_q(np.ldexp(q, k))
             gpu.step_global(0.1, 0.3 / (4 * mx))
             assert relerr(np.ldexp(gpu.get_q().astype(np.float64), -k), want) <= tol, k
+
+
+@pytest.mark.parametrize("variant", [1, 3])
+@pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf])
+def test_limited_waves_beside_cells_without_value(variant, bad):
+    """A jump that is NaN limits to 0: what the oracle computes from the
+    cells around one that is not finite, the updates compute too."""
+    for mx in (8, 32):
+        w = synth.swirl(3, lmin=1, lmax=2, mx=mx)
+        g = np.random.Generator(np.random.PCG64(mx))
+        for dtype, tol in ((fc.F64, F64_TOL), (fc.F32, 1e-5)):
+            ref, gpu = pair(fc, w, dtype)
+            q = g.random(ref.get_q().shape)
+            q.reshape(-1)[g.integers(0, q.size, 3)] = bad
+            gpu.set_advance_variant(variant, 4)
+            ref.set_q(q)
+            gpu.set_q(q)
+            ref.step_global(0.1, 0.3 / (4 * mx))
+            gpu.step_global(0.1, 0.3 / (4 * mx))
+            want, got = ref.get_q(), gpu.get_q().astype(np.float64)
+            ok = np.isfinite(want)
+            assert 0 < np.count_nonzero(~ok) < 200
+            assert np.abs(got[ok] - want[ok]).max() <= tol
