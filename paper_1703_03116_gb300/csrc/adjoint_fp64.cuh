@@ -8,7 +8,8 @@
 // signs and selections are taken on the bits, and an edge's forward values
 // and its transpose together take about 27 FP64 instructions, half of what
 // the form in the speeds' own units takes.  4 coarse steps of 229 patches of
-// 32^2 and their gradient: 5.0 -> 3.7 ms.
+// 32^2 and their gradient: 5.0 -> 3.7 ms, and 3.3 ms with magnitudes and
+// negations on the bits too (magnitude_bits()).
 //
 // FP32 keeps that form (adjoint.cu): its instructions are not what bounds it
 // (2% of the adjoint of a global step), and its velocity-scale derivative is
@@ -29,15 +30,20 @@ __device__ __forceinline__ bool same_sign(double a, double b) {
   return (x ^ y) >= 0 && (x << 1) != 0 && (y << 1) != 0;
 }
 // |a| <= |b|, |a| <= 4 |b| (unsigned: 4 |b| may pass the largest double)
-__device__ __forceinline__ unsigned long long mag(double a) {
-  return (unsigned long long)__double_as_longlong(a) & 0x7fffffffffffffffull;
+__device__ __forceinline__ bool mag_le(double a, double b) {
+  return magnitude_bits(a) <= magnitude_bits(b);
 }
-__device__ __forceinline__ bool mag_le(double a, double b) { return mag(a) <= mag(b); }
 __device__ __forceinline__ bool mag_le4(double a, double b) {
-  return mag(a) <= mag(b) + (2ull << 52);
+  return magnitude_bits(a) <= magnitude_bits(b) + (2ull << 52);
+}
+// |a|, -a
+__device__ __forceinline__ double magnitude(double a) {
+  return __longlong_as_double((long long)magnitude_bits(a));
 }
 __device__ __forceinline__ double turned(double a) {
-  return __longlong_as_double(__double_as_longlong(a) ^ (long long)0x8000000000000000ull);
+  int hi;
+  asm("xor.b32 %0, %1, 0x80000000;" : "=r"(hi) : "r"(__double2hiint(a)));
+  return __hiloint2double(hi, __double2loint(a));
 }
 
 // Forward values of an edge that its transpose reads: jump W, limited wave L
@@ -56,7 +62,7 @@ __device__ __forceinline__ EdgeFw<real> edge_fw(const AdjScheme& sc, real c, rea
   EdgeFw<real> e;
   e.up = upwind_left(c);
   e.W = qc - qb;
-  const real a = fabs(c);
+  const real a = magnitude(c);
   if (sc.mc) {
     const real U = upwind_jump(c, qa, qb, qc, qd);
     const real S = e.W + U;
@@ -97,7 +103,7 @@ __device__ __forceinline__ EdgeAdj<real> edge_transpose(const EdgeFw<real>& e, c
                                                        real c, real qb, real qc, real lF,
                                                        real lP, real lM, real& ds) {
   const real lFt = sc.t2 ? lF + (lM - lP) : lF;
-  const real a = fabs(c);
+  const real a = magnitude(c);
   const real lsel = sc.t1 ? (e.up ? lP : lM) : real(0);
   const real cl = c * lsel, g = e.kap * lFt;
   EdgeAdj<real> o;

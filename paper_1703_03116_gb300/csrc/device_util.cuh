@@ -11,14 +11,23 @@ __device__ __forceinline__ float minmod(float a, float b) {
   if ((a <= 0.f && b >= 0.f) || (a >= 0.f && b <= 0.f)) return 0.f;
   return fabsf(a) < fabsf(b) ? a : b;
 }
-// the same on the bits: no FP64 instruction (the FP64 pipe issues 1/64 of an
-// SM's slots); a NaN gives b, as the comparisons do
+// The magnitude's bits of a double, by a 32-bit instruction in a form the
+// compiler keeps: it turns a 64-bit mask back into an absolute value, which is
+// an instruction of the FP64 pipe (1/64 of an SM's issue slots).  Three an
+// edge of the update, of twelve: a coarse step of the swirl forest in FP64 716
+// -> 605 us, 64 forests of 16^2 patches 2.46 -> 2.03 ms.
+__device__ __forceinline__ unsigned long long magnitude_bits(double a) {
+  unsigned hi;
+  asm("and.b32 %0, %1, 0x7fffffff;" : "=r"(hi) : "r"(__double2hiint(a)));
+  return ((unsigned long long)hi << 32) | (unsigned)__double2loint(a);
+}
+// the same on the bits, without an FP64 instruction; a NaN gives b, as the
+// comparisons do
 __device__ __forceinline__ double minmod(double a, double b) {
-  constexpr long long kMag = 0x7fffffffffffffffll, kInf = 0x7ff0000000000000ll;
-  const long long x = __double_as_longlong(a), y = __double_as_longlong(b);
-  const long long ax = x & kMag, ay = y & kMag;
+  constexpr unsigned long long kInf = 0x7ff0000000000000ull;
+  const unsigned long long ax = magnitude_bits(a), ay = magnitude_bits(b);
   if (ax > kInf || ay > kInf) return b;
-  if ((x ^ y) < 0 || ax == 0 || ay == 0) return 0.0;
+  if ((__double2hiint(a) ^ __double2hiint(b)) < 0 || ax == 0 || ay == 0) return 0.0;
   return ax < ay ? a : b;
 }
 
