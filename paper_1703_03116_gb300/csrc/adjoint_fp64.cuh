@@ -25,17 +25,6 @@ struct AdjScheme {
   bool o2, mc, t1, t2;  // second order, MC limiter, transverse fluctuations, corrections
 };
 
-__device__ __forceinline__ bool same_sign(double a, double b) {
-  const long long x = __double_as_longlong(a), y = __double_as_longlong(b);
-  return (x ^ y) >= 0 && (x << 1) != 0 && (y << 1) != 0;
-}
-// |a| <= |b|, |a| <= 4 |b| (unsigned: 4 |b| may pass the largest double)
-__device__ __forceinline__ bool mag_le(double a, double b) {
-  return magnitude_bits(a) <= magnitude_bits(b);
-}
-__device__ __forceinline__ bool mag_le4(double a, double b) {
-  return magnitude_bits(a) <= magnitude_bits(b) + (2ull << 52);
-}
 // |a|, -a
 __device__ __forceinline__ double magnitude(double a) {
   return __longlong_as_double((long long)magnitude_bits(a));
@@ -67,8 +56,10 @@ __device__ __forceinline__ EdgeFw<real> edge_fw(const AdjScheme& sc, real c, rea
     const real U = upwind_jump(c, qa, qb, qc, qd);
     const real S = e.W + U;
     // the pieces (W + U) / 2, 2 W, 2 U; ties take the first
-    const bool on = same_sign(e.W, U);
-    const bool half = mag_le4(S, e.W) && mag_le4(S, U), byW = mag_le(e.W, U);
+    const unsigned long long mW = magnitude_bits(e.W), mU = magnitude_bits(U);
+    const unsigned long long mS = magnitude_bits(S), k4 = 2ull << 52;  // (4 x: exponent + 2)
+    const bool on = (__double2hiint(e.W) ^ __double2hiint(U)) >= 0 && mW != 0 && mU != 0;
+    const bool half = mS <= mW + k4 && mS <= mU + k4, byW = mW <= mU;
     const real f = half ? real(0.5) : real(2);
     e.L = on ? f * (half ? S : byW ? e.W : U) : real(0);
     e.dW = on && (half || byW) ? f : real(0);
