@@ -638,8 +638,9 @@ __global__ void __launch_bounds__(NT, sizeof(real) == 4 && NT >= 384 ? 2 : 1)
       }
       __syncthreads();
       if (threadIdx.x < NW)
-        dsum += half::band_transpose<real, MX, R>(Q, LQ, LN, XMe, YPm, YMm, sc, uvel, vvel,
-                                                  threadIdx.x);
+        dsum += half::band_transpose<real, MX, R>(
+            Q, LQ, LN, XMe, YPm, YMm, sc,
+            half::AdjSpeeds<real>{Sx, Sy, Tx, Ty, ucoef, cu, cv, swirl}, threadIdx.x);
       else
         dsum += half::side_transpose<real, MX>(Q, LQ, LN, sc, uvel, vvel, threadIdx.x - NW, NS);
     } else {

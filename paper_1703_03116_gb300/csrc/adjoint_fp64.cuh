@@ -8,8 +8,9 @@
 // signs and selections are taken on the bits, and an edge's forward values
 // and its transpose together take about 27 FP64 instructions, half of what
 // the form in the speeds' own units takes.  4 coarse steps of 229 patches of
-// 32^2 and their gradient: 5.0 -> 3.7 ms, and 3.3 ms with magnitudes and
-// negations on the bits too (magnitude_bits()).
+// 32^2 and their gradient: 5.0 -> 3.7 ms, 3.2 ms with magnitudes and
+// negations on the bits too (magnitude_bits()), 3.1 ms with a column's factors
+// kept over its rows and one addition less an edge.
 //
 // FP32 keeps that form (adjoint.cu): its instructions are not what bounds it
 // (2% of the adjoint of a global step), and its velocity-scale derivative is
@@ -100,10 +101,11 @@ __device__ __forceinline__ EdgeAdj<real> edge_transpose(const EdgeFw<real>& e, c
   EdgeAdj<real> o;
   o.cF = c * lF;
   const real lW = fma(e.dW, g, cl), lU = e.dU * g;
-  const real nU = turned(lU);
-  const real v = o.cF + (e.up ? lU : nU);  // on the upwind cell
-  o.b = (e.up ? v : real(0)) - lW;
-  o.c = (e.up ? real(0) : v) + lW;
+  const real nU = turned(lU), nW = turned(lW);
+  // on the upwind cell, then with the jump's share of its side
+  const real v = (o.cF + (e.up ? lU : nU)) + (e.up ? nW : lW);
+  o.b = e.up ? v : nW;
+  o.c = e.up ? lW : v;
   o.a = e.up ? nU : real(0);
   o.d = e.up ? real(0) : lU;
   // d(kap)/dc c = |c| (1/2 - 2 |c|) = kap - |c|^2
@@ -116,6 +118,19 @@ template <typename real>
 __device__ __forceinline__ real pos(real c) { return upwind_left(c) ? c : real(0); }
 template <typename real>
 __device__ __forceinline__ real neg(real c) { return upwind_left(c) ? real(0) : c; }
+
+// The edges' half Courant numbers: a factor of the column times one of the
+// row (swirl), or constant.
+template <typename real>
+struct AdjSpeeds {
+  const real *Sx, *Sy, *Tx, *Ty;  // the patch's tables, node k at [k + 1]
+  real uc, cu, cv;
+  bool swirl;
+  __device__ __forceinline__ real xfac(int i) const { return swirl ? uc * Sx[i + 1] : real(0); }
+  __device__ __forceinline__ real yfac(int i) const { return swirl ? -uc * Tx[i + 1] : real(0); }
+  __device__ __forceinline__ real u(real f, int j) const { return swirl ? f * Ty[j + 1] : cu; }
+  __device__ __forceinline__ real v(real f, int j) const { return swirl ? f * Sy[j + 1] : cv; }
+};
 
 // Transpose of the update of one patch (its final fluxes, their transverse
 // increments and every edge), as a row walk: thread tid's lane li owns
@@ -132,14 +147,20 @@ __device__ __forceinline__ real neg(real c) { return upwind_left(c) ? real(0) : 
 // adjoint of the new interior (the update's factor); XMe[j + 1]: forward M
 // of x-edge (MX, j); YPm[j], YMm[j]: forward P (turned), M of y-edge (-1, j).
 // Returns the lane's share of sum ds.
-template <typename real, int MX, int R, class UV, class VV>
+template <typename real, int MX, int R>
 __device__ __forceinline__ real band_transpose(const real* Q, real* LQ, const real* LN,
                                                const real* XMe, const real* YPm, const real* YMm,
-                                               const AdjScheme& sc, UV uvel, VV vvel, int tid) {
+                                               const AdjScheme& sc, const AdjSpeeds<real>& sp,
+                                               int tid) {
   constexpr int S = MX + 4;
   constexpr unsigned kAll = 0xffffffffu;
   const int li = tid % MX, r0 = (tid / MX) * R, r1 = r0 + R;
   const bool last = r1 == MX;
+  // a column's factors, kept (the tables would be read and multiplied again
+  // after every atomic add)
+  const real ux = sp.xfac(li), uxE = sp.xfac(MX), vy = sp.yfac(li);
+  auto uvel = [&](int j) -> real { return sp.u(ux, j); };
+  auto vvel = [&](int j) -> real { return sp.v(vy, j); };
   auto q = [&](int i, int j) -> real { return Q[(j + kMbc) * S + i + kMbc]; };
   auto ln = [&](int j) -> real { return (j >= 0 && j < MX) ? LN[j * MX + li] : real(0); };
   auto flush = [&](int row, real v) {
@@ -149,7 +170,7 @@ __device__ __forceinline__ real band_transpose(const real* Q, real* LQ, const re
   real A0 = 0, A1 = 0, A2 = 0, A3 = 0;  // contributions to rows j-2 .. j+1
   real qa = q(li, r0 - 2), qb = q(li, r0 - 1), qc = q(li, r0), qd = 0;
   real ln_cur = ln(r0 - 1);
-  real v_cur = r0 - 1 >= 0 ? vvel(li, r0 - 1) : real(0);
+  real v_cur = r0 - 1 >= 0 ? vvel(r0 - 1) : real(0);
   real lGf_cur = r0 - 1 >= 0 ? ln_cur - ln(r0 - 2) : real(0);
   real nP_prev = 0, nX_prev = 0, lY_prev = 0;
   EdgeFw<real> ey{};  // forward y-edge (li, j)
@@ -160,13 +181,13 @@ __device__ __forceinline__ real band_transpose(const real* Q, real* LQ, const re
     const bool yrow = (j >= r0 && j < r1) || (last && j == MX);
     if (j + 2 <= MX + 1) qd = q(li, j + 2);
     // forward: x-edge (li, j), y-edge (li, j + 1)
-    const real su = uvel(li, j);
+    const real su = uvel(j);
     const real ql = q(li - 1, j);
     const EdgeFw<real> ex = edge_fw(sc, su, q(li - 2, j), ql, qb, q(li + 1, j));
     real vn = 0;
     EdgeFw<real> eyn{};
     if (j + 1 <= MX) {
-      vn = vvel(li, j + 1);
+      vn = vvel(j + 1);
       eyn = edge_fw(sc, vn, qa, qb, qc, qd);
     }
     // adjoints of the final fluxes and of the fluctuation sums
@@ -180,7 +201,7 @@ __device__ __forceinline__ real band_transpose(const real* Q, real* LQ, const re
     real su_r = __shfl_down_sync(kAll, su, 1, MX);
     if (li == MX - 1) {
       lFf_r = frow ? turned(ln_cur) : real(0);
-      su_r = uvel(MX, j);
+      su_r = sp.u(uxE, j);
     }
     // (turned: nlY, nlX the negated adjoints of Y(li, j), X(li, j))
     const real nlY = frow && sc.t1 ? fma(pos(su_r), lFf_r, neg(su) * lFf) : real(0);
