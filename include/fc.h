@@ -256,7 +256,9 @@ fc_status fc_step_multirate(fc_forest* forest, double t, double dt_coarse, void*
 fc_status fc_tag_regrid(fc_forest* forest, double tau_refine, double tau_coarsen,
                         const int* lmax_per_forest, int* changed, void* stream);
 
-/* The per-leaf indicator alone, into a host array of nleaves doubles. */
+/* The per-leaf indicator alone, into a host array of nleaves doubles.  It and
+ * fc_tag_regrid return FC_ERR_TIMEOUT, the layout and the field as they were,
+ * when a bounded device wait gave up in the tag or in a step before it. */
 fc_status fc_tag(fc_forest* forest, double* delta_host, void* stream);
 
 /* Velocity scale sigma: every edge speed is multiplied by sigma (default 1).
@@ -521,13 +523,13 @@ fc_status fc_set_advance_variant(fc_forest* forest, int variant, int warps);
  *   walk_ctas   cap on the persistent walk grid (0: as many CTAs as the SMs
  *               hold at once); a small cap makes every warp loop over many
  *               groups of patches through both of its tile buffers.
- *   wait_polls  polls of the patch-update kernels' bounded wait for their
- *               tile copies before they give up (negative: the default,
+ *   wait_polls  polls of the patch-update and ghost-fill kernels' bounded wait
+ *               for their tile copies before they give up (negative: the default,
  *               2^22); 0 makes every such wait give up at once.  A kernel
  *               that gives up sets the forest's device error word (the next
  *               synchronising call returns FC_ERR_TIMEOUT and clears it),
  *               still waits, with the default limit, for the copies it has
- *               in flight, and leaves its patches not updated.
+ *               in flight, and leaves its patches not updated (or filled).
  * Captured steps are discarded (they carry the old values). */
 fc_status fc_set_limits(fc_forest* forest, int walk_ctas, int64_t wait_polls);
 fc_status fc_timers_read(fc_forest* forest, int phase, double* ms, int64_t* launches,

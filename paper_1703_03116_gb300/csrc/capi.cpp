@@ -576,7 +576,7 @@ fc_status upload(fc_forest* F, bool alloc_store, bool metrics = true) {
   const size_t uploaded = off;
   const size_t o_nbr = part(sizeof(NbrEntry) * n * 8);  // its own copy, from the host table
   const size_t o_sums = part(sizeof(double) * n), o_mass = part(sizeof(double) * nf),
-               o_delta = part(sizeof(double) * n);
+               o_delta = part(sizeof(double) * (n + 1));  // (fc_tag: and the error word)
   std::vector<char> host(uploaded, 0);
   std::memcpy(host.data() + o_meta, H.meta.data(), sizeof(PatchMeta) * n);
   if (!lists.empty()) std::memcpy(host.data() + o_lists, lists.data(), sizeof(int) * lists.size());
@@ -792,7 +792,7 @@ fc_status fill_all_t(fc_forest* F, cudaStream_t s, double* delta, bool* tagged) 
   const double gb = ghost_bytes(F);
   if (F->fuse && !H.partial) {
     Timed tm(F, 1, s, gb * H.npatch());
-    FC_CUDA(launch_fill_tag(D, H.desc.indicator, delta, F->d_err, s));
+    FC_CUDA(launch_fill_tag(D, H.desc.indicator, delta, F->wait_polls, F->d_err, s));
     if (tagged) *tagged = delta != nullptr;
     return FC_OK;
   }
@@ -2270,9 +2270,16 @@ fc_status fc_tag(fc_forest* F, double* delta_host, void* stream) {
                       : launch_tag(dev<double>(F), kind, F->d_delta, s);
   }
   if (e != cudaSuccess) return cuda_fail(e, "tag");
-  std::vector<double> dd(n);
-  FC_CUDA(cudaMemcpyAsync(dd.data(), F->d_delta, sizeof(double) * n, cudaMemcpyDeviceToHost, s));
+  // the error word comes with the indicators (one copy to the host): a tag or
+  // an update before it that gave up must not decide a layout
+  std::vector<double> dd(n + 1);
+  FC_CUDA(cudaMemcpyAsync(F->d_delta + n, F->d_err, sizeof(int), cudaMemcpyDeviceToDevice, s));
+  FC_CUDA(cudaMemcpyAsync(dd.data(), F->d_delta, sizeof(double) * (n + 1), cudaMemcpyDeviceToHost,
+                          s));
   FC_CUDA(cudaStreamSynchronize(s));
+  int word = 0;
+  std::memcpy(&word, &dd[n], sizeof word);
+  if (word != 0) return check_device_error(F, s);
   for (int k = 0; k < F->host.napi(); ++k) delta_host[k] = dd[F->host.dev_of[k]];
   return FC_OK;
 }

@@ -582,10 +582,11 @@ cudaError_t launch_fill_coarse(const DevForest<real>& D, const FillArgs& A, cuda
 template <typename real>
 cudaError_t launch_fill_fine(const DevForest<real>& D, const FillArgs& A, cudaStream_t s);
 // Alg. 1 for every patch at one time, and the indicator of launch_tag into
-// delta (null: none), in one launch
+// delta (null: none), in one launch; a patch whose tile's copy does not land
+// within wait_limit polls sets the error word and leaves both as they were
 template <typename real>
-cudaError_t launch_fill_tag(const DevForest<real>& D, int kind, double* delta, int* err,
-                            cudaStream_t s);
+cudaError_t launch_fill_tag(const DevForest<real>& D, int kind, double* delta,
+                            uint32_t wait_limit, int* err, cudaStream_t s);
 template <typename real>
 cudaError_t launch_advance(const DevForest<real>& D, int p0, int p1, const AdvArgs& a, int* err,
                            cudaStream_t s);

@@ -30,7 +30,8 @@ namespace {
 // 6 us; the tag with its copy to the host 47 -> 29 us).
 template <typename real, int MX, bool CAP>
 __global__ void __launch_bounds__(288) fill_tag_kernel(const __grid_constant__ DevForest<real> D,
-                                                       int kind, double* delta, int* err) {
+                                                       int kind, double* delta, uint32_t wait_limit,
+                                                       int* err) {
   constexpr int S = MX + 4, NT = 288, NG = num_ghosts<MX>();
   constexpr uint32_t bytes = sizeof(real) * S * S;
   __shared__ __align__(128) real Q[S * S];
@@ -55,10 +56,10 @@ __global__ void __launch_bounds__(288) fill_tag_kernel(const __grid_constant__ D
                           real(1), true, ring, ring_w, tid, NT);
   else
     part = ring_read<real, MX, CAP>(D, p, pm, L, L - 1, real(1), true, ring, tid, nullptr, 0);
-  const bool landed = tid == 0 ? mbar_wait(&bar, 0, kWaitLimit) : true;
+  const bool landed = tid == 0 ? mbar_wait(&bar, 0, wait_limit) : true;
   if (!__syncthreads_and(landed)) {
     if (tid == 0) atomicOr(err, kErrTimeout);
-    mbar_wait(&bar, 0, kWaitLimit);
+    mbar_wait(&bar, 0, kWaitLimit);  // let the copy land before leaving
     return;
   }
   if (tid != 0) mbar_wait(&bar, 0, kWaitLimit);
@@ -235,28 +236,28 @@ cudaError_t launch_fill_fine(const DevForest<real>& D, const FillArgs& A, cudaSt
 }
 
 template <typename real>
-cudaError_t launch_fill_tag(const DevForest<real>& D, int kind, double* delta, int* err,
-                            cudaStream_t s) {
+cudaError_t launch_fill_tag(const DevForest<real>& D, int kind, double* delta,
+                            uint32_t wait_limit, int* err, cudaStream_t s) {
   if (D.npatch <= 0) return cudaSuccess;
   const bool cap = D.metric != nullptr;
   switch (D.mx) {
     case 8:
       if (cap)
-        fill_tag_kernel<real, 8, true><<<D.npatch, 288, 0, s>>>(D, kind, delta, err);
+        fill_tag_kernel<real, 8, true><<<D.npatch, 288, 0, s>>>(D, kind, delta, wait_limit, err);
       else
-        fill_tag_kernel<real, 8, false><<<D.npatch, 288, 0, s>>>(D, kind, delta, err);
+        fill_tag_kernel<real, 8, false><<<D.npatch, 288, 0, s>>>(D, kind, delta, wait_limit, err);
       break;
     case 16:
       if (cap)
-        fill_tag_kernel<real, 16, true><<<D.npatch, 288, 0, s>>>(D, kind, delta, err);
+        fill_tag_kernel<real, 16, true><<<D.npatch, 288, 0, s>>>(D, kind, delta, wait_limit, err);
       else
-        fill_tag_kernel<real, 16, false><<<D.npatch, 288, 0, s>>>(D, kind, delta, err);
+        fill_tag_kernel<real, 16, false><<<D.npatch, 288, 0, s>>>(D, kind, delta, wait_limit, err);
       break;
     case 32:
       if (cap)
-        fill_tag_kernel<real, 32, true><<<D.npatch, 288, 0, s>>>(D, kind, delta, err);
+        fill_tag_kernel<real, 32, true><<<D.npatch, 288, 0, s>>>(D, kind, delta, wait_limit, err);
       else
-        fill_tag_kernel<real, 32, false><<<D.npatch, 288, 0, s>>>(D, kind, delta, err);
+        fill_tag_kernel<real, 32, false><<<D.npatch, 288, 0, s>>>(D, kind, delta, wait_limit, err);
       break;
     default: return cudaErrorInvalidValue;
   }
@@ -264,10 +265,10 @@ cudaError_t launch_fill_tag(const DevForest<real>& D, int kind, double* delta, i
   return cudaGetLastError();
 }
 
-template cudaError_t launch_fill_tag<float>(const DevForest<float>&, int, double*, int*,
-                                            cudaStream_t);
-template cudaError_t launch_fill_tag<double>(const DevForest<double>&, int, double*, int*,
-                                             cudaStream_t);
+template cudaError_t launch_fill_tag<float>(const DevForest<float>&, int, double*, uint32_t,
+                                            int*, cudaStream_t);
+template cudaError_t launch_fill_tag<double>(const DevForest<double>&, int, double*, uint32_t,
+                                             int*, cudaStream_t);
 template cudaError_t launch_fill_coarse<float>(const DevForest<float>&, const FillArgs&,
                                                cudaStream_t);
 template cudaError_t launch_fill_coarse<double>(const DevForest<double>&, const FillArgs&,
