@@ -56,10 +56,14 @@ __device__ __forceinline__ EdgeFw<real> edge_fw(const AdjScheme& sc, real c, rea
   if (sc.mc) {
     const real U = upwind_jump(c, qa, qb, qc, qd);
     const real S = e.W + U;
-    // the pieces (W + U) / 2, 2 W, 2 U; ties take the first
+    // the pieces (W + U) / 2, 2 W, 2 U; ties take the first.  A wave that
+    // the forward limiter drops has no partials: jumps of two signs, one below
+    // the normal range (where adding 2 to the exponent is not 4 x), a NaN
+    constexpr unsigned long long kInf = 0x7ff0000000000000ull, kMin = 1ull << 52;
     const unsigned long long mW = magnitude_bits(e.W), mU = magnitude_bits(U);
     const unsigned long long mS = magnitude_bits(S), k4 = 2ull << 52;  // (4 x: exponent + 2)
-    const bool on = (__double2hiint(e.W) ^ __double2hiint(U)) >= 0 && mW != 0 && mU != 0;
+    const bool on = (__double2hiint(e.W) ^ __double2hiint(U)) >= 0 && mW >= kMin && mU >= kMin &&
+                    mS <= kInf;
     const bool half = mS <= mW + k4 && mS <= mU + k4, byW = mW <= mU;
     const real f = half ? real(0.5) : real(2);
     e.L = on ? f * (half ? S : byW ? e.W : U) : real(0);
