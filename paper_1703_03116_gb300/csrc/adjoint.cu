@@ -43,7 +43,7 @@ namespace {
 template <typename real>
 __device__ __forceinline__ real mc_piece(real W, real Wup, real& dW, real& dWup) {
   dW = dWup = real(0);
-  if (!(W * Wup > real(0))) return real(0);
+  if (!wave_passes(W, Wup)) return real(0);
   const real a = real(0.5) * fabs(W + Wup);
   const real b = real(2) * fabs(W), c = real(2) * fabs(Wup);
   if (a <= b && a <= c) {
@@ -149,10 +149,11 @@ __device__ void adj_interp_patch(const DevForest<real>& D, const NbrStage& st, c
     L[(j + kMbc) * S + i + kMbc] = real(0);
     const real q0 = C[0];
     const real ax = C[1] - q0, bx = q0 - C[-1], ay = C[S] - q0, by = q0 - C[-S];
-    const real dax = (ax * bx > real(0) && fabs(ax) < fabs(bx)) ? real(1) : real(0);
-    const real dbx = (ax * bx > real(0) && !(fabs(ax) < fabs(bx))) ? real(1) : real(0);
-    const real day = (ay * by > real(0) && fabs(ay) < fabs(by)) ? real(1) : real(0);
-    const real dby = (ay * by > real(0) && !(fabs(ay) < fabs(by))) ? real(1) : real(0);
+    const bool onx = same_sign(ax, bx), ony = same_sign(ay, by);
+    const real dax = (onx && fabs(ax) < fabs(bx)) ? real(1) : real(0);
+    const real dbx = (onx && !(fabs(ax) < fabs(bx))) ? real(1) : real(0);
+    const real day = (ony && fabs(ay) < fabs(by)) ? real(1) : real(0);
+    const real dby = (ony && !(fabs(ay) < fabs(by))) ? real(1) : real(0);
     const real lsx = real(0.25) * dx * lg, lsy = real(0.25) * dy * lg;
     atomicAdd(LC, lg + lsx * (dbx - dax) + lsy * (dby - day));
     atomicAdd(LC + 1, lsx * dax);

@@ -31,6 +31,29 @@ __device__ __forceinline__ double minmod(double a, double b) {
   return ax < ay ? a : b;
 }
 
+// the smaller magnitude with the product of the signs (NaN where an operand is)
+__device__ __forceinline__ float min_mag_signs(float a, float b) {
+  float m;
+  asm("min.NaN.xorsign.abs.f32 %0, %1, %2;" : "=f"(m) : "f"(a), "f"(b));
+  return m;
+}
+// do two jumps share a sign (neither zero or NaN): not by their product, which
+// leaves the range before they do (in FP32 jumps of 1e-23)
+__device__ __forceinline__ bool same_sign(float a, float b) { return min_mag_signs(a, b) > 0.f; }
+__device__ __forceinline__ bool same_sign(double a, double b) {
+  constexpr unsigned long long kInf = 0x7ff0000000000000ull;
+  const unsigned long long ax = magnitude_bits(a), ay = magnitude_bits(b);
+  return (__double2hiint(a) ^ __double2hiint(b)) >= 0 && ax != 0 && ay != 0 && ax <= kInf &&
+         ay <= kInf;
+}
+// does the MC limiter pass the wave W beside the upwind one (FP64: a jump below
+// the normal range counts as none, see limited() of the row walks)
+__device__ __forceinline__ bool wave_passes(float W, float Wup) { return same_sign(W, Wup); }
+__device__ __forceinline__ bool wave_passes(double W, double Wup) {
+  constexpr unsigned long long kMin = 1ull << 52;
+  return same_sign(W, Wup) && magnitude_bits(W) >= kMin && magnitude_bits(Wup) >= kMin;
+}
+
 // Signed permutation A of Eq. (transform): bit 0 swaps the axes, bits 1 and
 // 2 negate the first and second output component.
 __device__ __forceinline__ int2 apply_a(int a, int x, int y) {
@@ -158,7 +181,7 @@ __device__ __forceinline__ double cospi_ratio<double>(double t, double T) { retu
 template <typename real>
 __device__ __forceinline__ real mc_limited(real W, real Wup) {
   const real m = fmin(real(0.5) * fabs(W + Wup), real(2) * fmin(fabs(W), fabs(Wup)));
-  return (W * Wup > real(0)) ? copysign(m, W) : real(0);
+  return wave_passes(W, Wup) ? copysign(m, W) : real(0);
 }
 
 }  // namespace fc

@@ -92,8 +92,7 @@ inline AdvConst<real> adv_const(const DevForest<real>& D, const AdvArgs& a) {
 __device__ __forceinline__ bool upwind_left(float c) { return c >= 0.f; }
 __device__ __forceinline__ bool upwind_left(double c) { return __double2hiint(c) >= 0; }
 
-// minima and maxima that are NaN where an operand is; the smaller magnitude
-// with the product of the signs
+// minima and maxima that are NaN where an operand is
 __device__ __forceinline__ float min_nan(float a, float b) {
   float m;
   asm("min.NaN.f32 %0, %1, %2;" : "=f"(m) : "f"(a), "f"(b));
@@ -107,11 +106,6 @@ __device__ __forceinline__ float min_nan(float a, float b, float c) {
 __device__ __forceinline__ float max_nan(float a, float b, float c) {
   float m;
   asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(m) : "f"(a), "f"(b), "f"(c));
-  return m;
-}
-__device__ __forceinline__ float min_mag_signs(float a, float b) {
-  float m;
-  asm("min.NaN.xorsign.abs.f32 %0, %1, %2;" : "=f"(m) : "f"(a), "f"(b));
   return m;
 }
 
