@@ -732,10 +732,11 @@ void choose_variant(const fc_forest* F, int n, AdvArgs* a) {
   } else if (t.tuned) {
     a->variant = t.variant;
     a->warps = t.warps;
-  } else if (n >= walk_from(mx, F->esize) && !F->d_metric &&
+  } else if (n >= walk_from(mx, F->esize) && !F->d_metric && !F->bflux &&
              F->host.desc.domain != FC_DOMAIN_SPHERE) {
-    // (it has no capacity form).  FP64: CTAs of two warps spread a launch of
-    // few groups over the SMs, whose FP64 pipes are what it waits for
+    // (it has no capacity form and records no face fluxes).  FP64: CTAs of two
+    // warps spread a launch of few groups over the SMs, whose FP64 pipes are
+    // what it waits for
     a->variant = ADV_WALK;
     a->warps = F->esize == 4 ? 8 : 2;
   } else {
@@ -748,7 +749,10 @@ void choose_variant(const fc_forest* F, int n, AdvArgs* a) {
     a->variant = ADV_BAND;
     a->warps = mx == 16 ? (F->esize == 8 && n >= 128 ? 2 : 4) : F->esize == 8 ? 4 : 8;
   }
-  // only the staged and band updates record the face fluxes
+  // Only the staged and band updates record the face fluxes.  Untuned launches
+  // that do take band at any size (us, staged / band, n = 1024 and 4096: mx = 32
+  // FP32 30.8 / 12.3 and 106 / 34.6, FP64 193 / 94 and 724 / 320; mx = 8 FP32
+  // 8.3 / 6.2 and 16.4 / 12.0, FP64 28.7 / 21.4 and 98 / 59)
   if (F->bflux && a->variant != ADV_STAGED && a->variant != ADV_BAND) {
     a->variant = ADV_STAGED;
     a->warps = 4;
