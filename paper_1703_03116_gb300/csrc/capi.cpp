@@ -1295,7 +1295,7 @@ fc_status fc_autotune(fc_forest* F, int* report, void* stream) {
   // (band with 16 warps is left out: timed a level at a time it can win,
   // but beside the other levels' branches of a captured step it measured
   // slower than with 8)
-  } cand[] = {{ADV_STAGED, 4}, {ADV_BAND, 4}, {ADV_BAND, 8},
+  } cand[] = {{ADV_STAGED, 4}, {ADV_BAND, 2}, {ADV_BAND, 4}, {ADV_BAND, 8},
               {ADV_WALK, 2},   {ADV_WALK, 4}, {ADV_WALK, 8}};
   constexpr int ncand = sizeof(cand) / sizeof(cand[0]);
   cudaEvent_t e0, e1;
@@ -1328,8 +1328,13 @@ fc_status fc_autotune(fc_forest* F, int* report, void* stream) {
       // below two patches per SM the walk's warps mostly idle: staged has
       // measured about twice as fast there (graph-replayed substeps)
       if (walk && p1 - p0 < 2 * nsm) continue;
-      // a band of one row recomputes three rows of x-edges
-      if (c.variant == ADV_BAND && H.desc.mx * H.desc.mx < 64 * c.warps) continue;
+      // the band's forms, those of choose_variant among them: bands of 4 and 2
+      // rows at mx = 16 (one row recomputes three rows of x-edges), of 8 and 4
+      // at mx = 32, and the one form of mx = 8
+      const int mx = H.desc.mx;
+      if (c.variant == ADV_BAND &&
+          !(mx == 8 ? c.warps == 4 : mx == 16 ? c.warps <= 4 : c.warps >= 4))
+        continue;
       a.variant = c.variant;
       a.warps = c.warps;
       a.gather = fused;
