@@ -455,7 +455,9 @@ fc_status fc_halo_unpack(fc_forest* forest, int peer, int level, const void* src
 /* Per-phase device timers (the paper's run-time breakdown, Sec. 5: advance,
  * ghost fill, regrid).  While enabled, every kernel launch of a phase is
  * bracketed by CUDA events on its stream.
- *   phase: 0 advance, 1 ghost fill, 2 regrid/tag/remap, 3 other.
+ *   phase: 0 advance, 1 ghost fill, 2 regrid/tag/remap, 3 other.  Fills made
+ *   inside another launch count with it: those of the fused updates with the
+ *   advance, a tag's (one launch with the indicator) with the tag.
  * fc_timers_read synchronises the forest's pending timed work and returns,
  * for one phase, the summed kernel time in ms, the number of timed launches
  * and the algorithmic bytes those launches must move (advance: every patch

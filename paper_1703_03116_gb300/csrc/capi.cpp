@@ -776,6 +776,11 @@ double ghost_bytes(const fc_forest* F) {
   return 2.0 * (4.0 * (mx + 4) + 4.0 * mx) * (double)F->esize;
 }
 
+// algorithmic bytes of the regrid indicator: every interior value read
+double tag_bytes(const fc_forest* F) {
+  return (double)F->host.npatch() * F->host.desc.mx * F->host.desc.mx * F->esize;
+}
+
 // algorithmic bytes of advancing n patches: read (mx+4)^2, write mx^2 each
 double advance_bytes(const fc_forest* F, int n) {
   const double mx = F->host.desc.mx;
@@ -795,7 +800,9 @@ fc_status fill_all_t(fc_forest* F, cudaStream_t s, double* delta, bool* tagged) 
   const HostForest& H = F->host;
   const double gb = ghost_bytes(F);
   if (F->fuse && !H.partial) {
-    Timed tm(F, 1, s, gb * H.npatch());
+    // (with the indicator it is a tag's launch: phase 2, which also reads
+    // every interior value)
+    Timed tm(F, delta ? 2 : 1, s, gb * H.npatch() + (delta ? tag_bytes(F) : 0.0));
     FC_CUDA(launch_fill_tag(D, H.desc.indicator, delta, F->wait_polls, F->d_err, s));
     if (tagged) *tagged = delta != nullptr;
     return FC_OK;
@@ -2274,7 +2281,7 @@ fc_status fc_tag(fc_forest* F, double* delta_host, void* stream) {
   const int n = F->host.npatch();
   cudaError_t e = cudaSuccess;
   if (!tagged) {
-    Timed tm(F, 2, s, (double)n * F->host.desc.mx * F->host.desc.mx * F->esize);
+    Timed tm(F, 2, s, tag_bytes(F));
     e = F->esize == 4 ? launch_tag(dev<float>(F), kind, F->d_delta, s)
                       : launch_tag(dev<double>(F), kind, F->d_delta, s);
   }
