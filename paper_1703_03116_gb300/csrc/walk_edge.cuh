@@ -23,6 +23,9 @@
 // 6.5 -> 6.0 ms.  (Those bits have to be taken as magnitude_bits() does.)
 #pragma once
 
+#include <algorithm>
+#include <limits>
+
 #include "device_util.cuh"
 
 namespace fc {
@@ -82,7 +85,11 @@ inline AdvConst<real> adv_const(const DevForest<real>& D, const AdvArgs& a) {
   c.cu = real(D.vel[0] * 0.5 * a.nu);
   c.cv = real(D.vel[1] * 0.5 * a.nu);
   c.hdt = real(0.5 * a.dt);
-  c.bfac = real(2.0 / (D.metric ? a.dt : a.nu));
+  // (a step so short that this leaves the type's range changes no value: its
+  // flux times dt / h is below every field's last bit, but inf times a zero
+  // flux is not)
+  c.bfac = real(std::min(2.0 / (D.metric ? a.dt : a.nu),
+                         double(std::numeric_limits<real>::max())));
   c.alpha = real(a.alpha);
   return c;
 }
