@@ -88,8 +88,7 @@ typedef enum { FC_VEL_CONST = 0, FC_VEL_SWIRL = 1, FC_VEL_ROTATION = 2, FC_VEL_D
  *               psi differences between the edges' end points, formed as
  *               k c (s_b - s_a)(s_b + s_a) - (2 pi/T_f)(Z_b - Z_a) with
  *               s = Y cos(2 pi t/T) - X sin(2 pi t/T), c = cos(pi t/T),
- *               from coefficients kept per edge (8 (mx+4)(mx+5) doubles a
- *               patch);
+ *               from coefficients kept per edge (fc_set_coef_budget);
  *               times the velocity scale.
  *               FC_VEL_ROTATION (sphere only): solid-body rotation
  *               u = omega x X, omega = (vel[0], vel[1], vel[2]).  The sphere
@@ -266,6 +265,16 @@ fc_status fc_tag(fc_forest* forest, double* delta_host, void* stream);
  * value drops the captured steps and tapes (their kernels carry the scale)
  * and synchronizes the device; setting the current value changes nothing. */
 fc_status fc_set_velocity_scale(fc_forest* forest, double scale);
+
+/* FC_VEL_DEFORM: the device memory that the edges' flux coefficients may take
+ * (bytes; negative: the default, 16 GiB).  A layout within it keeps 64 (mx+1)
+ * (mx+2) bytes of them a patch; one beyond it, or one whose coefficients do not
+ * fit on the device, keeps the 24 (mx+3)^2 bytes of its grid corners, from which
+ * every refresh forms the same coefficients: the same results, bit for bit, by
+ * a slower refresh.  Holds from the call on, across regrids; a forest is
+ * created with the default.  Drops the captured steps and synchronizes the
+ * device; no effect on the other flows. */
+fc_status fc_set_coef_budget(fc_forest* forest, int64_t bytes);
 
 /* Adjoint of one global time step (the transposes of Alg. 1 and of the
  * wave-propagation update; an extension for differentiation, with no

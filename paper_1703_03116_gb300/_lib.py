@@ -77,6 +77,7 @@ SIGNATURES = {
     "fc_set_graphs": (ctypes.c_int, [_vp, ctypes.c_int]),
     "fc_autotune": (ctypes.c_int, [_vp, _ip, _vp]),
     "fc_set_fused_fill": (ctypes.c_int, [_vp, ctypes.c_int]),
+    "fc_set_coef_budget": (ctypes.c_int, [_vp, ctypes.c_int64]),
     "fc_set_velocity_scale": (ctypes.c_int, [_vp, ctypes.c_double]),
     "fc_adjoint_step_global": (ctypes.c_int, [_vp, ctypes.c_double, ctypes.c_double, _vp, _vp,
                                               _vp]),

@@ -244,7 +244,9 @@ struct fc_forest {
   int trig_len[kMaxLevel + 1] = {};     // 0: not held
   double* d_metric = nullptr;             // cubed sphere: FP64 cell areas per patch
   void* d_umetric = nullptr;              // and the update's block in the field's precision
-  double* d_coef = nullptr;               // deformational flow: edge coefficients per patch
+  double* d_coef = nullptr;               // deformational flow: edge coefficients per patch,
+  bool coef_corners = false;              // or grid corners beyond the budget (coef_stride)
+  int64_t coef_budget = kCoefBudget;      // bytes
   void* lam[2] = {nullptr, nullptr};      // adjoint tiles (patch-store layout), lazily allocated
   void* madj[3] = {nullptr, nullptr, nullptr};  // multirate adjoint: current, previous, qT tiles
   void* mio = nullptr;                    // multirate adjoint: lam in field layout (graph input)
@@ -435,8 +437,8 @@ void free_device(fc_forest* F) {
 // cubed sphere: (re)compute the metric blocks of the current layout for the
 // rotation vector times the velocity scale (synchronous); after a regrid the
 // kept patches copy theirs from the old layout (rm, old: device).  The
-// deformational flow keeps every patch's edge coefficients instead of fixed
-// edge fluxes (its fluxes are refreshed per substep): all patches are
+// deformational flow keeps every patch's edge coefficients or corners instead
+// of fixed edge fluxes (its fluxes are refreshed per substep): all patches are
 // computed.
 fc_status update_metrics(fc_forest* F, const RemapEntry* rm = nullptr,
                          const fc_forest* old = nullptr) {
@@ -451,8 +453,20 @@ fc_status update_metrics(fc_forest* F, const RemapEntry* rm = nullptr,
   if (dmalloc(&F->d_metric, (size_t)n * S * S) != cudaSuccess ||
       dmalloc_bytes(&F->d_umetric, (size_t)n * umetric_stride(S) * F->esize) != cudaSuccess)
     return fail(FC_ERR_OOM, "metric allocation failed");
-  if (deform && dmalloc(&F->d_coef, (size_t)n * coef_stride(S)) != cudaSuccess)
-    return fail(FC_ERR_OOM, "edge coefficient allocation failed");
+  if (deform) {
+    // the coefficients within the budget, and while they fit beside what else
+    // is on the device; else the corners
+    const size_t bytes = (size_t)n * coef_stride(H.desc.mx, false) * sizeof(double);
+    F->coef_corners = bytes > (size_t)F->coef_budget;
+    if (!F->coef_corners &&
+        dmalloc_bytes(reinterpret_cast<void**>(&F->d_coef), bytes) != cudaSuccess) {
+      cudaGetLastError();
+      F->coef_corners = true;
+    }
+    if (F->coef_corners &&
+        dmalloc(&F->d_coef, (size_t)n * coef_stride(H.desc.mx, true)) != cudaSuccess)
+      return fail(FC_ERR_OOM, "grid corner allocation failed");
+  }
   double w[3] = {F->vel_scale * H.desc.vel[0], F->vel_scale * H.desc.vel[1],
                  F->vel_scale * H.desc.vel[2]};
   if (deform) {
@@ -465,13 +479,13 @@ fc_status update_metrics(fc_forest* F, const RemapEntry* rm = nullptr,
                                   static_cast<float*>(F->d_umetric), rm,
                                   old ? old->d_metric : nullptr,
                                   old ? static_cast<const float*>(old->d_umetric) : nullptr,
-                                  F->d_coef, g_alloc_stream));
+                                  F->d_coef, F->coef_corners, g_alloc_stream));
   else
     FC_CUDA(launch_sphere_metrics(F->d_meta, n, H.desc.mx, w, F->d_metric,
                                   static_cast<double*>(F->d_umetric), rm,
                                   old ? old->d_metric : nullptr,
                                   old ? static_cast<const double*>(old->d_umetric) : nullptr,
-                                  F->d_coef, g_alloc_stream));
+                                  F->d_coef, F->coef_corners, g_alloc_stream));
   return FC_OK;
 }
 
@@ -513,11 +527,11 @@ fc_status deform_fluxes(fc_forest* F, int p0, int p1, const AdvArgs& a, cudaStre
   if (d.vel_kind != FC_VEL_DEFORM || p1 <= p0) return FC_OK;
   const double kc = d.vel[0] * F->vel_scale, rot = 2.0 * M_PI / d.vel[2] * F->vel_scale;
   if (F->esize == 4)
-    FC_CUDA(launch_deform_fluxes(p0, p1, d.mx, F->d_coef, static_cast<float*>(F->d_umetric), kc,
-                                 d.vel[1], rot, a.t_half, a.t0_dev, a.t_off, s));
+    FC_CUDA(launch_deform_fluxes(p0, p1, d.mx, F->d_coef, F->coef_corners,
+                                 static_cast<float*>(F->d_umetric), kc, d.vel[1], rot, a.t_half, a.t0_dev, a.t_off, s));
   else
-    FC_CUDA(launch_deform_fluxes(p0, p1, d.mx, F->d_coef, static_cast<double*>(F->d_umetric), kc,
-                                 d.vel[1], rot, a.t_half, a.t0_dev, a.t_off, s));
+    FC_CUDA(launch_deform_fluxes(p0, p1, d.mx, F->d_coef, F->coef_corners,
+                                 static_cast<double*>(F->d_umetric), kc, d.vel[1], rot, a.t_half, a.t0_dev, a.t_off, s));
   return FC_OK;
 }
 
@@ -1120,7 +1134,7 @@ fc_status fc_forest_info(const fc_forest* F, fc_info* out) {
   if (F->bflux) bytes += n * 2 * 4 * H.desc.mx * F->esize;
   bytes += sizeof(NbrEntry) * n * 8 + sizeof(PatchMeta) * n + 3 * sizeof(double) * n;
   if (F->d_metric) bytes += n * (sizeof(double) * S * S + F->esize * umetric_stride((int)S));
-  if (F->d_coef) bytes += sizeof(double) * n * coef_stride((int)S);
+  if (F->d_coef) bytes += sizeof(double) * n * coef_stride(H.desc.mx, F->coef_corners);
   for (void* b : F->lam) bytes += b ? store : 0;
   for (void* b : F->madj) bytes += b ? store : 0;
   bytes += F->trig_bytes;
@@ -1426,6 +1440,17 @@ fc_status fc_set_velocity_scale(fc_forest* F, double scale) {
   destroy_graphs(F);
   FC_CUDA(cudaDeviceSynchronize());  // no launch may still read the old metrics
   fc_status st = update_metrics(F);   // sphere: the edge fluxes carry the scale
+  if (st == FC_OK) FC_CUDA(cudaStreamSynchronize(0));
+  return st;
+}
+
+fc_status fc_set_coef_budget(fc_forest* F, int64_t bytes) {
+  if (!F) return fail(FC_ERR_INVALID_ARG, "null forest");
+  F->coef_budget = bytes < 0 ? kCoefBudget : bytes;
+  if (F->host.desc.vel_kind != FC_VEL_DEFORM) return FC_OK;
+  destroy_graphs(F);                 // captured launches carry the old block
+  FC_CUDA(cudaDeviceSynchronize());  // no launch may still read it
+  fc_status st = update_metrics(F);
   if (st == FC_OK) FC_CUDA(cudaStreamSynchronize(0));
   return st;
 }
@@ -2333,6 +2358,7 @@ fc_status fc_tag_regrid(fc_forest* F, double tau_refine, double tau_coarsen,
   G->host.desc = F->host.desc;
   G->esize = F->esize;
   G->vel_scale = F->vel_scale;  // the sphere's metrics carry it
+  G->coef_budget = F->coef_budget;
   G->host.leaves = nl;
   // the new layout's build carries over the rows of the old one that it
   // keeps (the old tables are read, not reused; the memory of the tables
@@ -2451,6 +2477,7 @@ fc_status fc_tag_regrid(fc_forest* F, double tau_refine, double tau_coarsen,
   F->d_metric = G->d_metric;
   F->d_umetric = G->d_umetric;
   F->d_coef = G->d_coef;
+  F->coef_corners = G->coef_corners;
   F->d_pairs = G->d_pairs;
   std::memcpy(F->pair_level, G->pair_level, sizeof F->pair_level);
   for (int l = 0; l <= kMaxLevel; ++l) F->cur[l] = 0;

@@ -401,9 +401,17 @@ void sort_leaves(std::vector<Leaf>* v);
 // row j at j*(S+1) + i, shifted by 2), then through every y-edge,
 // phiy[(S+1)*S] (edge j-1/2 of column i at j*S + i, shifted by 2).
 __host__ __device__ constexpr int umetric_stride(int S) { return S * S + 2 * S * (S + 1); }
-// The deformational flow's four time-independent coefficients per edge (FP64,
-// planes over the x-edges, then the y-edges).
-__host__ __device__ constexpr int coef_stride(int S) { return 4 * 2 * S * (S + 1); }
+// The deformational flow keeps, in FP64, the four time-independent coefficients
+// of each edge that an update reads (planes over the x-edges 0..mx of rows
+// -1..mx, then the y-edges 0..mx of columns -1..mx: 71.8 KB a patch at mx =
+// 32), or for layouts whose coefficients exceed the forest's budget the grid
+// corners -1..mx+1 they are formed from (planes X, Y, Z: 29.4 KB), from which
+// the refresh forms the same coefficients every time.
+__host__ __device__ constexpr int edges_read(int mx) { return (mx + 1) * (mx + 2); }
+__host__ __device__ constexpr int coef_stride(int mx, bool corners) {
+  return corners ? 3 * (mx + 3) * (mx + 3) : 4 * 2 * edges_read(mx);
+}
+constexpr int64_t kCoefBudget = (int64_t)16 << 30;
 
 // Cubed sphere (FC_DOMAIN_SPHERE): block b is the face of the cube [-1,1]^3
 // with outward normal n; its block coordinates (x, y) in [0,1]^2 sit at
@@ -633,20 +641,21 @@ cudaError_t launch_coarse_sources(NbrEntry* nbr, const PatchMeta* meta, int n, i
 // stream function -omega . X (Sec. 5.3 mapped grids).  With a remap list (rm,
 // device, one entry per patch), RM_COPY patches copy their blocks from the old
 // layout's (same omega) instead.  With coef set, every patch's edge
-// coefficients of the deformational flow are written there.
+// coefficients of the deformational flow (corners: its grid corners) are
+// written there.
 template <typename real>
 cudaError_t launch_sphere_metrics(const PatchMeta* meta, int npatch, int mx, const double* omega,
                                   double* metric, real* umetric, const RemapEntry* rm,
                                   const double* old_metric, const real* old_umetric, double* coef,
-                                  cudaStream_t s);
+                                  bool corners, cudaStream_t s);
 
 // The deformational flow (FC_VEL_DEFORM): the edge volume fluxes of the
 // update's blocks of patches [p0, p1) for time t (t0_dev ? *t0_dev + t_off :
-// t_half) from their edge coefficients; kc = k * scale, rot = 2 pi / T_f *
-// scale.
+// t_half) from their edge coefficients or corners; kc = k * scale, rot = 2 pi
+// / T_f * scale.
 template <typename real>
-cudaError_t launch_deform_fluxes(int p0, int p1, int mx, const double* coef, real* umetric,
-                                 double kc, double T, double rot, double t_half,
+cudaError_t launch_deform_fluxes(int p0, int p1, int mx, const double* coef, bool corners,
+                                 real* umetric, double kc, double T, double rot, double t_half,
                                  const double* t0_dev, double t_off, cudaStream_t s);
 
 // fc_mass_noalloc's kernels (scratch in a file-scope device array)

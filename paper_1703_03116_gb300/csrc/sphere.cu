@@ -30,7 +30,12 @@
 // These four are kept per edge, so a substep's flux is four multiply-adds an
 // edge instead of the twelve of the end points' form (the FP64 pipe bounds the
 // refresh), and the time's sine and cosines are taken once per CTA, by three
-// threads of three warps.  432 patches of 32^2: 47 -> 20 us.
+// threads of three warps.  432 patches of 32^2: 47 -> 20 us.  They take more
+// memory than the corners (71.8 against 29.4 KB a 32^2 patch), so a layout
+// whose coefficients exceed the forest's budget keeps the corners and forms
+// the same values at each refresh: the same bits.  A global step of 1536
+// patches of 32^2, FP32 and FP64: 63 and 202 us from coefficients, 141 and 279
+// from corners (the end points' form from corners: 210 and 592).
 #include <atomic>
 #include <cmath>
 
@@ -58,6 +63,18 @@ __device__ __forceinline__ double tri_area(const double* a, const double* b, con
   return 2.0 * atan2(num, 1.0 + ab + bcd + ca);
 }
 
+// an edge's four coefficients from its end points a, b; sg: the sign of psi(b)
+// less psi(a) in the flux (the roundings written out: the kept and the
+// refresh's own are the same bits)
+struct EdgeCoef {
+  double e1, e2, e3, e4;
+};
+__device__ __forceinline__ EdgeCoef edge_coef(const double* a, const double* b, double sg) {
+  const double dX = sg * (b[0] - a[0]), dY = sg * (b[1] - a[1]);
+  const double sX = a[0] + b[0], sY = a[1] + b[1];
+  return EdgeCoef{dY * sY, fma(dY, sX, __dmul_rn(dX, sY)), dX * sX, sg * (b[2] - a[2])};
+}
+
 // one CTA per patch; X: the (S+1)^2 grid corners on the sphere, in shared
 // memory as three planes.  After a regrid (rm != null) a patch that kept its
 // quadrant copies its blocks from the old layout's store instead.
@@ -67,7 +84,8 @@ __global__ void __launch_bounds__(256) metrics_kernel(const PatchMeta* meta, int
                                                       double* metric, real* umetric,
                                                       const RemapEntry* rm,
                                                       const double* old_metric,
-                                                      const real* old_umetric, double* coef) {
+                                                      const real* old_umetric, double* coef,
+                                                      bool corners) {
   extern __shared__ double Xs[];
   const int S = mx + 2 * kMbc, SN = S + 1, NE = S * SN;
   double* X0 = Xs;
@@ -134,32 +152,43 @@ __global__ void __launch_bounds__(256) metrics_kernel(const PatchMeta* meta, int
       } else {
         U[S * S + k] = real(w0 * (b[0] - a[0]) + w1 * (b[1] - a[1]) + w2 * (b[2] - a[2]));
       }
-      if (coef) {
-        // psi differences: lower less upper end of an x-edge, right less left
-        // end of a y-edge
-        const double sg = y ? 1.0 : -1.0;
-        const double dX = sg * (b[0] - a[0]), dY = sg * (b[1] - a[1]);
-        const double sX = a[0] + b[0], sY = a[1] + b[1];
-        double* C = coef + (size_t)p * coef_stride(S) + k;
-        C[0] = dY * sY;
-        C[2 * NE] = dY * sX + dX * sY;
-        C[4 * NE] = dX * sX;
-        C[6 * NE] = sg * (b[2] - a[2]);
+      // of the edges an update reads: the flux is psi's difference
+      // of the lower less the upper end of an x-edge, the right less the left
+      // end of a y-edge
+      const int ei = i - kMbc, ej = j - kMbc;
+      if (coef && !corners && ei >= (y ? -1 : 0) && ei <= mx && ej >= (y ? 0 : -1) && ej <= mx) {
+        const EdgeCoef c = edge_coef(a, b, y ? 1.0 : -1.0);
+        const int NK = 2 * edges_read(mx);
+        double* C = coef + (size_t)p * coef_stride(mx, false) +
+                    (y ? NK / 2 + ej * (mx + 2) + ei + 1 : (ej + 1) * (mx + 1) + ei);
+        C[0] = c.e1;
+        C[NK] = c.e2;
+        C[2 * NK] = c.e3;
+        C[3 * NK] = c.e4;
       }
+    }
+    if (coef && corners) {
+      const int M = mx + 3;  // nodes -1..mx+1
+      double* C = coef + (size_t)p * coef_stride(mx, true);
+      for (int k = threadIdx.x; k < M * M; k += blockDim.x)
+        for (int c = 0; c < 3; ++c)
+          C[c * M * M + k] = (c == 0 ? X0 : c == 1 ? X1 : X2)[(k / M + 1) * SN + k % M + 1];
     }
     __syncthreads();
   }
 }
 
-// phi_x, phi_y of the update's blocks of patches [p0, p1) at time t: the
-// edges an update reads (x-edges 0..mx of rows -1..mx, y-edges alike)
-template <typename real, int MX>
+// phi_x, phi_y of the update's blocks of patches [p0, p1) at time t, of the
+// edges an update reads; CORNERS: coef holds the grid corners (the coefficients
+// are formed here: 13 FP64 instructions an edge instead of 4)
+template <typename real, int MX, bool CORNERS>
 __global__ void __launch_bounds__(512) deform_fluxes_kernel(int p0, int p1,
                                                             const double* __restrict__ coef,
                                                             real* __restrict__ umetric, double kc,
                                                             double T, double rot, double t_half,
                                                             const double* t0_dev, double t_off) {
-  constexpr int S = MX + 2 * kMbc, SN = S + 1, NE = S * SN, NU = (MX + 1) * (MX + 2);
+  constexpr int S = MX + 2 * kMbc, SN = S + 1, NE = S * SN, NK = 2 * edges_read(MX);
+  constexpr int M = MX + 3;
   __shared__ double tr[3];
   const double t = t0_dev ? *t0_dev + t_off : t_half;
   if (threadIdx.x == 0) tr[0] = cospi(2.0 * t / T);
@@ -169,43 +198,56 @@ __global__ void __launch_bounds__(512) deform_fluxes_kernel(int p0, int p1,
   const double c1 = tr[2] * tr[0] * tr[0], c2 = -tr[2] * tr[0] * tr[1],
                c3 = tr[2] * tr[1] * tr[1];
   for (int p = p0 + blockIdx.x; p < p1; p += gridDim.x) {
-    const double* C = coef + (size_t)p * coef_stride(S);
+    const double* C = coef + (size_t)p * coef_stride(MX, CORNERS);
     real* U = umetric + (size_t)p * umetric_stride(S) + S * S;
-    for (int k = threadIdx.x; k < 2 * NU; k += blockDim.x) {
-      const bool y = k >= NU;
-      const int e = y ? k - NU : k;
+    for (int k = threadIdx.x; k < NK; k += blockDim.x) {
+      const bool y = k >= NK / 2;
+      const int e = y ? k - NK / 2 : k;
       // x-edges: MX + 1 a row, rows 1..MX + 2 of the extended range; y-edges:
       // MX + 2 a row
       const int o = y ? NE + (e / (MX + 2) + 2) * S + e % (MX + 2) + 1
                       : (e / (MX + 1) + 1) * SN + e % (MX + 1) + 2;
-      U[o] = real(fma(-rot, C[6 * NE + o], fma(c1, C[o], fma(c2, C[2 * NE + o], c3 * C[4 * NE + o]))));
+      if constexpr (CORNERS) {
+        const double* A = C + (y ? (e / (MX + 2) + 1) * M + e % (MX + 2)
+                                 : (e / (MX + 1)) * M + e % (MX + 1) + 1);
+        const double* B = A + (y ? 1 : M);
+        const double a[3] = {A[0], A[M * M], A[2 * M * M]};
+        const double b[3] = {B[0], B[M * M], B[2 * M * M]};
+        const EdgeCoef f = edge_coef(a, b, y ? 1.0 : -1.0);
+        U[o] = real(fma(-rot, f.e4, fma(c1, f.e1, fma(c2, f.e2, c3 * f.e3))));
+      } else {  // (written out: through an EdgeCoef a refresh took 0.3 us longer)
+        U[o] = real(
+            fma(-rot, C[3 * NK + k], fma(c1, C[k], fma(c2, C[NK + k], c3 * C[2 * NK + k]))));
+      }
     }
   }
 }
 
 template <typename real, int MX>
-void deform_launch(int p0, int p1, const double* coef, real* umetric, double kc, double T,
-                   double rot, double t_half, const double* t0_dev, double t_off, cudaStream_t s) {
+void deform_launch(int p0, int p1, const double* coef, bool corners, real* umetric, double kc,
+                   double T, double rot, double t_half, const double* t0_dev, double t_off,
+                   cudaStream_t s) {
   // (an SM's share of the patches by one CTA of as many threads as a patch
   // feeds for some rounds: the time's functions once a CTA)
   const int n = p1 - p0, grid = n < 304 ? n : 304;
-  deform_fluxes_kernel<real, MX><<<grid, MX == 32 ? 512 : 128, 0, s>>>(
-      p0, p1, coef, umetric, kc, T, rot, t_half, t0_dev, t_off);
+  auto kern = corners ? deform_fluxes_kernel<real, MX, true> : deform_fluxes_kernel<real, MX, false>;
+  kern<<<grid, MX == 32 ? 512 : 128, 0, s>>>(p0, p1, coef, umetric, kc, T, rot, t_half, t0_dev,
+                                             t_off);
 }
 
 }  // namespace
 
 template <typename real>
-cudaError_t launch_deform_fluxes(int p0, int p1, int mx, const double* coef, real* umetric,
-                                 double kc, double T, double rot, double t_half,
+cudaError_t launch_deform_fluxes(int p0, int p1, int mx, const double* coef, bool corners,
+                                 real* umetric, double kc, double T, double rot, double t_half,
                                  const double* t0_dev, double t_off, cudaStream_t s) {
   if (p1 <= p0) return cudaSuccess;
-  switch (mx) {
-    case 8: deform_launch<real, 8>(p0, p1, coef, umetric, kc, T, rot, t_half, t0_dev, t_off, s); break;
-    case 16: deform_launch<real, 16>(p0, p1, coef, umetric, kc, T, rot, t_half, t0_dev, t_off, s); break;
-    case 32: deform_launch<real, 32>(p0, p1, coef, umetric, kc, T, rot, t_half, t0_dev, t_off, s); break;
-    default: return cudaErrorInvalidValue;
-  }
+  auto launch = mx == 8    ? deform_launch<real, 8>
+                : mx == 16 ? deform_launch<real, 16>
+                : mx == 32 ? deform_launch<real, 32>
+                           : nullptr;
+  if (!launch) return cudaErrorInvalidValue;
+  launch(p0, p1, coef, corners, umetric, kc, T, rot, t_half, t0_dev, t_off, s);
   ++launch_counter();
   return cudaGetLastError();
 }
@@ -214,7 +256,7 @@ template <typename real>
 cudaError_t launch_sphere_metrics(const PatchMeta* meta, int npatch, int mx, const double* omega,
                                   double* metric, real* umetric, const RemapEntry* rm,
                                   const double* old_metric, const real* old_umetric, double* coef,
-                                  cudaStream_t s) {
+                                  bool corners, cudaStream_t s) {
   if (npatch <= 0) return cudaSuccess;
   const int SN = mx + 2 * kMbc + 1;
   const size_t smem = sizeof(double) * 3 * (size_t)SN * SN;
@@ -229,18 +271,19 @@ cudaError_t launch_sphere_metrics(const PatchMeta* meta, int npatch, int mx, con
   if (smem > 64 * 1024) return cudaErrorInvalidValue;
   const int grid = npatch < 65535 * 8 ? npatch : 65535 * 8;
   metrics_kernel<real><<<grid, 256, smem, s>>>(meta, npatch, mx, omega[0], omega[1], omega[2],
-                                               metric, umetric, rm, old_metric, old_umetric, coef);
+                                               metric, umetric, rm, old_metric, old_umetric, coef,
+                                               corners);
   ++launch_counter();
   return cudaGetLastError();
 }
 
 #define FC_INSTANTIATE(real)                                                                     \
-  template cudaError_t launch_deform_fluxes<real>(int, int, int, const double*, real*, double,   \
-                                                  double, double, double, const double*, double, \
-                                                  cudaStream_t);                                 \
+  template cudaError_t launch_deform_fluxes<real>(int, int, int, const double*, bool, real*,     \
+                                                  double, double, double, double, const double*, \
+                                                  double, cudaStream_t);                         \
   template cudaError_t launch_sphere_metrics<real>(const PatchMeta*, int, int, const double*,    \
                                                    double*, real*, const RemapEntry*,            \
-                                                   const double*, const real*, double*,          \
+                                                   const double*, const real*, double*, bool,    \
                                                    cudaStream_t);
 
 FC_INSTANTIATE(float)

@@ -206,6 +206,11 @@ class Forest:
         wait (polls; negative: default) -- see fc_set_limits."""
         check(load().fc_set_limits(self._h, int(walk_ctas), int(wait_polls)))
 
+    def set_coef_budget(self, nbytes: int = -1):
+        """Device memory the deformational flow's edge coefficients may take
+        (negative: the default); see fc_set_coef_budget."""
+        check(load().fc_set_coef_budget(self._h, int(nbytes)))
+
     def set_velocity_scale(self, scale: float):
         check(load().fc_set_velocity_scale(self._h, float(scale)))
 
