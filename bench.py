@@ -43,6 +43,7 @@ import synth  # noqa: E402
 
 METRIC = "cell-updates/s"
 L2_FLUSH_BYTES = 512 << 20
+VARIANTS = ["staged", "walk", "walk1", "band"]  # update kernels by number (walk1: walk again)
 WORKLOAD = ("adaptive swirl forest, levels 2-6, 32x32 patches, mbc 2, walls, MC + transverse, "
             "CFL 0.9, multirate, regrid every 4 coarse steps")
 SPHERE_WORKLOAD = ("cubed sphere (6 trees), levels 1-7, 32x32 patches, mbc 2, solid-body rotation "
@@ -65,8 +66,8 @@ def parse():
     ap.add_argument("--ensemble", type=int, default=256, help="forests in the batched variant")
     ap.add_argument("--variant", default="auto",
                     help="update kernel of the headline (and --mode batched) forest: auto "
-                         "(autotuned per launch size), or NAME[:WARPS] with NAME staged, walk, "
-                         "walk1 or band -- e.g. to profile the kernels a default run's tuning "
+                         "(autotuned per launch size), or NAME[:WARPS] with NAME staged, walk "
+                         "or band -- e.g. to profile the kernels a default run's tuning "
                          "chose (a profiler distorts the tuner's timings)")
     ap.add_argument("--mode", choices=["full", "batched", "sphere", "sphere_deform", "adjoint",
                                        "sweep"],
@@ -201,15 +202,14 @@ class Runner:
                             smooth=int(w.smooth))
         self.F = fc.initial_forest(desc, q0_fn(workloads), lmax_f=self.lmax_f,
                                    tau_r=w.tau_refine, tau_c=w.tau_coarsen)
-        names = ["staged", "walk", "walk1", "band"]
         if variant != "auto":  # one kernel for every launch
             name, _, warps = variant.partition(":")
             warps = int(warps or 4)
-            self.F.set_advance_variant(names.index(name), warps)
+            self.F.set_advance_variant(VARIANTS.index(name), warps)
             self.tuning = {"all": {"variant": name, "warps": warps, "fill": "fused"}}
         else:
             # pick the patch-update kernel per launch size on this layout (untimed setup)
-            self.tuning = {int(b): {"variant": names[v], "warps": k,
+            self.tuning = {int(b): {"variant": VARIANTS[v], "warps": k,
                                     "fill": "fused" if fu else "separate", "ns": ns}
                            for b, (v, k, fu, ns) in self.F.autotune().items()}
         self.n = 0
@@ -358,7 +358,7 @@ def adjoint_cost(fc, torch, flush_buf, ncoarse: int = 25, variant: str = "auto")
         F.autotune()
     else:  # one update kernel for every launch (see --variant)
         name, _, warps = variant.partition(":")
-        F.set_advance_variant(["staged", "walk", "walk1", "band"].index(name), int(warps or 4))
+        F.set_advance_variant(VARIANTS.index(name), int(warps or 4))
     leaves = F.leaves()
     dev = flush_buf.device
     q0 = torch.tensor(q0_fn([w])(leaves), dtype=torch.float32, device=dev)
@@ -440,7 +440,7 @@ def granularity_sweep(fc, torch, hbm):
             v, warps, fused, ns = rep[b]
             cells = n * mx * mx
             nbytes = n * ((mx + 4) ** 2 + mx * mx) * 4
-            rows.append({"mx": mx, "patches": n, "variant": ["staged", "walk", "walk1", "band"][v],
+            rows.append({"mx": mx, "patches": n, "variant": VARIANTS[v],
                          "warps": warps, "us_per_substep": ns * 1e-3,
                          "cell_updates_per_s": cells / (ns * 1e-9),
                          "hbm_frac": nbytes / (ns * 1e-9) / 1e9 / hbm})

@@ -491,26 +491,27 @@ fc_status fc_set_graphs(fc_forest* forest, int enable);
 /* Patch-update kernel variants: 0 "staged" (one CTA per patch, the whole
  * tile in shared memory, every thread on every phase -- low latency for
  * launches of few patches), 1 "walk" (lanes own patch columns and walk
- * the rows with warp shuffles, tiles double-buffered per warp by TMA, a
- * persistent grid of `warps`-warp CTAs -- fewest instructions per cell),
- * 2 (walk1: the walk with one tile buffer per warp, twice the warps per SM)
- * and 3 "band" (one CTA of `warps` warps per patch, each warp walking a band
- * of rows as the walk does: mx^2 / (32 warps) rows a band, at least one;
- * with refluxing and the cubed sphere's capacity form).  Where the walk
- * lacks what the forest needs (refluxing, the capacity form) the launch
- * runs staged.
+ * the rows with warp shuffles, tiles by TMA, a persistent grid of
+ * `warps`-warp CTAs -- fewest instructions per cell), 2 (another name of 1,
+ * kept for callers of a form of the walk that is gone) and 3 "band" (one CTA
+ * per patch whose warps each walk a band of rows as the walk does: at mx = 32
+ * 8, 4 or 2 rows a band with up to 4, 8 or 16 `warps`, at mx = 16 4, 2 or 1
+ * with 2, 4 or more, at mx = 8 one row; with refluxing and the cubed sphere's
+ * capacity form).  Where the walk is forced and lacks what the forest needs
+ * (refluxing, the capacity form) the launch runs staged.
  *
- * Untuned launch sizes run walk from 1024 patches up on planar grids, band
- * with 8 warps otherwise.
+ * Untuned launches run walk from a number of patches up that depends on the
+ * precision and mx (384 to 4096) on planar grids without refluxing, band
+ * otherwise.
  *
- * fc_autotune times every candidate (staged; band with 4 or 8 warps;
- * walk with 2, 4, 8 warps per
- * CTA; walk1 with 4 or 8; each with the level's ghosts filled inside the update kernel or by
- * separate fill kernels) as a whole level substep of the current layout,
+ * fc_autotune times every candidate (staged; band in each of its forms but
+ * those of one row at mx = 16 and of two at mx = 32; walk with 2, 4 and 8
+ * warps per CTA; each with the level's ghosts filled inside the update kernel
+ * or by separate fill kernels) as a whole level substep of the current layout,
  * eight substeps replayed from one CUDA graph as in a captured step (walk
- * only for launches of at least two patches per SM: below that staged has
- * measured about twice as fast), and keeps the fastest per launch size (sizes bucketed by powers of two; a
- * bucket is tuned once per forest).  It overwrites the previous-state
+ * only for launches of at least two patches per SM: below that its warps
+ * mostly idle), and keeps the fastest per launch size (sizes bucketed by
+ * powers of two; a bucket is tuned once per forest).  It overwrites the previous-state
  * buffers, so call it when all levels hold the same time (after set_q or a
  * regrid).  report: host, nullable, 32 x 4 ints per bucket b (patches in
  * [2^b, 2^(b+1))): (variant or -1 if untuned, warps, fused, ns per substep).
@@ -521,19 +522,19 @@ fc_status fc_set_graphs(fc_forest* forest, int enable);
  * (FC_ERR_INVALID_ARG otherwise). */
 fc_status fc_autotune(fc_forest* forest, int* report, void* stream);
 
-/* Fused ghost fill in multirate substeps (on by default): the patch-update
- * kernel applies Alg. 1 to the ghost ring of the tile it holds in shared
- * memory, so a level substep is one fill launch (the coarse neighbours'
- * time-interpolated data) plus the update, and the level's ghost cells are
- * never written to HBM.  enable = 0: separate fill kernels write every ghost
- * ring first (same results, bit for bit). */
+/* Fused ghost fill (on by default): in multirate substeps and global steps the
+ * patch-update kernel applies Alg. 1 to the ghost ring of the tile it holds in
+ * shared memory, computing what it reads of a coarser neighbour's fill itself,
+ * so a level's update is one launch and its ghost cells are never written to
+ * HBM; a whole forest's fill and its tag are one launch.  enable = 0: separate
+ * fill kernels write every ghost ring first (same results, bit for bit). */
 fc_status fc_set_fused_fill(fc_forest* forest, int enable);
 fc_status fc_set_advance_variant(fc_forest* forest, int variant, int warps);
 
 /* Launch limits (tests and tuning).
  *   walk_ctas   cap on the persistent walk grid (0: as many CTAs as the SMs
  *               hold at once); a small cap makes every warp loop over many
- *               groups of patches through both of its tile buffers.
+ *               groups of patches.
  *   wait_polls  polls of the patch-update and ghost-fill kernels' bounded wait
  *               for their tile copies before they give up (negative: the default,
  *               2^22); 0 makes every such wait give up at once.  A kernel

@@ -918,7 +918,7 @@ fc_status advance_level_t(fc_forest* F, int L, double t, double dt, cudaStream_t
       // tiles, all the reverse reads of them.  The walk computes each coarse
       // cell beside a face once for its four ghosts; in the adjoint's replay
       // it keeps the fill, which leaves the tiles the reverse reads
-      const bool walk = a.variant == ADV_WALK || a.variant == ADV_WALK1;
+      const bool walk = a.variant == ADV_WALK;
       const bool direct = tlevel >= 0 && !(walk && F->keep_qT);
       if (direct) A.ntargets = 0;
       a.direct = direct ? 1 : 0;
@@ -1292,7 +1292,7 @@ fc_status fc_set_advance_variant(fc_forest* F, int variant, int warps) {
   if (!F || variant < -1 || variant > ADV_BAND || !warps_ok)
     return fail(FC_ERR_INVALID_ARG,
                 "variant must be -1, 0, 1, 2 or 3 and warps 2, 4 or 8 (16 with variant 3)");
-  F->forced_variant = variant;
+  F->forced_variant = variant == 2 ? ADV_WALK : variant;  // (2: walk under its other name)
   F->forced_warps = warps;
   destroy_graphs(F);
   return FC_OK;
@@ -1342,7 +1342,7 @@ fc_status fc_autotune(fc_forest* F, int* report, void* stream) {
       const auto& c = cand[c2 % ncand];
       const int fused = c2 / ncand;
       if (fused && !F->fuse) continue;
-      const bool walk = c.variant == ADV_WALK || c.variant == ADV_WALK1;
+      const bool walk = c.variant == ADV_WALK;
       // no capacity form in walk
       if (walk && (F->d_metric || H.desc.domain == FC_DOMAIN_SPHERE)) continue;
       if (walk && F->bflux) continue;  // (it would run staged)
