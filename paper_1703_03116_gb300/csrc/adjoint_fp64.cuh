@@ -12,9 +12,11 @@
 // negations on the bits too (magnitude_bits()), 3.1 ms with a column's factors
 // kept over its rows and one addition less an edge.
 //
-// FP32 keeps that form (adjoint.cu): its instructions are not what bounds it
-// (2% of the adjoint of a global step), and its velocity-scale derivative is
-// an FP64 sum of FP32 terms, which other roundings of the terms move by 1e-7.
+// FP32 keeps that form (adjoint.cu): in the adjoint of a global step its
+// instructions are 2% (in the multirate reverse, which this does not say
+// anything of, its transposes are what the time goes to).  Its velocity-scale
+// derivative is summed in FP32 by a thread and a warp and in FP64 from there
+// on; other roundings of the terms move it by 1e-7.
 #pragma once
 
 #include "walk_edge.cuh"

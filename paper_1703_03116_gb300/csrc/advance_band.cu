@@ -40,8 +40,9 @@ constexpr int band_threads() {
   return MX * MX / R > most ? MX * MX / R : most;
 }
 
-// resident CTAs the register budget is sized for: 1024 FP32 / 512 FP64
-// threads per SM at most 64 / 128 registers a thread
+// resident CTAs the register budget is sized for: as many whole CTAs as 1024
+// FP32 / 512 FP64 threads hold (FP32 mx = 32: 4 of 256 threads, at most 64
+// registers a thread; FP64 in bands of 8 rows: 2 of 192, at most 168, 141 used)
 template <typename real, int MX, int R>
 constexpr int band_min_blocks() {
   return (sizeof(real) == 4 ? 1024 : 512) / band_threads<real, MX, R>() > 0

@@ -528,10 +528,12 @@ fc_status deform_fluxes(fc_forest* F, int p0, int p1, const AdvArgs& a, cudaStre
   const double kc = d.vel[0] * F->vel_scale, rot = 2.0 * M_PI / d.vel[2] * F->vel_scale;
   if (F->esize == 4)
     FC_CUDA(launch_deform_fluxes(p0, p1, d.mx, F->d_coef, F->coef_corners,
-                                 static_cast<float*>(F->d_umetric), kc, d.vel[1], rot, a.t_half, a.t0_dev, a.t_off, s));
+                                 static_cast<float*>(F->d_umetric), kc, d.vel[1], rot,
+                                 a.t_half, a.t0_dev, a.t_off, s));
   else
     FC_CUDA(launch_deform_fluxes(p0, p1, d.mx, F->d_coef, F->coef_corners,
-                                 static_cast<double*>(F->d_umetric), kc, d.vel[1], rot, a.t_half, a.t0_dev, a.t_off, s));
+                                 static_cast<double*>(F->d_umetric), kc, d.vel[1], rot,
+                                 a.t_half, a.t0_dev, a.t_off, s));
   return FC_OK;
 }
 
@@ -719,16 +721,20 @@ int size_bucket(int n) {
   return b;
 }
 
-// From how many patches a launch of a planar level is the walk's: where its
-// one-level step (uniform forests, one GB300) passes the band's.
-//   us, band / walk   n = 640        1280         2560         6400
-//   FP32 mx = 32   15.3 / 16.6  20.8 / 18.7  31.2 / 22.9  66.0 / 39.3
-//        mx = 16   12.2 / 18.7  14.7 / 18.7  18.8 / 20.8  35.1 / 23.0
-//        mx = 8    10.6 / 16.7  10.6 / 16.8  14.5 / 16.8  23.0 / 18.7
-//   FP64 mx = 32   90.5 / 74.3   156 / 115    289 / 217    721 / 496
-//        mx = 16   35.2 / 39.2  49.4 / 45.9  88.6 / 69.9   203 / 148
-//        mx = 8    18.7 / 27.1  29.1 / 28.9  49.8 / 33.1   103 / 53.5
-// (FP64 mx = 32 at 320: 57.7 / 61.8)
+// From how many patches a launch of a planar level is the walk's.  One level's
+// step alone (uniform forests, one GB300), us, band / walk:
+//        n =       384          768          1280         3072         4096         6400
+//   FP32 mx = 32    6.2 / 10.3  10.3 / 10.3  14.4 / 14.4  24.7 / 18.5  32.7 / 22.6  47.2 / 32.8
+//        mx = 16    6.2 / 12.6   6.2 / 13.8   8.3 / 14.2  12.4 / 14.4  15.7 / 14.4  21.4 / 18.5
+//        mx = 8     6.2 / 12.3   6.2 / 12.3   6.2 / 12.3   8.3 / 12.4  10.3 / 12.4  14.4 / 12.4
+//   FP64 mx = 32   46.1 / 46.7  67.7 / 55.4   111 / 86.1   238 / 184    303 / 229    467 / 374
+//        mx = 16   14.4 / 28.1  30.7 / 28.7  43.2 / 33.4  85.3 / 59.4   100 / 69.7   156 / 111
+//        mx = 8    10.3 / 20.5  18.3 / 20.5  21.0 / 20.5  47.1 / 22.6  57.4 / 28.7  84.1 / 38.9
+// The lines were drawn where these times crossed for an earlier band; for this
+// one they cross near 1000, 3700 and 5000 (FP32), 450, 700 and 1100 (FP64).
+// They stay: an FP64 launch beside the other levels' counts by its FP64 work,
+// of which the walk has less (lines at 512 / 768 took 13 forests of 32^2 to 0.84
+// of the speed), and in FP32 the two differ by 2 us where the lines are off.
 int walk_from(int mx, size_t esize) {
   if (esize == 4) return mx == 32 ? 768 : mx == 16 ? 3072 : 4096;
   return mx == 32 ? 384 : mx == 16 ? 1024 : 1280;
@@ -755,11 +761,16 @@ void choose_variant(const fc_forest* F, int n, AdvArgs* a) {
     a->warps = F->esize == 4 ? 8 : 2;
   } else {
     // rows a band, by warps: at mx = 16 one row of a patch a warp segment (8
-    // warps) computes every x-edge three times; FP64, 320 patches: 31.0 us,
-    // two rows 23.0, four 20.9 (64 patches: 16.7, 16.6, 18.7); FP32, 1280
-    // patches: 16.7, 14.7, 14.7 (64: the same).  At mx = 32 FP64 takes 8 rows a
-    // band (4 warps) and two CTAs an SM: a step of the swirl forest's levels
-    // of 35 to 248 patches 718 us, 740 with 4 rows; FP32 473 and 416
+    // warps) computes every x-edge three times; FP64, 256 patches: 14.4 us, two
+    // and four rows 12.4; 512 patches (recording fluxes) 20.5 by two, 18.5 by
+    // four; 64 patches 10.3, 10.3, 12.4; FP32 the same but for 4096 patches, 16.4
+    // by two and 18.5 by four.  At mx = 32 FP64 takes 8 rows a band (4 warps) and
+    // two CTAs an SM: a step of the swirl forest's levels of 35 to 248 patches
+    // 718 us, 740 with 4 rows; 4096 patches (recording) 320 and 349; below 128
+    // patches 4 rows are 2 us faster alone.  On the sphere 288, 576, 864 and 1824
+    // patches 30.8, 57.5, 84.6, 169 us by 8 rows, 32.9, 63.5, 92.2, 183 by 4.
+    // FP32 takes 4 rows: the swirl forest 416 us, 473 by 8; the sphere's launches
+    // 8.2, 8.3, 12.3, 18.5 us by 4, 8.2, 10.2, 12.5, 20.1 by 8
     a->variant = ADV_BAND;
     a->warps = mx == 16 ? (F->esize == 8 && n >= 128 ? 2 : 4) : F->esize == 8 ? 4 : 8;
   }
