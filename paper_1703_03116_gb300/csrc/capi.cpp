@@ -833,12 +833,12 @@ fc_status fill_all_t(fc_forest* F, cudaStream_t s, double* delta, bool* tagged) 
     return FC_OK;
   }
   FillArgs A{F->d_lists + F->off_all, (int)H.list_all.size(), -1, 0.0};
-  {
+  if (A.ntargets > 0) {
     Timed tm(F, 1, s, gb * A.ntargets);
     FC_CUDA(launch_fill_coarse(D, A, s));
   }
   FillArgs B{F->d_lists + F->off_coarse_all, (int)H.list_coarse_all.size(), -1, 0.0};
-  {
+  if (B.ntargets > 0) {
     Timed tm(F, 1, s, gb * B.ntargets);
     FC_CUDA(launch_fill_fine(D, B, s));
   }
@@ -939,7 +939,7 @@ fc_status advance_level_t(fc_forest* F, int L, double t, double dt, cudaStream_t
       }
       // (inside a captured step this runs on the level's own stream, after
       // the waits above: see fc_forest::dag_levels)
-      {
+      if (A.ntargets > 0) {
         Timed tm(F, 1, s, gb * A.ntargets);
         FC_CUDA(launch_fill_coarse(D, A, s));
       }
@@ -949,12 +949,12 @@ fc_status advance_level_t(fc_forest* F, int L, double t, double dt, cudaStream_t
       a.alpha = alpha;
     } else {
       FillArgs A{F->d_lists + F->off_a[L], (int)H.list_a[L].size(), tlevel, alpha};
-      {
+      if (A.ntargets > 0) {
         Timed tm(F, 1, s, gb * A.ntargets);
         FC_CUDA(launch_fill_coarse(D, A, s));
       }
       FillArgs B{F->d_lists + F->off_b[L], (int)H.list_b[L].size(), tlevel, alpha};
-      {
+      if (B.ntargets > 0) {
         Timed tm(F, 1, s, gb * B.ntargets);
         FC_CUDA(launch_fill_fine(D, B, s));
       }
