@@ -92,9 +92,10 @@ typedef enum { FC_VEL_CONST = 0, FC_VEL_SWIRL = 1, FC_VEL_ROTATION = 2, FC_VEL_D
  *               times the velocity scale.
  *               FC_VEL_ROTATION (sphere only): solid-body rotation
  *               u = omega x X, omega = (vel[0], vel[1], vel[2]).  The sphere
- *               runs the capacity form: FP64 metrics per patch (cell
- *               areas kappa, edge volume fluxes omega . (X_b - X_a) between
- *               the edge's end points), ghost-cell metrics from the patch's
+ *               runs the capacity form: metrics per patch computed in FP64
+ *               (cell areas kappa, edge volume fluxes omega . (X_b - X_a)
+ *               between the edge's end points) and read by the update in the
+ *               field's precision, ghost-cell metrics from the patch's
  *               own mapping, area-weighted fine-to-coarse averages, and
  *               corner ghosts beyond a cube vertex set to the mean of the
  *               two edge ghosts next to them.

@@ -28,7 +28,7 @@
 // its field moves: 256 forests (67168 patches of 32^2, FP32) 6.0 -> 2.6 ms,
 // 64 forests (13852 patches of 16^2, FP64) 3.7 -> 2.0 ms; 16384 patches of
 // 32^2 at one level 94 -> 67 us.  About 3500 warp instructions a 32^2 patch
-// (of 6200), at 55% of the issue slots with 24 warps an SM; its sides are one
+// (of 6200), at 58% of the issue slots with 24 warps an SM; its sides are one
 // loop over strides because as four copies of the code they overflowed the
 // instruction cache (4.1 against 2.7 ms).
 //
